@@ -85,7 +85,7 @@ ipt::SceneBuffers buffers(const ipt_ctx* ctx, const DeviceScene* s) {
   b.vnrm = s->vnrm;
   b.seg_tris = s->seg_tris;
   b.seg_begin = s->seg_begin;
-  b.tri_cdf = s->tri_cdf;
+  b.tri_sel = s->tri_sel;
   b.seg_area = s->seg_area;
   b.orig_to_internal = s->orig_to_internal;
   b.n_seg = s->n_seg;
@@ -651,14 +651,14 @@ ipt_status ipt_scene_upload(ipt_ctx* ctx, const float* pos, uint32_t n_vert, con
   if (!hs.vnrm.empty()) A(&s->vnrm, 3 * (size_t)n_tri);
   A(&s->seg_tris, n_tri);
   A(&s->seg_begin, S + 1);
-  A(&s->tri_cdf, n_tri);
+  A(&s->tri_sel, n_tri);
   A(&s->seg_area, S);
   A(&s->orig_to_internal, n_tri);
   A(&s->tab.mat_a, S);
   A(&s->tab.mat_b, S);
   A(&s->tab.emis, S);
   A(&s->tab.samp, S);
-  A(&s->tab.pspec, S);
+  A(&s->tab.sel, S + 1);
   A(&s->tab.cdf, S);
   A(&s->tab.lum, S);
   A(&s->tab.W, 1);
@@ -682,7 +682,7 @@ ipt_status ipt_scene_upload(ipt_ctx* ctx, const float* pos, uint32_t n_vert, con
   if (s->vnrm) H(s->vnrm, hs.vnrm.data(), hs.vnrm.size() * sizeof(float));
   H(s->seg_tris, hs.seg_tris.data(), hs.seg_tris.size() * sizeof(uint32_t));
   H(s->seg_begin, hs.seg_begin.data(), hs.seg_begin.size() * sizeof(uint32_t));
-  H(s->tri_cdf, hs.tri_cdf.data(), hs.tri_cdf.size() * sizeof(double));
+  H(s->tri_sel, hs.tri_sel.data(), hs.tri_sel.size() * sizeof(float));
   H(s->seg_area, hs.seg_area.data(), hs.seg_area.size() * sizeof(double));
   H(s->orig_to_internal, hs.orig_to_internal.data(), hs.orig_to_internal.size() * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(s->params, 0, 10 * sizeof(float) * S);

@@ -40,11 +40,11 @@ ipt_status ipt_capi::disney_state(ipt_ctx* ctx, DeviceScene* s, DisneyState** ou
   if (S > ipt::disney_max_shared_segments()) A(&d->gacc, np);
   A(&d->tab.emis, S);
   A(&d->tab.samp, S);
+  A(&d->tab.sel, S + 1);
   A(&d->tab.cdf, S);
   A(&d->tab.lum, S);
   A(&d->tab.W, 1);
   A(&d->dt.mat, 4 * S);
-  A(&d->dt.lobe, S);
   A(&d->dt.samp, 2 * S);
   if (e != cudaSuccess) {
     free_disney(d);
@@ -70,7 +70,7 @@ ipt::WfScene disney_entry(const ipt_ctx* ctx, int32_t scene, const DeviceScene* 
                           uint32_t begin, uint32_t n) {
   ipt::WfScene e = wf_entry(ctx, scene, s, begin, n);
   e.t = ipt::seg_dev(d->tab);
-  e.dis = ipt::DisneyDev{d->dt.mat, d->dt.lobe, d->dt.samp};
+  e.dis = ipt::DisneyDev{d->dt.mat, d->dt.samp};
   e.n_all = (uint32_t)s->n_pix;
   return e;
 }

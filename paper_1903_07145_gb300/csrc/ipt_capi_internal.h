@@ -81,7 +81,7 @@ struct DisneyState {
   int* step_dev = nullptr;
   double* grad_acc = nullptr;
   float* gacc = nullptr;     // global accumulators when shared memory is too small
-  ipt::SegBuffers tab{};     // emission, light selection (mat_a, mat_b, pspec unused)
+  ipt::SegBuffers tab{};     // emission, light selection (mat_a, mat_b unused)
   ipt::DisneyBuffers dt{};
   bool tab_is_ctx = false;
   uint64_t iteration = 0;
@@ -109,7 +109,7 @@ struct DeviceScene {
   float4* vnrm = nullptr;
   uint32_t* seg_tris = nullptr;
   uint32_t* seg_begin = nullptr;
-  double* tri_cdf = nullptr;
+  float* tri_sel = nullptr;
   double* seg_area = nullptr;
   uint32_t* orig_to_internal = nullptr;
   // parameter tables

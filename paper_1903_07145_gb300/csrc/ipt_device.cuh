@@ -74,7 +74,8 @@ struct PathRng {
 //   vnrm: 3 float4 per triangle (vertex normals) or nullptr.
 //   Light selection (static): seg_tris lists the triangles of each segment
 //     (internal ids, by increasing original id), seg_begin[s]..seg_begin[s+1];
-//     tri_cdf is the inclusive FP64 area prefix inside each segment.
+//     tri_sel holds, per entry, the inclusive FP64 area prefix inside the
+//     segment as a threshold on the uniform (see SegDev).
 // ---------------------------------------------------------------------------
 struct SceneDev {
   const float4* nodes;
@@ -84,8 +85,7 @@ struct SceneDev {
   const float4* vnrm;
   const uint32_t* seg_tris;
   const uint32_t* seg_begin;
-  const double* tri_cdf;
-  const double* seg_area;
+  const float* tri_sel;
   uint32_t n_seg;
   uint32_t n_tri;
   float eps;  // spawn offset along the oriented geometric normal
@@ -104,22 +104,32 @@ __device__ __forceinline__ void count_ray(const SceneDev& s, int kind, uint32_t 
 
 // Per-segment tables derived from the parameters (rebuilt whenever the
 // parameters change).  Evaluation uses params; sampling uses sampling params.
+//
+// Integer decisions (which segment, which triangle, which lobe) compare a
+// 24-bit uniform u with an FP64 value: u * W < cdf[i], u < P.  The paths do
+// not evaluate them in FP64: sm_103a issues one FP64 warp instruction per 16
+// cycles and SM, and the ~14 of a vertex kept that pipe 41% busy in the
+// shading stage and held its warps on it.  Every left side is monotonic in
+// u, so the decision equals u < T, T the smallest multiple of 2^-24 for
+// which the FP64 comparison fails; T is exact in FP32 and is tabulated with
+// the parameters (unit_threshold), and the paths compare FP32 values.
+// Measured: one loss-and-gradient evaluation of the 61k room 110.0 -> 108.1
+// ms, eight steps of the 64-scene Cornell batch 7.76 -> 7.59 ms.
 struct SegDev {
   const float4* mat_a;   // kd.rgb, roughness            (params)
   const float4* mat_b;   // ks.rgb, alpha = max(r^2,1e-4) (params)
   const float4* emis;    // emission_scale * e.rgb, -    (params)
-  const float4* samp;    // alpha_s, P_spec (float), p_A = lum_s / W (float), -   (sampling)
-  const double* pspec;   // P_spec in FP64 (lobe decision)
-  const double* cdf;     // inclusive FP64 prefix of lum(e_s) A_s
-  const double* W;       // total; 0 disables light sampling
+  const float4* samp;    // alpha_s, P_spec, p_A = lum_s / W, threshold of the FP64 P_spec   (sampling)
+  const float* sel;      // thresholds of the inclusive FP64 prefix of lum(e_s) A_s; entry
+                         // n_seg: 1 when the total W is positive, 0 disables light sampling
 };
 
 // Disney material model tables (see ipt_disney.cuh); null pointers when a
 // scene traces with Lambert + GGX.
 struct DisneyDev {
   const float4* mat;    // 4 per segment: the 13 material values, then zeros
-  const double2* lobe;  // cumulative lobe probabilities (P_d, P_d + P_s), FP64
-  const float4* samp;   // 2 per segment: (a_x, a_y, a_c, 0), (P_d, P_s, P_c, 0)
+  const float4* samp;   // 2 per segment: (a_x, a_y, a_c, T_d), (P_d, P_s, P_c, T_ds); T_d, T_ds the
+                        // thresholds of the FP64 cumulative lobe probabilities P_d, P_d + P_s
 };
 
 struct ViewDev {
@@ -824,17 +834,17 @@ __device__ __forceinline__ float bsdf_pdf(float P, float a_s, float3 n, float3 w
   return (1.0f - P) * (co * (1.0f / kPi)) + P * ps;
 }
 
-// Lobe by u_lobe < P_spec (FP64 decision); diffuse: cosine-weighted
+// Lobe by u_lobe < T (threshold of the FP64 P_spec); diffuse: cosine-weighted
 // (r = sqrt(u1), phi = 2 pi u2); specular: GGX visible normals (Heitz, JCGT
 // 7(4), 2018) and a mirror reflection of wi.
-__device__ __forceinline__ float3 bsdf_sample(double P, float a_s, float3 n, float3 wi, float u_lobe,
+__device__ __forceinline__ float3 bsdf_sample(float T, float a_s, float3 n, float3 wi, float u_lobe,
                                               float u1, float u2) {
   float3 b1, b2;
   onb(n, b1, b2);
   float sphi, cphi;
   sincospif(2.0f * u2, &sphi, &cphi);
   const float rr = sqrtf(u1);
-  if ((double)u_lobe < P) {
+  if (u_lobe < T) {
     const float3 vl = f3(dot(wi, b1), dot(wi, b2), dot(wi, n));
     const float3 vh = normalize(f3(a_s * vl.x, a_s * vl.y, vl.z));
     const float lensq = vh.x * vh.x + vh.y * vh.y;
@@ -853,12 +863,12 @@ __device__ __forceinline__ float3 bsdf_sample(double P, float a_s, float3 n, flo
   return b1 * (rr * cphi) + b2 * (rr * sphi) + n * z;
 }
 
-// First index i in [b, e) with x < a[i] (e - 1 if none); a non-decreasing.
-__device__ __forceinline__ int upper_bound_d(const double* a, int b, int e, double x) {
+// First index i in [b, e) with u < a[i] (e - 1 if none); a non-decreasing.
+__device__ __forceinline__ int upper_bound_f(const float* a, int b, int e, float u) {
   int lo = b, hi = e - 1;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (x < __ldg(&a[mid]))
+    if (u < __ldg(&a[mid]))
       hi = mid;
     else
       lo = mid + 1;

@@ -15,7 +15,7 @@ namespace {
 constexpr int kDisneyThreads = 128;
 
 // Per-segment tables of one scene (one block): material values, emission,
-// the FP64 lobe probabilities and sampling widths from the sampling
+// the lobe probabilities, their FP64 decisions as thresholds, sampling widths from the sampling
 // parameters, and the emission-proportional light-selection CDF.
 __device__ void disney_tables_body(const float* params, const float* sparams, uint32_t S, float es,
                                    const double* seg_area, const SegBuffers& t, const DisneyBuffers& d) {
@@ -41,11 +41,11 @@ __device__ void disney_tables_body(const float* params, const float* sparams, ui
       p1 = __ddiv_rn(ws, sum);
       p2 = __ddiv_rn(wc, sum);
     }
-    d.lobe[s] = make_double2(p0, __dadd_rn(p0, p1));
     const float k = sqrtf(1.0f - 0.9f * q[8]);
     const float r2 = q[7] * q[7];
-    d.samp[2 * s] = make_float4(fmaxf(r2 / k, 1e-3f), fmaxf(r2 * k, 1e-3f), 0.1f - 0.099f * q[12], 0.0f);
-    d.samp[2 * s + 1] = make_float4((float)p0, (float)p1, (float)p2, 0.0f);
+    d.samp[2 * s] = make_float4(fmaxf(r2 / k, 1e-3f), fmaxf(r2 * k, 1e-3f), 0.1f - 0.099f * q[12],
+                                  unit_threshold(p0, 1.0));
+    d.samp[2 * s + 1] = make_float4((float)p0, (float)p1, (float)p2, unit_threshold(__dadd_rn(p0, p1), 1.0));
     double le = lum_d(q[13], q[14], q[15]);
     if (!(le > 0.0)) le = 0.0;
     t.lum[s] = le;
@@ -64,7 +64,9 @@ __device__ void disney_tables_body(const float* params, const float* sparams, ui
   for (uint32_t s = threadIdx.x; s < S; s += blockDim.x) {
     const double le = t.lum[s];
     t.samp[s] = make_float4(0.0f, 0.0f, (W > 0.0 && le > 0.0) ? (float)(le / W) : 0.0f, 0.0f);
+    t.sel[s] = unit_threshold(t.cdf[s], W);
   }
+  if (threadIdx.x == 0) t.sel[S] = W > 0.0 ? 1.0f : 0.0f;
 }
 
 __global__ void k_disney_tables(const float* params, const float* sparams, uint32_t S, float es,
@@ -133,14 +135,14 @@ __device__ __forceinline__ void add3d(float* acc, int i, float3 v) {
 // the Disney material and sampler).
 __device__ float3 disney_forward_path(const SceneDev& s, const SegDev& t, const DisneyDev& D, const ViewDev& vw,
                                       uint32_t px, uint32_t py, uint32_t pid, uint32_t sample, const PathParams& pp,
-                                      double W, uint32_t* err) {
+                                      bool light, uint32_t* err) {
   PathRng rng;
   rng.base = make_uint4(pid, sample, pp.set_iter, 0);
   rng.key = pp.key;
   float3 o;
   float3 d = camera_ray(vw, px, py, rng, o);
   float3 beta = f3(1.0f, 1.0f, 1.0f), L = f3(0.0f, 0.0f, 0.0f);
-  const bool light_on = pp.nee && W > 0.0;
+  const bool light_on = pp.nee && light;
   int skip = -1;
   float prev_pdf = 0.0f;
   for (uint32_t k = 0;; ++k) {
@@ -158,7 +160,7 @@ __device__ float3 disney_forward_path(const SceneDev& s, const SegDev& t, const 
     float m[kDisneyMat];
     load_disney(D, v.seg, m);
     if (light_on) {
-      NeeResult ne = nee_prepare_with(s, t, v, ua, ub, W, pp.profile, pp.mis,
+      NeeResult ne = nee_prepare_with(s, t, v, ua, ub, pp.profile, pp.mis,
                                       [&](float3 wl) { return disney_pdf(D, v.seg, v.ns, X, Y, v.wi, wl); });
       if (ne.valid && trace_any(s, ne.so, ne.sd, ne.st, v.tri, ne.tri, err)) ne.valid = false;
       if (ne.valid) L = L + beta * disney_eval(m, v.ns, X, Y, v.wi, ne.wl) * xyz(__ldg(&t.emis[ne.seg])) * ne.k;
@@ -187,14 +189,14 @@ __device__ float3 disney_forward_path(const SceneDev& s, const SegDev& t, const 
 template <int MAXD>
 __device__ void disney_adjoint_path(const SceneDev& s, const SegDev& t, const DisneyDev& D, const ViewDev& vw,
                                     uint32_t px, uint32_t py, uint32_t pid, uint32_t sample, const PathParams& pp,
-                                    double W, float3 gp, float* acc, uint32_t* err) {
+                                    bool light, float3 gp, float* acc, uint32_t* err) {
   PathRng rng;
   rng.base = make_uint4(pid, sample, pp.set_iter, 0);
   rng.key = pp.key;
   float3 o;
   float3 d = camera_ray(vw, px, py, rng, o);
   float3 beta = f3(1.0f, 1.0f, 1.0f);
-  const bool light_on = pp.nee && W > 0.0;
+  const bool light_on = pp.nee && light;
   const float es = pp.emission_scale;
   float3 T[MAXD], U[MAXD], WI[MAXD], WO[MAXD], NS[MAXD], TX[MAXD];
   float KK[MAXD];
@@ -225,7 +227,7 @@ __device__ void disney_adjoint_path(const SceneDev& s, const SegDev& t, const Di
       ua = rng.draw(k, 0);
       const float4 ub = rng.draw(k, 1);
       if (light_on) {
-        NeeResult ne = nee_prepare_with(s, t, v, ua, ub, W, pp.profile, pp.mis,
+        NeeResult ne = nee_prepare_with(s, t, v, ua, ub, pp.profile, pp.mis,
                                         [&](float3 wl) { return disney_pdf(D, v.seg, v.ns, X, Y, v.wi, wl); });
         if (ne.valid && trace_any(s, ne.so, ne.sd, ne.st, v.tri, ne.tri, err)) ne.valid = false;
         if (ne.valid) {
@@ -305,7 +307,7 @@ __global__ void __launch_bounds__(kDisneyThreads)
   const uint32_t warps_per_block = blockDim.x >> 5;
   const uint32_t n_tasks = (n_pix + ppw - 1) / ppw;
   const uint32_t stride = gridDim.x * warps_per_block;
-  const double W = *t.W;
+  const bool light = any_light(s, t);
   const float inv_spp = 1.0f / (float)pp.spp;
   double loss_acc = 0.0;
   for (uint32_t task = blockIdx.x * warps_per_block + (threadIdx.x >> 5); task < n_tasks; task += stride) {
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(kDisneyThreads)
       const uint32_t lp = pid - vw.offset;
       const uint32_t px = lp % vw.w, py = lp / vw.w;
       for (uint32_t smp = sub; smp < pp.spp; smp += G) {
-        const float3 L = disney_forward_path(s, t, D, vw, px, py, pid, s0 + smp, pp, W, err);
+        const float3 L = disney_forward_path(s, t, D, vw, px, py, pid, s0 + smp, pp, light, err);
         a = a + L;
         a2 = a2 + L * L;
       }
@@ -395,7 +397,7 @@ __global__ void __launch_bounds__(kDisneyThreads)
   const uint32_t warps_per_block = blockDim.x >> 5;
   const uint32_t n_tasks = (n_pix + ppw - 1) / ppw;
   const uint32_t stride = gridDim.x * warps_per_block;
-  const double W = *t.W;
+  const bool light = any_light(s, t);
   const float inv_spp = 1.0f / (float)pp.spp;
   for (uint32_t task = blockIdx.x * warps_per_block + (threadIdx.x >> 5); task < n_tasks; task += stride) {
     const uint32_t local = task * ppw + lane / G;
@@ -408,7 +410,7 @@ __global__ void __launch_bounds__(kDisneyThreads)
     const uint32_t lp = pid - vw.offset;
     const uint32_t px = lp % vw.w, py = lp / vw.w;
     for (uint32_t smp = sub; smp < pp.spp; smp += G)
-      disney_adjoint_path<MAXD>(s, t, D, vw, px, py, pid, s0 + smp, pp, W, gp, sgrad, err);
+      disney_adjoint_path<MAXD>(s, t, D, vw, px, py, pid, s0 + smp, pp, light, gp, sgrad, err);
   }
   __syncthreads();
   if (!gacc)
@@ -452,7 +454,7 @@ cudaError_t launch_disney_forward(const Launcher& L, const SceneBuffers& s, cons
   // the loss partials hold one row per block of the fixed loss grid
   const int cap = loss_partials_capacity(L);
   const int grid = loss_partials ? cap : disney_grid(n_pix, pp.group, cap);
-  k_disney_forward<<<grid, kDisneyThreads, 0, st>>>(scene_dev(s), seg_dev(t), DisneyDev{d.mat, d.lobe, d.samp},
+  k_disney_forward<<<grid, kDisneyThreads, 0, st>>>(scene_dev(s), seg_dev(t), DisneyDev{d.mat, d.samp},
                                                     reinterpret_cast<const ViewDev*>(views_dev), n_views, pix_begin,
                                                     n_pix, pp, img, msq, target, g_out, loss_partials, g_scale,
                                                     loss_kind, err);
@@ -473,7 +475,7 @@ cudaError_t launch_disney_adjoint(const Launcher& L, const SceneBuffers& s, cons
     cudaError_t e = cudaMemsetAsync(gacc, 0, sizeof(float) * n_par, st);
     if (e != cudaSuccess) return e;
   }
-  const DisneyDev D{d.mat, d.lobe, d.samp};
+  const DisneyDev D{d.mat, d.samp};
   const ViewDev* vd = reinterpret_cast<const ViewDev*>(views_dev);
   const int md = tp.max_depth < 1 ? 1 : (int)tp.max_depth;
   const int cap = L.num_sms * 4;

@@ -404,22 +404,22 @@ __device__ __forceinline__ float disney_pdf(const DisneyDev& D, int seg, float3 
   return pdf;
 }
 
-// Direction from the lobe chosen by u_lobe (FP64 comparison with the
-// cumulative probabilities) and (u1, u2).
+// Direction from the lobe chosen by u_lobe (against the thresholds of the
+// FP64 cumulative probabilities) and (u1, u2).
 __device__ __forceinline__ float3 disney_sample(const DisneyDev& D, int seg, float3 n, float3 X, float3 Y,
                                                 float3 wi, float u_lobe, float u1, float u2) {
-  const double2 cum = __ldg(&D.lobe[seg]);
   const float4 w = __ldg(&D.samp[2 * seg]);
+  const float t_ds = __ldg(&D.samp[2 * seg + 1]).w;
   float sphi, cphi;
   sincospif(2.0f * u2, &sphi, &cphi);
   const float rr = sqrtf(u1);
-  if ((double)u_lobe < cum.x) {
+  if (u_lobe < w.w) {
     float3 b1, b2;
     onb(n, b1, b2);
     return b1 * (rr * cphi) + b2 * (rr * sphi) + n * sqrtf(fmaxf(0.0f, 1.0f - u1));
   }
   float3 hw;
-  if ((double)u_lobe < cum.y) {
+  if (u_lobe < t_ds) {
     const float3 vl = f3(dot(wi, X), dot(wi, Y), dot(wi, n));
     const float3 vh = normalize(f3(w.x * vl.x, w.y * vl.y, vl.z));
     const float lensq = vh.x * vh.x + vh.y * vh.y;

@@ -10,6 +10,36 @@
 namespace ipt {
 
 // Result of the host scene build: BVH, triangle layout and light tables.
+#ifdef __CUDACC__
+#define IPT_HD __host__ __device__
+#else
+#define IPT_HD
+#endif
+
+// The decision u * W < a, taken in FP64 for a uniform u = k * 2^-24 (k in
+// [0, 2^24)), as an FP32 threshold T on u: the smallest multiple of 2^-24 in
+// [0, 1] for which it fails (the product is monotonic in u, so it holds below
+// T and fails from T on).  An FP32 guess brackets T; one that does not
+// (overflow, denormals) leaves the whole range to the search.
+inline IPT_HD float unit_threshold(double a, double W) {
+  const auto below = [&](int k) { return (double)k * 0x1p-24 * W < a; };
+  int lo = 0, hi = 1 << 24;
+  const float g = (float)a / (float)W * 16777216.0f;
+  if (g >= 0.0f && g <= 16777216.0f) {
+    const int k = (int)g;
+    if (k >= 8 && below(k - 8)) lo = k - 7;
+    if (k + 8 < hi && !below(k + 8)) hi = k + 8;
+  }
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (below(mid))
+      lo = mid + 1;
+    else
+      hi = mid;
+  }
+  return (float)lo * 0x1p-24f;
+}
+
 struct HostScene {
   uint32_t n_tri = 0, n_seg = 0, n_nodes = 0, depth = 0;
   std::vector<float> nodes;      // 16 floats per inner node
@@ -23,6 +53,7 @@ struct HostScene {
   std::vector<uint32_t> seg_tris;
   std::vector<uint32_t> seg_begin;
   std::vector<double> tri_cdf;
+  std::vector<float> tri_sel;    // tri_cdf as thresholds on the uniform (see unit_threshold)
   std::vector<double> seg_area;
   double diameter = 0.0;
 };
@@ -41,7 +72,7 @@ struct SceneBuffers {
   const float4* vnrm;
   const uint32_t* seg_tris;
   const uint32_t* seg_begin;
-  const double* tri_cdf;
+  const float* tri_sel;
   const double* seg_area;
   const uint32_t* orig_to_internal;
   uint32_t n_seg, n_tri;
@@ -57,8 +88,8 @@ struct SegBuffers {
   float4* mat_b;
   float4* emis;
   float4* samp;
-  double* pspec;
-  double* cdf;
+  float* sel;   // S + 1: light-selection thresholds, then 1 if any segment emits
+  double* cdf;  // FP64 prefix sums behind sel
   double* lum;
   double* W;
 };
@@ -219,11 +250,10 @@ int wf_max_blocks(const Launcher& L);
 
 // Disney material model (megakernel integrator): per-segment tables built
 // from the 16-value parameter blocks, next to the shared light-selection
-// tables in SegBuffers (emis, samp.z = p_A, cdf, lum, W).
+// tables in SegBuffers (emis, samp.z = p_A, sel, cdf, lum, W).
 struct DisneyBuffers {
-  float4* mat;    // 4 per segment: the 13 material values, then zeros
-  double2* lobe;  // cumulative lobe probabilities (P_d, P_d + P_s), FP64
-  float4* samp;   // 2 per segment: (a_x, a_y, a_c, 0), (P_d, P_s, P_c, 0)
+  float4* mat;   // 4 per segment: the 13 material values, then zeros
+  float4* samp;  // 2 per segment: (a_x, a_y, a_c, T_d), (P_d, P_s, P_c, T_ds) (see DisneyDev)
 };
 
 cudaError_t launch_disney_tables(const SceneBuffers& s, const SegBuffers& t, const DisneyBuffers& d,

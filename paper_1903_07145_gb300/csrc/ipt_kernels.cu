@@ -30,7 +30,7 @@ __global__ void k_prepare(const float* params, const float* sparams, uint32_t S,
 
 // Radiance estimate of one camera path.
 __device__ float3 forward_path(const SceneDev& s, const SegDev& t, const ViewDev& vw, uint32_t px, uint32_t py,
-                               uint32_t pid, uint32_t sample, const PathParams& pp, double W,
+                               uint32_t pid, uint32_t sample, const PathParams& pp, bool light,
                                uint32_t* err) {
   PathRng rng;
   rng.base = make_uint4(pid, sample, pp.set_iter, 0);
@@ -38,7 +38,7 @@ __device__ float3 forward_path(const SceneDev& s, const SegDev& t, const ViewDev
   float3 o;
   float3 d = camera_ray(vw, px, py, rng, o);
   float3 beta = f3(1.0f, 1.0f, 1.0f), L = f3(0.0f, 0.0f, 0.0f);
-  const bool light_on = pp.nee && W > 0.0;
+  const bool light_on = pp.nee && light;
   int skip = -1;
   float prev_pdf = 0.0f;
   for (uint32_t k = 0;; ++k) {
@@ -54,14 +54,14 @@ __device__ float3 forward_path(const SceneDev& s, const SegDev& t, const ViewDev
     const float4 ma = __ldg(&t.mat_a[v.seg]), mb = __ldg(&t.mat_b[v.seg]);
     const float4 sa = __ldg(&t.samp[v.seg]);
     if (light_on) {
-      const NeeResult ne = next_event(s, t, v, ua, ub, W, pp.profile, pp.mis, sa.y, sa.x, err);
+      const NeeResult ne = next_event(s, t, v, ua, ub, pp.profile, pp.mis, sa.y, sa.x, err);
       if (ne.valid) {
         const BrdfVal bv = brdf_eval(ma, mb, v.ns, v.wi, ne.wl);
         L = L + beta * bv.f * xyz(__ldg(&t.emis[ne.seg])) * ne.k;
       }
     }
     if (!(dot(v.wi, v.ns) > 0.0f)) break;
-    const float3 wo = bsdf_sample(__ldg(&t.pspec[v.seg]), sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
+    const float3 wo = bsdf_sample(sa.w, sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
     const float pdf = bsdf_pdf(sa.y, sa.x, v.ns, v.wi, wo);
     const float co = dot(wo, v.ns);
     if (!(dot(wo, v.ng) > 0.0f) || !(co > 0.0f) || !(pdf > 0.0f)) break;
@@ -90,7 +90,7 @@ __device__ __forceinline__ void add3(float* acc, int i, float3 v) {
 // are differentiated on the spot.  Pdfs and MIS weights are held constant.
 template <int MAXD>
 __device__ void adjoint_path(const SceneDev& s, const SegDev& t, const ViewDev& vw, uint32_t px, uint32_t py,
-                             uint32_t pid, uint32_t sample, const PathParams& pp, double W, float3 gp,
+                             uint32_t pid, uint32_t sample, const PathParams& pp, bool light, float3 gp,
                              float* acc, uint32_t* err) {
   PathRng rng;
   rng.base = make_uint4(pid, sample, pp.set_iter, 0);
@@ -98,7 +98,7 @@ __device__ void adjoint_path(const SceneDev& s, const SegDev& t, const ViewDev& 
   float3 o;
   float3 d = camera_ray(vw, px, py, rng, o);
   float3 beta = f3(1.0f, 1.0f, 1.0f);
-  const bool light_on = pp.nee && W > 0.0;
+  const bool light_on = pp.nee && light;
   const float es = pp.emission_scale;
   float3 T[MAXD], U[MAXD];
   float AD[MAXD], AS[MAXD], AR[MAXD];
@@ -127,7 +127,7 @@ __device__ void adjoint_path(const SceneDev& s, const SegDev& t, const ViewDev& 
       ua = rng.draw(k, 0);
       const float4 ub = rng.draw(k, 1);
       if (light_on) {
-        const NeeResult ne = next_event(s, t, v, ua, ub, W, pp.profile, pp.mis, sa.y, sa.x, err);
+        const NeeResult ne = next_event(s, t, v, ua, ub, pp.profile, pp.mis, sa.y, sa.x, err);
         if (ne.valid) {
           const BrdfVal bv = brdf_eval(ma, mb, v.ns, v.wi, ne.wl);
           const float3 Le = xyz(__ldg(&t.emis[ne.seg]));
@@ -144,7 +144,7 @@ __device__ void adjoint_path(const SceneDev& s, const SegDev& t, const ViewDev& 
     for (int l = 0; l < MAXD; ++l)
       if (l < nv) U[l] = U[l] + T[l] * C;
     if (last || !(dot(v.wi, v.ns) > 0.0f)) break;
-    const float3 wo = bsdf_sample(__ldg(&t.pspec[v.seg]), sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
+    const float3 wo = bsdf_sample(sa.w, sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
     const float pdf = bsdf_pdf(sa.y, sa.x, v.ns, v.wi, wo);
     const float co = dot(wo, v.ns);
     if (!(dot(wo, v.ng) > 0.0f) || !(co > 0.0f) || !(pdf > 0.0f)) break;
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_forward(SceneDev s, SegDev t,
   const uint32_t warps_per_block = blockDim.x >> 5;
   const uint32_t n_tasks = (n_pix + ppw - 1) / ppw;
   const uint32_t stride = gridDim.x * warps_per_block;
-  const double W = *t.W;
+  const bool light = any_light(s, t);
   const float inv_spp = 1.0f / (float)pp.spp;
   double loss_acc = 0.0;
   for (uint32_t task = blockIdx.x * warps_per_block + (threadIdx.x >> 5); task < n_tasks; task += stride) {
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_forward(SceneDev s, SegDev t,
       const uint32_t lp = pid - vw.offset;
       const uint32_t px = lp % vw.w, py = lp / vw.w;
       for (uint32_t smp = sub; smp < pp.spp; smp += G) {
-        const float3 L = forward_path(s, t, vw, px, py, pid, s0 + smp, pp, W, err);
+        const float3 L = forward_path(s, t, vw, px, py, pid, s0 + smp, pp, light, err);
         a = a + L;
         a2 = a2 + L * L;
       }
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_adjoint(SceneDev s, SegDev t,
   const uint32_t warps_per_block = blockDim.x >> 5;
   const uint32_t n_tasks = (n_pix + ppw - 1) / ppw;
   const uint32_t stride = gridDim.x * warps_per_block;
-  const double W = *t.W;
+  const bool light = any_light(s, t);
   const float inv_spp = 1.0f / (float)pp.spp;
   for (uint32_t task = blockIdx.x * warps_per_block + (threadIdx.x >> 5); task < n_tasks; task += stride) {
     const uint32_t local = task * ppw + lane / G;
@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(kBlockThreads) k_adjoint(SceneDev s, SegDev t,
     const uint32_t lp = pid - vw.offset;
     const uint32_t px = lp % vw.w, py = lp / vw.w;
     for (uint32_t smp = sub; smp < pp.spp; smp += G)
-      adjoint_path<MAXD>(s, t, vw, px, py, pid, s0 + smp, pp, W, gp, sgrad, err);
+      adjoint_path<MAXD>(s, t, vw, px, py, pid, s0 + smp, pp, light, gp, sgrad, err);
   }
   __syncthreads();
   if (!gacc)
@@ -382,11 +382,11 @@ __global__ void __launch_bounds__(kBlockThreads, 4)
       pid = e.pick ? e.pick[entry] : entry;
       const uint32_t s0 = e.pick ? entry * pp.stride : 0u;
       const PathParams q = scene_params(pp, e, set_iter);
-      const double W = *e.t.W;
+      const bool light = any_light(e.s, e.t);
       const ViewDev& vw = find_view(e.views, e.n_views, pid);
       const uint32_t lp = pid - vw.offset;
       const uint32_t px = lp % vw.w, py = lp / vw.w;
-      for (uint32_t smp = sub; smp < pp.spp; smp += G) a = a + forward_path(e.s, e.t, vw, px, py, pid, s0 + smp, q, W, err);
+      for (uint32_t smp = sub; smp < pp.spp; smp += G) a = a + forward_path(e.s, e.t, vw, px, py, pid, s0 + smp, q, light, err);
     }
     for (uint32_t off = G >> 1; off >= 1; off >>= 1) {
       a.x += __shfl_xor_sync(0xffffffffu, a.x, off);
@@ -446,13 +446,13 @@ __global__ void __launch_bounds__(kBlockThreads)
     const float3 gp = f3(e.g_img[3 * entry], e.g_img[3 * entry + 1], e.g_img[3 * entry + 2]) * inv_spp;
     if (gp.x == 0.0f && gp.y == 0.0f && gp.z == 0.0f) continue;
     const PathParams q = scene_params(pp, e, set_iter);
-    const double W = *e.t.W;
+    const bool light = any_light(e.s, e.t);
     const ViewDev& vw = find_view(e.views, e.n_views, pid);
     const uint32_t lp = pid - vw.offset;
     const uint32_t px = lp % vw.w, py = lp / vw.w;
     float* sacc = acc + 10u * e.seg_offset;
     for (uint32_t smp = sub; smp < pp.spp; smp += G)
-      adjoint_path<MAXD>(e.s, e.t, vw, px, py, pid, s0 + smp, q, W, gp, sacc, err);
+      adjoint_path<MAXD>(e.s, e.t, vw, px, py, pid, s0 + smp, q, light, gp, sacc, err);
   }
   __syncthreads();
   if (!gacc)
@@ -631,7 +631,9 @@ __global__ void k_tables_seg(const float* params, const float* sparams, uint32_t
     const double ld = lum_d(q[0], q[1], q[2]);
     const double ls = lum_d(q[3], q[4], q[5]);
     const double sum = __dadd_rn(ld, ls);
-    t.pspec[s] = sum > 0.0 ? __ddiv_rn(ls, sum) : 0.0;
+    const double P = sum > 0.0 ? __ddiv_rn(ls, sum) : 0.0;
+    const float rs = q[6];
+    t.samp[s] = make_float4(fmaxf(rs * rs, 1e-4f), (float)P, 0.0f, unit_threshold(P, 1.0));
     double le = lum_d(q[7], q[8], q[9]);
     if (!(le > 0.0)) le = 0.0;
     t.lum[s] = le;
@@ -685,14 +687,14 @@ __global__ void __launch_bounds__(1024) k_tables_cdf(uint32_t S, const double* s
   }
 }
 
-__global__ void k_tables_samp(const float* sparams, uint32_t S, SegBuffers t) {
+__global__ void k_tables_samp(uint32_t S, SegBuffers t) {
   const double W = *t.W;
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < S; s += gridDim.x * blockDim.x) {
-    const float rs = sparams[10 * s + 6];
     const double le = t.lum[s];
-    t.samp[s] = make_float4(fmaxf(rs * rs, 1e-4f), (float)t.pspec[s],
-                            (W > 0.0 && le > 0.0) ? (float)(le / W) : 0.0f, 0.0f);
+    t.samp[s].z = (W > 0.0 && le > 0.0) ? (float)(le / W) : 0.0f;
+    t.sel[s] = unit_threshold(t.cdf[s], W);
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) t.sel[S] = W > 0.0 ? 1.0f : 0.0f;
 }
 
 static cudaError_t launch_tables_wide(const SceneBuffers& s, const SegBuffers& t, const float* params,
@@ -700,7 +702,7 @@ static cudaError_t launch_tables_wide(const SceneBuffers& s, const SegBuffers& t
   const int grid = (int)std::min<uint32_t>((s.n_seg + 255u) / 256u, 1024u);
   k_tables_seg<<<grid, 256, 0, st>>>(params, sparams, s.n_seg, s.emission_scale, t);
   k_tables_cdf<<<1, 1024, 0, st>>>(s.n_seg, s.seg_area, t, step_dev, skip);
-  k_tables_samp<<<grid, 256, 0, st>>>(sparams, s.n_seg, t);
+  k_tables_samp<<<grid, 256, 0, st>>>(s.n_seg, t);
   return cudaGetLastError();
 }
 

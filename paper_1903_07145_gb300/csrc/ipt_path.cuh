@@ -60,8 +60,7 @@ inline SceneDev scene_dev(const SceneBuffers& s) {
   d.vnrm = s.vnrm;
   d.seg_tris = s.seg_tris;
   d.seg_begin = s.seg_begin;
-  d.tri_cdf = s.tri_cdf;
-  d.seg_area = s.seg_area;
+  d.tri_sel = s.tri_sel;
   d.n_seg = s.n_seg;
   d.n_tri = s.n_tri;
   d.eps = s.eps;
@@ -76,15 +75,14 @@ inline SegDev seg_dev(const SegBuffers& t) {
   d.mat_b = t.mat_b;
   d.emis = t.emis;
   d.samp = t.samp;
-  d.pspec = t.pspec;
-  d.cdf = t.cdf;
-  d.W = t.W;
+  d.sel = t.sel;
   return d;
 }
 
 // ---------------------------------------------------------------------------
 // Parameter tables.  Decisions that pick an integer (light segment, lobe) are
-// taken in FP64 from FP64 tables evaluated without contraction.
+// defined in FP64, from FP64 values evaluated without contraction, and
+// tabulated as FP32 thresholds on the uniform that take the same decision.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double lum_d(double r, double g, double b) {
   return __dadd_rn(__dadd_rn(__dmul_rn(kLumR, r), __dmul_rn(kLumG, g)), __dmul_rn(kLumB, b));
@@ -102,7 +100,9 @@ inline __device__ void build_tables(const float* params, const float* sparams, u
     const double ld = lum_d(q[0], q[1], q[2]);
     const double ls = lum_d(q[3], q[4], q[5]);
     const double sum = __dadd_rn(ld, ls);
-    t.pspec[s] = sum > 0.0 ? __ddiv_rn(ls, sum) : 0.0;
+    const double P = sum > 0.0 ? __ddiv_rn(ls, sum) : 0.0;
+    const float rs = q[6];
+    t.samp[s] = make_float4(fmaxf(rs * rs, 1e-4f), (float)P, 0.0f, unit_threshold(P, 1.0));
     double le = lum_d(q[7], q[8], q[9]);
     if (!(le > 0.0)) le = 0.0;
     t.lum[s] = le;
@@ -119,11 +119,11 @@ inline __device__ void build_tables(const float* params, const float* sparams, u
   __syncthreads();
   const double W = *t.W;
   for (uint32_t s = threadIdx.x; s < S; s += blockDim.x) {
-    const float rs = sparams[10 * s + 6];
     const double le = t.lum[s];
-    t.samp[s] = make_float4(fmaxf(rs * rs, 1e-4f), (float)t.pspec[s],
-                            (W > 0.0 && le > 0.0) ? (float)(le / W) : 0.0f, 0.0f);
+    t.samp[s].z = (W > 0.0 && le > 0.0) ? (float)(le / W) : 0.0f;
+    t.sel[s] = unit_threshold(t.cdf[s], W);
   }
+  if (threadIdx.x == 0) t.sel[S] = W > 0.0 ? 1.0f : 0.0f;
 }
 
 
@@ -187,6 +187,9 @@ __device__ __forceinline__ float3 camera_ray(const ViewDev& vw, uint32_t px, uin
                       M[8] * dc.x + M[9] * dc.y + M[10] * dc.z));
 }
 
+// Whether light sampling is on: some segment emits.
+__device__ __forceinline__ bool any_light(const SceneDev& s, const SegDev& t) { return __ldg(&t.sel[s.n_seg]) > 0.0f; }
+
 struct NeeResult {
   bool valid;
   int seg;       // emitting segment
@@ -205,14 +208,14 @@ struct NeeResult {
 // material sampler's solid-angle pdf towards wl (for the MIS weight).
 template <class PdfTo>
 __device__ __forceinline__ NeeResult nee_prepare_with(const SceneDev& s, const SegDev& t, const Vtx& v, float4 ua,
-                                                      float4 ub, double W, int profile, int mis,
+                                                      float4 ub, int profile, int mis,
                                                       const PdfTo& bsdf_pdf_to) {
   NeeResult r;
   r.valid = false;
-  const int sl = upper_bound_d(t.cdf, 0, (int)s.n_seg, (double)ua.w * W);
+  const int sl = upper_bound_f(t.sel, 0, (int)s.n_seg, ua.w);
   const int b = (int)__ldg(&s.seg_begin[sl]), e = (int)__ldg(&s.seg_begin[sl + 1]);
   if (e <= b) return r;  // a segment without triangles is never selectable; guard anyway
-  const int j = upper_bound_d(s.tri_cdf, b, e, (double)ub.x * __ldg(&s.seg_area[sl]));
+  const int j = upper_bound_f(s.tri_sel, b, e, ub.x);
   const int lt = (int)__ldg(&s.seg_tris[j]);
   const float3 p0 = xyz(__ldg(&s.tris[3 * lt + 0]));
   const float3 p1 = xyz(__ldg(&s.tris[3 * lt + 1]));
@@ -250,16 +253,16 @@ __device__ __forceinline__ NeeResult nee_prepare_with(const SceneDev& s, const S
 
 // Lambert + GGX: the mixture sampler of bsdf_sample.
 __device__ __forceinline__ NeeResult nee_prepare(const SceneDev& s, const SegDev& t, const Vtx& v, float4 ua,
-                                                 float4 ub, double W, int profile, int mis, float P, float a_s) {
-  return nee_prepare_with(s, t, v, ua, ub, W, profile, mis,
+                                                 float4 ub, int profile, int mis, float P, float a_s) {
+  return nee_prepare_with(s, t, v, ua, ub, profile, mis,
                           [&](float3 wl) { return bsdf_pdf(P, a_s, v.ns, v.wi, wl); });
 }
 
 // Next-event estimation with the visibility test done in place.
 __device__ __forceinline__ NeeResult next_event(const SceneDev& s, const SegDev& t, const Vtx& v, float4 ua,
-                                                float4 ub, double W, int profile, int mis, float P,
+                                                float4 ub, int profile, int mis, float P,
                                                 float a_s, uint32_t* err) {
-  NeeResult r = nee_prepare(s, t, v, ua, ub, W, profile, mis, P, a_s);
+  NeeResult r = nee_prepare(s, t, v, ua, ub, profile, mis, P, a_s);
   if (r.valid && trace_any(s, r.so, r.sd, r.st, v.tri, r.tri, err)) r.valid = false;
   return r;
 }

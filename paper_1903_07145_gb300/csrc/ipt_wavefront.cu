@@ -791,8 +791,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_shade_fwd(const WfScene* tab
     Vtx v;
     if (tri >= 0) {
       const WfScene& e = tab[lp.n_scenes == 1 ? 0u : b];
-      const double W = *e.t.W;
-      const bool light_on = lp.nee && W > 0.0;
+      const bool light_on = lp.nee && any_light(e.s, e.t);
       const float4 rd = w.ray_d[slot];
       Hit h;
       h.tri = tri;
@@ -828,7 +827,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_shade_fwd(const WfScene* tab
           float m[kDisneyMat];
           load_disney(e.dis, v.seg, m);
           if (light_on) {
-            ne = nee_prepare_with(e.s, e.t, v, ua, ub, W, lp.profile, lp.mis,
+            ne = nee_prepare_with(e.s, e.t, v, ua, ub, lp.profile, lp.mis,
                                   [&](float3 wl) { return disney_pdf(e.dis, v.seg, v.ns, X, Y, v.wi, wl); });
             if (ne.valid) {
               shc = beta * disney_eval(m, v.ns, X, Y, v.wi, ne.wl) * xyz(__ldg(&e.t.emis[ne.seg])) * ne.k;
@@ -849,7 +848,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_shade_fwd(const WfScene* tab
           const float4 ma = __ldg(&e.t.mat_a[v.seg]), mb = __ldg(&e.t.mat_b[v.seg]);
           const float4 sa = __ldg(&e.t.samp[v.seg]);
           if (light_on && (!lp.cache_record || k >= lp.cache_k)) {
-            ne = nee_prepare(e.s, e.t, v, ua, ub, W, lp.profile, lp.mis, sa.y, sa.x);
+            ne = nee_prepare(e.s, e.t, v, ua, ub, lp.profile, lp.mis, sa.y, sa.x);
             if (ne.valid) {
               const BrdfVal bv = brdf_eval(ma, mb, v.ns, v.wi, ne.wl);
               shc = beta * bv.f * xyz(__ldg(&e.t.emis[ne.seg])) * ne.k;
@@ -857,7 +856,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_shade_fwd(const WfScene* tab
             }
           }
           if (dot(v.wi, v.ns) > 0.0f) {
-            wo = bsdf_sample(__ldg(&e.t.pspec[v.seg]), sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
+            wo = bsdf_sample(sa.w, sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
             pdf = bsdf_pdf(sa.y, sa.x, v.ns, v.wi, wo);
             const float co = dot(wo, v.ns);
             if (dot(wo, v.ng) > 0.0f && co > 0.0f && pdf > 0.0f) {
@@ -1204,8 +1203,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, Wf
       finish = true;
       w.beta[slot] = make_float4(bt.x, bt.y, bt.z, __uint_as_float(st | kDead));
     } else {
-      const double W = *e.t.W;
-      const bool light_on = lp.nee && W > 0.0;
+      const bool light_on = lp.nee && any_light(e.s, e.t);
       const float3 beta = xyz(bt);
       Hit h;
       h.tri = tri;
@@ -1238,7 +1236,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, Wf
         if constexpr (kD) {
           float3 X, Y;
           hit_frame(e.s, tri, v.ns, X, Y);
-          ne = nee_prepare_with(e.s, e.t, v, ua, ub, W, lp.profile, lp.mis,
+          ne = nee_prepare_with(e.s, e.t, v, ua, ub, lp.profile, lp.mis,
                                 [&](float3 wl) { return disney_pdf(e.dis, v.seg, v.ns, X, Y, v.wi, wl); });
           if (ne.valid) {
             float m[kDisneyMat];
@@ -1253,7 +1251,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, Wf
           }
         } else {
           const float4 sa = __ldg(&e.t.samp[v.seg]);
-          ne = nee_prepare(e.s, e.t, v, ua, ub, W, lp.profile, lp.mis, sa.y, sa.x);
+          ne = nee_prepare(e.s, e.t, v, ua, ub, lp.profile, lp.mis, sa.y, sa.x);
           if (ne.valid) {
             const float4 ma = __ldg(&e.t.mat_a[v.seg]), mb = __ldg(&e.t.mat_b[v.seg]);
             const BrdfVal bv = brdf_eval(ma, mb, v.ns, v.wi, ne.wl);
@@ -1436,7 +1434,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_b(const WfScene* tab, Wf
         }
       } else if (dot(v.wi, v.ns) > 0.0f) {
         const float4 sa = __ldg(&e.t.samp[v.seg]);
-        wo = bsdf_sample(__ldg(&e.t.pspec[v.seg]), sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
+        wo = bsdf_sample(sa.w, sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
         pdf = bsdf_pdf(sa.y, sa.x, v.ns, v.wi, wo);
         const float co = dot(wo, v.ns);
         if (dot(wo, v.ng) > 0.0f && co > 0.0f && pdf > 0.0f) {

@@ -843,6 +843,7 @@ bool build_scene(const float* pos, uint32_t n_vert, const float* nrm, const uint
   for (uint32_t k = 0; k < n_seg; ++k) s.seg_begin[k + 1] += s.seg_begin[k];
   s.seg_tris.assign(n_tri, 0);
   s.tri_cdf.assign(n_tri, 0.0);
+  s.tri_sel.assign(n_tri, 0.0f);
   s.seg_area.assign(n_seg, 0.0);
   std::vector<uint32_t> fill(s.seg_begin.begin(), s.seg_begin.end() - 1);
   std::vector<uint32_t> orig_list(n_tri);
@@ -855,6 +856,7 @@ bool build_scene(const float* pos, uint32_t n_vert, const float* nrm, const uint
       s.seg_tris[j] = s.orig_to_internal[orig_list[j]];
     }
     s.seg_area[k] = acc;
+    for (uint32_t j = s.seg_begin[k]; j < s.seg_begin[k + 1]; ++j) s.tri_sel[j] = unit_threshold(s.tri_cdf[j], acc);
   }
   if (s.depth + 2 > 64) {
     *err = "BVH deeper than the traversal stack";
