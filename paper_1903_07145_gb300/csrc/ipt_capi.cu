@@ -678,7 +678,14 @@ ipt_status ipt_scene_upload(ipt_ctx* ctx, const float* pos, uint32_t n_vert, con
   H(s->nodes, hs.nodes.data(), hs.nodes.size() * sizeof(float));
   H(s->nodes4, hs.nodes4.data(), hs.nodes4.size() * sizeof(uint32_t));
   H(s->nodes8, hs.nodes8.data(), hs.nodes8.size() * sizeof(uint32_t));
-  H(s->tris, hs.tris.data(), hs.tris.size() * sizeof(float));
+  // one float4 per axis: (p0, p1, p2 coordinates, then the original id, segment id, 0)
+  std::vector<float> tris(12 * (size_t)n_tri, 0.0f);
+  for (size_t i = 0; i < n_tri; ++i)
+    for (int a = 0; a < 3; ++a) {
+      for (int v = 0; v < 3; ++v) tris[12 * i + 4 * a + v] = hs.tris[12 * i + 4 * v + a];
+      tris[12 * i + 4 * a + 3] = hs.tris[12 * i + 4 * a + 3];
+    }
+  H(s->tris, tris.data(), tris.size() * sizeof(float));
   if (s->vnrm) H(s->vnrm, hs.vnrm.data(), hs.vnrm.size() * sizeof(float));
   H(s->seg_tris, hs.seg_tris.data(), hs.seg_tris.size() * sizeof(uint32_t));
   H(s->seg_begin, hs.seg_begin.data(), hs.seg_begin.size() * sizeof(uint32_t));

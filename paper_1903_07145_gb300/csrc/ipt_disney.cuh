@@ -445,8 +445,9 @@ __device__ __forceinline__ float3 disney_sample(const DisneyDev& D, int seg, flo
 
 // Tangent frame of the hit triangle at the oriented shading normal.
 __device__ __forceinline__ void hit_frame(const SceneDev& s, int tri, float3 ns, float3& X, float3& Y) {
-  const float3 p0 = xyz(__ldg(&s.tris[3 * tri + 0]));
-  const float3 p1 = xyz(__ldg(&s.tris[3 * tri + 1]));
+  float3 p0, p1, p2;
+  int seg;
+  tri_vertices(s.tris, tri, p0, p1, p2, seg);
   tangent_frame(p1 - p0, ns, X, Y);
 }
 

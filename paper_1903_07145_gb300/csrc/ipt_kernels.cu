@@ -717,7 +717,7 @@ __global__ void k_trace_rays(SceneDev s, const uint32_t* orig_to_internal, uint3
   int sk = -1;
   if (skip && skip[i] >= 0 && (uint32_t)skip[i] < s.n_tri) sk = (int)orig_to_internal[skip[i]];
   const Hit h = trace_closest(s, o, d, __int_as_float(0x7f800000), sk, err);
-  tri_out[i] = h.tri >= 0 ? __float_as_int(__ldg(&s.tris[3 * h.tri]).w) : -1;
+  tri_out[i] = h.tri >= 0 ? tri_orig(s.tris, h.tri) : -1;
   if (t_out) t_out[i] = h.t;
   if (u_out) u_out[i] = h.u;
   if (v_out) v_out[i] = h.v;

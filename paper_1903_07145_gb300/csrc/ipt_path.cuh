@@ -140,12 +140,9 @@ struct Vtx {
 __device__ __forceinline__ Vtx make_vertex(const SceneDev& s, const Hit& h, float3 d, int profile) {
   Vtx v;
   v.tri = h.tri;
-  const float4 q0 = __ldg(&s.tris[3 * h.tri + 0]);
-  const float4 q1 = __ldg(&s.tris[3 * h.tri + 1]);
-  const float4 q2 = __ldg(&s.tris[3 * h.tri + 2]);
-  v.seg = __float_as_int(q1.w);
+  float3 p0, p1, p2;
+  tri_vertices(s.tris, h.tri, p0, p1, p2, v.seg);
   const float w0 = 1.0f - h.u - h.v;
-  const float3 p0 = xyz(q0), p1 = xyz(q1), p2 = xyz(q2);
   v.x = p0 * w0 + p1 * h.u + p2 * h.v;
   const float3 ng0 = normalize(cross(p1 - p0, p2 - p0));
   float3 ns = ng0;
@@ -217,9 +214,9 @@ __device__ __forceinline__ NeeResult nee_prepare_with(const SceneDev& s, const S
   if (e <= b) return r;  // a segment without triangles is never selectable; guard anyway
   const int j = upper_bound_f(s.tri_sel, b, e, ub.x);
   const int lt = (int)__ldg(&s.seg_tris[j]);
-  const float3 p0 = xyz(__ldg(&s.tris[3 * lt + 0]));
-  const float3 p1 = xyz(__ldg(&s.tris[3 * lt + 1]));
-  const float3 p2 = xyz(__ldg(&s.tris[3 * lt + 2]));
+  float3 p0, p1, p2;
+  int lseg;
+  tri_vertices(s.tris, lt, p0, p1, p2, lseg);
   const float su = sqrtf(ub.y);
   const float b0 = 1.0f - su, b1 = ub.z * su, b2 = 1.0f - b0 - b1;
   const float3 y = p0 * b0 + p1 * b1 + p2 * b2;

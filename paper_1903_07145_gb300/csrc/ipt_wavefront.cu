@@ -389,7 +389,7 @@ struct Trav {
   int gnode;         // 8-wide: node whose hit slots are being entered
   uint32_t gmask;    // 8-wide: its hit slots not yet entered (visiting order)
   uint32_t sgn;      // 8-wide: direction sign bits of the ray
-  int best, best_orig;
+  int best;
   float bt, bu, bv;
   bool occluded;
   uint32_t n_nodes, n_tests;
@@ -432,7 +432,6 @@ __device__ __forceinline__ void trav_init(Trav& T, float3 o, float3 d, float tma
   T.gmask = 0u;
   T.sgn = ray_sgn(T.r);
   T.best = -1;
-  T.best_orig = 0x7fffffff;
   T.bt = tmax;
   T.bu = T.bv = 0.0f;
   T.occluded = false;
@@ -446,23 +445,18 @@ __device__ __forceinline__ bool leaf_tests(const SceneDev& s, Trav& T, int leaf)
   T.n_tests += count;
   for (int i = first; i < first + count; ++i) {
     if (i == T.skip_a || i == T.skip_b) continue;
-    const float4 q0 = __ldg(&s.tris[3 * i + 0]);
-    const float4 q1 = __ldg(&s.tris[3 * i + 1]);
-    const float4 q2 = __ldg(&s.tris[3 * i + 2]);
     float t, u, v;
     if (kAny) {
-      if (tri_test(T.r, xyz(q0), xyz(q1), xyz(q2), T.tmax, t, u, v)) {
+      if (tri_test(T.r, s.tris, i, T.tmax, t, u, v)) {
         T.occluded = true;
         return true;
       }
-    } else if (tri_test(T.r, xyz(q0), xyz(q1), xyz(q2), T.bt * 1.0000002f, t, u, v)) {
-      const int orig = __float_as_int(q0.w);
-      if (t < T.bt || (t == T.bt && orig < T.best_orig)) {
+    } else if (tri_test(T.r, s.tris, i, T.bt * 1.0000002f, t, u, v)) {
+      if (t < T.bt || wins_tie(s.tris, t, T.bt, i, T.best)) {
         T.best = i;
         T.bt = t;
         T.bu = u;
         T.bv = v;
-        T.best_orig = orig;
       }
     }
   }
@@ -533,23 +527,18 @@ template <bool kAny>
 __device__ __forceinline__ bool tri_unit(const SceneDev& s, Trav& T) {
   const int i = T.tri++;
   if (i == T.skip_a || i == T.skip_b) return false;
-  const float4 q0 = __ldg(&s.tris[3 * i + 0]);
-  const float4 q1 = __ldg(&s.tris[3 * i + 1]);
-  const float4 q2 = __ldg(&s.tris[3 * i + 2]);
   float t, u, v;
   if (kAny) {
-    if (tri_test(T.r, xyz(q0), xyz(q1), xyz(q2), T.tmax, t, u, v)) {
+    if (tri_test(T.r, s.tris, i, T.tmax, t, u, v)) {
       T.occluded = true;
       return true;
     }
-  } else if (tri_test(T.r, xyz(q0), xyz(q1), xyz(q2), T.bt * 1.0000002f, t, u, v)) {
-    const int orig = __float_as_int(q0.w);
-    if (t < T.bt || (t == T.bt && orig < T.best_orig)) {
+  } else if (tri_test(T.r, s.tris, i, T.bt * 1.0000002f, t, u, v)) {
+    if (t < T.bt || wins_tie(s.tris, t, T.bt, i, T.best)) {
       T.best = i;
       T.bt = t;
       T.bu = u;
       T.bv = v;
-      T.best_orig = orig;
     }
   }
   return false;
