@@ -77,9 +77,12 @@ void stage_end(void* user) {
 ipt::SceneBuffers buffers(const ipt_ctx* ctx, const DeviceScene* s) {
   ipt::SceneBuffers b;
   b.counters = ctx->counters_dev;
-  b.wide = ctx->cfg.bvh_width == 2 ? 0 : (ctx->cfg.bvh_width == 8 ? 2 : 1);
+  b.wide = ctx->cfg.bvh_width == 2 ? 0 : (ctx->cfg.bvh_width == 8 ? 2 : (s->nodes4g ? 3 : 1));
   b.nodes = s->nodes;
   b.nodes4 = s->nodes4;
+  b.nodes4g = s->nodes4g;
+  std::copy(s->grid_lo, s->grid_lo + 3, b.grid_lo);
+  std::copy(s->grid_s, s->grid_s + 3, b.grid_s);
   b.nodes8 = s->nodes8;
   b.tris = s->tris;
   b.vnrm = s->vnrm;
@@ -646,6 +649,11 @@ ipt_status ipt_scene_upload(ipt_ctx* ctx, const float* pos, uint32_t n_vert, con
   };
   A(&s->nodes, 4 * (size_t)hs.n_nodes);
   A(&s->nodes4, 4 * (size_t)hs.n_nodes4);
+  if (!hs.nodes4g.empty()) {
+    A(&s->nodes4g, 4 * (size_t)hs.n_nodes4);
+    std::copy(hs.grid_lo, hs.grid_lo + 3, s->grid_lo);
+    std::copy(hs.grid_s, hs.grid_s + 3, s->grid_s);
+  }
   A(&s->nodes8, 6 * (size_t)hs.n_nodes8);
   A(&s->tris, 3 * (size_t)n_tri);
   if (!hs.vnrm.empty()) A(&s->vnrm, 3 * (size_t)n_tri);
@@ -677,6 +685,7 @@ ipt_status ipt_scene_upload(ipt_ctx* ctx, const float* pos, uint32_t n_vert, con
   };
   H(s->nodes, hs.nodes.data(), hs.nodes.size() * sizeof(float));
   H(s->nodes4, hs.nodes4.data(), hs.nodes4.size() * sizeof(uint32_t));
+  if (s->nodes4g) H(s->nodes4g, hs.nodes4g.data(), hs.nodes4g.size() * sizeof(uint32_t));
   H(s->nodes8, hs.nodes8.data(), hs.nodes8.size() * sizeof(uint32_t));
   // one float4 per axis: (p0, p1, p2 coordinates, then the original id, segment id, 0)
   std::vector<float> tris(12 * (size_t)n_tri, 0.0f);

@@ -104,6 +104,8 @@ struct DeviceScene {
   // geometry
   float4* nodes = nullptr;
   uint4* nodes4 = nullptr;
+  uint4* nodes4g = nullptr;  // planes on the scene grid, or null (see HostScene)
+  float grid_lo[3] = {0, 0, 0}, grid_s[3] = {0, 0, 0};
   uint4* nodes8 = nullptr;
   float4* tris = nullptr;
   float4* vnrm = nullptr;

@@ -45,6 +45,12 @@ struct HostScene {
   std::vector<float> nodes;      // 16 floats per inner node
   std::vector<uint32_t> nodes4;  // 16 words per 4-wide quantized node
   uint32_t n_nodes4 = 0;
+  // the same 4-wide nodes with their planes on one 15-bit grid over the scene
+  // (plane q of axis a at grid_lo[a] + q * grid_s[a] / 32768); empty when the
+  // grid would widen the boxes too much
+  std::vector<uint32_t> nodes4g;
+  float grid_lo[3] = {0, 0, 0}, grid_s[3] = {0, 0, 0};
+  double grid_cost = 0.0;        // growth of the child boxes against nodes4's (see the builder)
   std::vector<uint32_t> nodes8;  // 24 words per 8-wide quantized node
   uint32_t n_nodes8 = 0;
   std::vector<float> tris;       // 12 floats per triangle (leaf order)
@@ -67,7 +73,9 @@ bool build_scene(const float* pos, uint32_t n_vert, const float* nrm, const uint
 struct SceneBuffers {
   const float4* nodes;
   const uint4* nodes4;
+  const uint4* nodes4g;
   const uint4* nodes8;
+  float grid_lo[3], grid_s[3];   // plane grid of nodes4g
   const float4* tris;
   const float4* vnrm;
   const uint32_t* seg_tris;
@@ -79,7 +87,7 @@ struct SceneBuffers {
   float eps;
   float emission_scale;
   unsigned long long* counters;  // nullptr unless counting
-  int wide;                      // 0: binary BVH, 1: 4-wide, 2: 8-wide quantized BVH
+  int wide;                      // BVH to walk, see SceneDev::wide
 };
 
 // Per-segment parameter tables (device).

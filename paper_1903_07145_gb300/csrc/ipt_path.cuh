@@ -55,6 +55,9 @@ inline SceneDev scene_dev(const SceneBuffers& s) {
   SceneDev d;
   d.nodes = s.nodes;
   d.nodes4 = s.nodes4;
+  d.nodes4g = s.nodes4g;
+  d.grid_lo = make_float3(s.grid_lo[0], s.grid_lo[1], s.grid_lo[2]);
+  d.grid_s = make_float3(s.grid_s[0], s.grid_s[1], s.grid_s[2]);
   d.nodes8 = s.nodes8;
   d.tris = s.tris;
   d.vnrm = s.vnrm;

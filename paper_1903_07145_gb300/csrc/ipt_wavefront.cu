@@ -379,8 +379,11 @@ __global__ void __launch_bounds__(kSortThreads) wf_bin_scatter(uint32_t n_bins, 
 // a per-lane local array.  An entry is (node link, entry distance bits).
 constexpr int kShortStack = 12;
 
+constexpr int kGrid4 = 5;  // kWidth of the 4-wide BVH with planes on the scene grid
+
 struct Trav {
   RayPre r;
+  GridRay g;  // kGrid4
   float3 oinv;
   float tmax;
   int skip_a, skip_b;
@@ -419,8 +422,10 @@ __device__ __forceinline__ uint2 st_pop(const Stack& S, Trav& T) {
   return T.sp < kShortStack ? S.sh[T.sp * kWfThreads] : S.deep[T.sp - kShortStack];
 }
 
-__device__ __forceinline__ void trav_init(Trav& T, float3 o, float3 d, float tmax, int skip_a, int skip_b) {
+template <int kWidth>
+__device__ __forceinline__ void trav_init(const WfScene& e, Trav& T, float3 o, float3 d, float tmax, int skip_a, int skip_b) {
   T.r = ray_pre(o, d);
+  if constexpr (kWidth == kGrid4) T.g = grid_ray(e.s.grid_lo, e.s.grid_s, T.r);
   T.oinv = f3(o.x * T.r.inv.x, o.y * T.r.inv.y, o.z * T.r.inv.z);
   T.tmax = tmax;
   T.skip_a = skip_a;
@@ -586,31 +591,43 @@ __device__ __forceinline__ bool tri_step(const SceneDev& s, Trav& T, const Stack
 // One 4-wide node test: hit children nearest first (for shadow rays too: an
 // occluder near the shading point is found after fewer visits, -5% shadow
 // traversal time on the 61k room against slot order), the nearest entered;
-// a missed node pops the next entry.
-template <bool kAny>
+// a missed node pops the next entry.  Hits are told by their finite distance
+// after the sort (no mask to build and count), and while the lane's stack
+// leaves room for three entries they are stored without a bound check each
+// (61k room: closest hit 39.8 -> 37.8 ms, shadow rays 22.1 -> 21.0 ms).
+template <bool kAny, bool kGrid>
 __device__ __forceinline__ bool node_step4(const SceneDev& s, Trav& T, const Stack& S, uint32_t* err) {
-  if (T.node >= 0) {
-    ++T.n_nodes;
-    float tn[4];
-    int ref[4];
-    const uint32_t mask = node4_children(s, T.node, T.r, kAny ? T.tmax : T.bt, tn, ref);
-    const int k = __popc(mask);
-    if (k > 0) {
-      if (T.sp + k - 1 > kStackSize) {
-        atomicOr(err, kErrStack);
-        T.best = -1;
-        T.occluded = true;
-        return true;
-      }
-      sort4(tn, ref);
+  ++T.n_nodes;
+  float tn[4];
+  int ref[4];
+  if constexpr (kGrid)
+    node4g_children(s, T.node, T.g, (kAny ? T.tmax : T.bt) * 1.0000005f, tn, ref);
+  else
+    node4_children(s, T.node, T.r, kAny ? T.tmax : T.bt, tn, ref);
+  sort4(tn, ref);
+  const float inf = __int_as_float(0x7f800000);
+  if (tn[0] == inf) return advance4<kAny>(T, S);  // no child hit
+  if (T.sp + 3 <= kShortStack) {  // the usual case: at most three entries, all in shared memory
 #pragma unroll
-      for (int i = 3; i >= 1; --i)
-        if (i < k) st_push(S, T, ref[i], tn[i]);
-      trav_enter(T, ref[0]);
-      return false;
+    for (int i = 3; i >= 1; --i)
+      if (tn[i] != inf) {
+        S.sh[T.sp * kWfThreads] = make_uint2((uint32_t)ref[i], __float_as_uint(tn[i]));
+        ++T.sp;
+      }
+  } else {
+    const int k = 1 + (tn[1] != inf) + (tn[2] != inf) + (tn[3] != inf);
+    if (T.sp + k - 1 > kStackSize) {
+      atomicOr(err, kErrStack);
+      T.best = -1;
+      T.occluded = true;
+      return true;
     }
+#pragma unroll
+    for (int i = 3; i >= 1; --i)
+      if (i < k) st_push(S, T, ref[i], tn[i]);
   }
-  return advance4<kAny>(T, S);
+  trav_enter(T, ref[0]);
+  return false;
 }
 
 // One 8-wide node test: a node with hits becomes the current group (the
@@ -727,13 +744,17 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_trace(const WfScene* tab, Wf
         item = i;
         // a launch over one scene skips the lookup of the ray's scene
         const uint32_t slot = kAny ? w.sh_meta[i].x : qsrc[i];
-        if (!one_scene) sd = tab[state_scene(__float_as_uint(w.beta[slot].w))].s;
+        uint32_t b = 0;
+        if (!one_scene) {
+          b = state_scene(__float_as_uint(w.beta[slot].w));
+          sd = tab[b].s;
+        }
         if (kAny) {
           const float4 o = w.sh_o[i], d = w.sh_d[i];
-          trav_init(T, xyz(o), xyz(d), d.w, __float_as_int(o.w), (int)w.sh_meta[i].y);
+          trav_init<kWidth>(tab[b], T, xyz(o), xyz(d), d.w, __float_as_int(o.w), (int)w.sh_meta[i].y);
         } else {
           const float4 o = w.ray_o[slot], d = w.ray_d[slot];
-          trav_init(T, xyz(o), xyz(d), __int_as_float(0x7f800000), __float_as_int(o.w), -1);
+          trav_init<kWidth>(tab[b], T, xyz(o), xyz(d), __int_as_float(0x7f800000), __float_as_int(o.w), -1);
         }
       }
     }
@@ -754,7 +775,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_trace(const WfScene* tab, Wf
         if (live && at_tri == tri_phase)
           fin = at_tri        ? tri_step<kAny, kWidth>(sd, T, S)
                 : kWidth == 8 ? node_step8<kAny>(sd, T, S, err)
-                              : node_step4<kAny>(sd, T, S, err);
+                              : node_step4<kAny, kWidth == kGrid4>(sd, T, S, err);
       }
     }
   }
@@ -1658,24 +1679,31 @@ static uint32_t total_pixels(const std::vector<WfScene>& tab) {
   return tab.empty() ? 0u : tab.back().pix_begin + tab.back().n_pix;
 }
 
-// BVH width every scene of the table can be traversed with: 8 when all of
-// them select the 8-wide BVH, 4 when all have a wide one, else 2.
+// BVH every scene of the table can be traversed with: 8 when all of them
+// select the 8-wide BVH, 4 when all have a wide one (kGrid4 when all have its
+// planes on their grid), else 2.
 static int table_width(const std::vector<WfScene>& tab) {
-  bool w8 = true, w4 = true;
+  bool w8 = true, w4 = true, grid = true;
   for (const WfScene& e : tab) {
     w8 = w8 && e.s.wide == 2 && e.s.nodes8;
     w4 = w4 && e.s.wide >= 1 && e.s.nodes4;
+    grid = grid && e.s.wide == 3;
   }
-  return w8 ? 8 : (w4 ? 4 : 2);
+  return w8 ? 8 : (grid ? kGrid4 : (w4 ? 4 : 2));
 }
 
-// One launch of traversal mode kMode over the table's BVH width.
+// One launch of traversal mode kMode over the table's BVH width.  The scene-
+// grid nodes serve closest hits only: shadow rays visit fewer nodes per ray
+// set-up and gained nothing (61k room 20.95 -> 20.7 ms, 516k room 30.9 -> 31.7
+// ms), where closest hit went 37.8 -> 35.7 and 56.2 -> 54.0 ms.
 template <int kMode, bool kCount>
 static void launch_trace_w(int width, int grid, const WfScene* tab_dev, int one, const WfDev& w, int cur, int steps,
                            uint32_t* err, cudaStream_t st, const uint32_t* order) {
   if (width == 8)
     wf_trace<kMode, 8, kCount><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
-  else if (width == 4)
+  else if (kMode == 0 && width == kGrid4)
+    wf_trace<0, kGrid4, kCount><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
+  else if (width == 4 || width == kGrid4)
     wf_trace<kMode, 4, kCount><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
   else
     wf_trace<kMode, 2, kCount><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
@@ -1985,9 +2013,11 @@ cudaError_t wf_init(Launcher* L) {
   const void* variants[] = {
       (const void*)wf_trace<0, 2, false>, (const void*)wf_trace<1, 2, false>, (const void*)wf_trace<2, 2, false>,
       (const void*)wf_trace<0, 4, false>, (const void*)wf_trace<1, 4, false>, (const void*)wf_trace<2, 4, false>,
+      (const void*)wf_trace<0, kGrid4, false>,
       (const void*)wf_trace<0, 8, false>, (const void*)wf_trace<1, 8, false>, (const void*)wf_trace<2, 8, false>,
       (const void*)wf_trace<0, 2, true>, (const void*)wf_trace<1, 2, true>, (const void*)wf_trace<2, 2, true>,
       (const void*)wf_trace<0, 4, true>, (const void*)wf_trace<1, 4, true>, (const void*)wf_trace<2, 4, true>,
+      (const void*)wf_trace<0, kGrid4, true>,
       (const void*)wf_trace<0, 8, true>, (const void*)wf_trace<1, 8, true>, (const void*)wf_trace<2, 8, true>};
   for (const void* k : variants) {
     int bk = 0;

@@ -1,0 +1,79 @@
+"""Every BVH form gives the same hits: binary, 4-wide (8-bit boxes, or planes
+on the scene grid where the builder picks it) and 8-wide, on meshes where the
+forms differ most: coincident triangles (exact ties), a flat sheet, a small
+detail in a large scene (keeps the 8-bit boxes), one and two triangles."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1903_07145_gb300 import scenes
+from paper_1903_07145_gb300.scenes import Scene
+from paper_1903_07145_gb300.tracer import TraceOptions, Tracer
+
+pytestmark = pytest.mark.gpu
+
+
+def _mesh(pos, seed=0):
+    pos = np.asarray(pos, np.float32).reshape(-1, 3, 3)
+    n = len(pos)
+    cam = scenes.look_camera(pos.mean((0, 1)) + np.array([0, 0, 3 * np.ptp(pos) / 2]), 0.0, 0.0, 60.0, 24, 20)
+    gt = np.full((2, 10), 0.4, np.float32)
+    return Scene("mesh", pos.reshape(-1, 3), np.arange(3 * n, dtype=np.uint32).reshape(n, 3),
+                 (np.arange(n) % 2).astype(np.uint32), 2, [cam], gt)
+
+
+def _soup(n, size=0.2, scale=1.0):
+    rng = np.random.default_rng(n)
+    return scale * (rng.uniform(-2, 2, (n, 1, 3)) + rng.uniform(-size, size, (n, 3, 3)))
+
+
+def _forms():
+    soup = _soup(600)
+    sheet = _soup(500)
+    sheet[..., 1] = 0.25
+    return {
+        "ties": np.concatenate([soup, soup, soup[::-1]]),
+        "flat": sheet,
+        "detail": np.concatenate([_soup(2000, 0.3, 1e-3), [[[-40, -40, -40], [-41, -40, -40], [-40, -41, -41]],
+                                                            [[40, 40, 40], [41, 40, 40], [40, 41, 41]]]]),
+        "one": _soup(1),
+        "two": _soup(2),
+    }
+
+
+@pytest.mark.parametrize("name", ["ties", "flat", "detail", "one", "two"])
+def test_bvh_forms_give_the_same_hits(name):
+    pos = _forms()[name].astype(np.float32)
+    sc = _mesh(pos)
+    tr = Tracer(sc, seed=1)
+    tr.set_params(sc.gt_params)
+    rng = np.random.default_rng(3)
+    n = 20011
+    # towards points on the triangles, and along the axes through them
+    tri = pos[rng.integers(0, len(pos), n)].astype(np.float64)
+    w = rng.dirichlet((1, 1, 1), n)
+    target = (tri * w[:, :, None]).sum(1)
+    o = target + rng.normal(size=(n, 3)) * rng.choice([1e-2, 1.0, 100.0], (n, 1))
+    d = target - o
+    ax = rng.integers(0, 3, n)
+    axis = rng.random(n) < 0.2
+    d[axis] = np.eye(3)[ax[axis]] * np.where(rng.random(axis.sum()) < 0.5, -1, 1)[:, None]
+    o[axis] = target[axis] - 2.0 * d[axis]
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    o, d = (torch.from_numpy(a.astype(np.float32)).cuda() for a in (o, d))
+    opts = TraceOptions(spp_r=4, max_depth=2)
+    ref = img = None
+    for width in (2, 4, 8):
+        tr.configure(bvh_width=width)
+        got = [v.cpu() for v in tr.trace_rays(o, d)]
+        pic = tr.render(opts).cpu()
+        if ref is None:
+            ref, img = got, pic
+            assert (ref[0] >= 0).float().mean() > 0.5
+        for a, b in zip(ref, got):
+            assert torch.equal(a, b), f"width {width}"
+        assert torch.equal(img, pic), f"width {width}"
+    if name == "ties":  # the smallest id of the coincident copies
+        hit = ref[0][ref[0] >= 0].numpy()
+        assert (hit < 600).all()
+    tr.close()
