@@ -229,7 +229,8 @@ ipt_status ensure_wf(ipt_ctx* ctx, bool adjoint, uint32_t n_params, bool disney,
     // block-private rows for chunks whose accumulators fit in shared memory;
     // a wider chunk accumulates in one row in global memory
     const size_t shared_params = std::min<size_t>(keep_params, 10u * ipt::wf_max_segments());
-    A(&w.blk, std::max((size_t)ipt::wf_max_blocks(ctx->L) * shared_params, (size_t)keep_params));
+    // (padded to 12 floats per 10)
+    A(&w.blk, std::max((size_t)ipt::wf_max_blocks(ctx->L) * shared_params, (size_t)keep_params * 6 / 5 + 16));
   }
   if (e != cudaSuccess) {
     wf_release(ctx);

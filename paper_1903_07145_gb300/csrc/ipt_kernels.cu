@@ -484,6 +484,11 @@ __global__ void k_finalize(const double* loss_partials, int n_partials, double* 
     for (uint32_t i = threadIdx.x; i < n_params; i += blockDim.x) grad_out[i] = (float)grad_acc[i];
 }
 
+__global__ void k_grad_out(const double* grad_acc, float* grad_out, uint32_t n_params) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_params; i += gridDim.x * blockDim.x)
+    grad_out[i] = (float)grad_acc[i];
+}
+
 // Adam on the concatenated parameters of a batch, one block per member,
 // followed by that member's tables for the next iteration.
 __device__ __forceinline__ void adam_range(float* params, float* m, float* v, const uint8_t* free_mask,
@@ -892,7 +897,13 @@ cudaError_t launch_adjoint_batch(const Launcher& L, const WfScene* tab_dev, uint
 cudaError_t launch_finalize(const double* loss_partials, int n_partials, double* loss_dev,
                             const double* grad_acc, float* grad_out, uint32_t n_params,
                             cudaStream_t st) {
-  k_finalize<<<1, 256, 0, st>>>(loss_partials, n_partials, loss_dev, grad_acc, grad_out, n_params);
+  // many parameters (a segment per triangle): the gradient leaves over a grid
+  // (100k values: 96 us by the one block)
+  const bool wide = grad_out && n_params > 10u * kWideSegments;
+  if (wide)
+    k_grad_out<<<(int)std::min<uint32_t>((n_params + 255u) / 256u, 1024u), 256, 0, st>>>(grad_acc, grad_out, n_params);
+  if (!wide || loss_dev)
+    k_finalize<<<1, 256, 0, st>>>(loss_partials, n_partials, loss_dev, grad_acc, wide ? nullptr : grad_out, n_params);
   return cudaGetLastError();
 }
 

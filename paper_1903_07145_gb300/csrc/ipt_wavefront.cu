@@ -1043,25 +1043,125 @@ __device__ __forceinline__ void warp_scatter(float* acc, int base, const float (
   }
 }
 
-__device__ __forceinline__ void warp_scatter3(float* acc, int base, float3 a) {
-  const float v[3] = {a.x, a.y, a.z};
-  warp_scatter<3>(acc, base, v);
+// Gradient accumulators of a stage, by row (a segment of the launch).  P: values
+// per segment.  kW = false: the block's shared rows.  kW (chunks with more
+// segments than shared memory holds): one array in global memory for all
+// blocks, rows padded to groups of four floats so that a vector reduction adds
+// a group at once: 12 floats (kd, roughness | ks, - | emission, -) for P = 10,
+// 16 for P = 16 (one reduction instead of three to seven per group).  Every
+// triangle of a 10k-triangle room a segment, 1.2M paths a pass, depth 4: first
+// adjoint stage 4.2 -> 0.9 ms, connection 5.4 -> 1.6 ms.  The rest of the
+// connection is the additions of nearly every path to a few light triangles'
+// rows.  (Collecting those in shared memory per block took it to 0.3 ms, but
+// rounds differently: single FP32 sums of millions of terms sit up to 0.6%
+// off, and a form that is right there no longer agrees with them to FP32.)
+__host__ __device__ constexpr uint32_t wide_stride(uint32_t P) { return P == 10u ? 12u : P; }
+
+__device__ __forceinline__ void red4(float* p, float a, float b, float c, float d) {
+  if (a != 0.0f || b != 0.0f || c != 0.0f || d != 0.0f)
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
+                 : "memory");
 }
 
-// Accumulator index of parameter j of segment `seg` of scene entry e.
-__device__ __forceinline__ int acc_ix(const WfScene& e, const WfParams& lp, int seg, int j) {
-  return (lp.gacc ? 10 : 11) * ((int)e.seg_offset + seg - (int)lp.seg_lo) + j;
+template <uint32_t P, bool kW>
+struct Accum {
+  static constexpr int kMat = P == 10u ? 7 : 13;  // material values of a row; 3 of emission follow
+  float* p;
+
+  __device__ __forceinline__ void init(uint32_t seg_n) {
+    if constexpr (!kW) acc_zero(p, acc_shared_floats(P, seg_n));
+  }
+
+  __device__ __forceinline__ void flush(uint32_t seg_n, float* blk) const {
+    if constexpr (!kW) acc_flush<P>(p, P * seg_n, blk);
+  }
+
+  __device__ __forceinline__ void add_emission(int row, float x, float y, float z) const {
+    float* q = p + (size_t)wide_stride(P) * row;
+    if constexpr (P == 10u)
+      red4(q + 8, x, y, z, 0.0f);
+    else
+      red4(q + 12, 0.0f, x, y, z);
+  }
+
+  __device__ __forceinline__ void add_material(int row, const float (&g)[kMat]) const {
+    float* q = p + (size_t)wide_stride(P) * row;
+    if constexpr (P == 10u) {
+      red4(q, g[0], g[1], g[2], g[6]);
+      red4(q + 4, g[3], g[4], g[5], 0.0f);
+    } else {
+      red4(q, g[0], g[1], g[2], g[3]);
+      red4(q + 4, g[4], g[5], g[6], g[7]);
+      red4(q + 8, g[8], g[9], g[10], g[11]);
+      red4(q + 12, g[12], 0.0f, 0.0f, 0.0f);
+    }
+  }
+
+  // Both: every lane of the warp calls; row < 0 adds nothing.
+  __device__ __forceinline__ void emission(int row, float3 v) const {
+    if constexpr (kW) {
+      const unsigned want = __ballot_sync(0xffffffffu, row >= 0);
+      if (!want) return;
+      const int r0 = __shfl_sync(0xffffffffu, row, __ffs(want) - 1);
+      if (__popc(want) > 1 && __all_sync(0xffffffffu, row < 0 || row == r0)) {
+        float3 t = row >= 0 ? v : f3(0.f, 0.f, 0.f);
+#pragma unroll
+        for (int off = 16; off >= 1; off >>= 1) {
+          t.x += __shfl_xor_sync(0xffffffffu, t.x, off);
+          t.y += __shfl_xor_sync(0xffffffffu, t.y, off);
+          t.z += __shfl_xor_sync(0xffffffffu, t.z, off);
+        }
+        if ((threadIdx.x & 31u) == 0) add_emission(r0, t.x, t.y, t.z);
+      } else if (row >= 0) {
+        add_emission(row, v.x, v.y, v.z);
+      }
+    } else {
+      const float a[3] = {v.x, v.y, v.z};
+      warp_scatter<3>(p, row < 0 ? -1 : (int)(P + 1u) * row + kMat, a);
+    }
+  }
+
+  __device__ __forceinline__ void material(int row, const float (&g)[kMat]) const {
+    if constexpr (kW) {
+      // a warp holds samples of a few pixels: groups of at least four lanes on
+      // one row (their first vertices) are summed before they are added
+      unsigned rest = __ballot_sync(0xffffffffu, row >= 0);
+#pragma unroll 1
+      for (int round = 0; round < 4 && rest; ++round) {
+        const int r0 = __shfl_sync(0xffffffffu, row, __ffs(rest) - 1);
+        const unsigned grp = __ballot_sync(0xffffffffu, row == r0) & rest;
+        if (__popc(grp) < 4) break;
+        float t[kMat];
+#pragma unroll
+        for (int j = 0; j < kMat; ++j) {
+          t[j] = row == r0 ? g[j] : 0.0f;
+#pragma unroll
+          for (int off = 16; off >= 1; off >>= 1) t[j] += __shfl_xor_sync(0xffffffffu, t[j], off);
+        }
+        if ((threadIdx.x & 31u) == 0) add_material(r0, t);
+        rest &= ~grp;
+      }
+      if (rest >> (threadIdx.x & 31u) & 1u) add_material(row, g);
+    } else {
+      warp_scatter<kMat>(p, row < 0 ? -1 : (int)(P + 1u) * row, g);
+    }
+  }
+};
+
+// The stage's accumulators (kW = false: in its dynamic shared memory).
+#define IPT_ACCUM(P, kW, acc)               \
+  extern __shared__ float sacc_sh[];        \
+  Accum<P, kW> acc{kW ? lp.gacc : sacc_sh}; \
+  acc.init(lp.seg_n)
+
+// Accumulator row of segment `seg` of scene entry e.
+__device__ __forceinline__ int acc_row(const WfScene& e, const WfParams& lp, int seg) {
+  return (int)e.seg_offset + seg - (int)lp.seg_lo;
 }
 
 __device__ __forceinline__ float3 pixel_grad(const WfScene& e, uint32_t entry, float inv_spp) {
   return f3(e.g_img[3 * entry], e.g_img[3 * entry + 1], e.g_img[3 * entry + 2]) * inv_spp;
 }
-
-// The same for the Disney model's 16 values per segment.
-__device__ __forceinline__ int acc_ix16(const WfScene& e, const WfParams& lp, int seg, int j) {
-  return (lp.gacc ? kDisneyStride : kDisneyStride + 1) * ((int)e.seg_offset + seg - (int)lp.seg_lo) + j;
-}
-
 
 // Continuation terms of the paths that finish: (dw_l / dtheta) . (g * U_l)
 // for every vertex l.  All 32 lanes call it; lanes with act = false (or with
@@ -1069,15 +1169,15 @@ __device__ __forceinline__ int acc_ix16(const WfScene& e, const WfParams& lp, in
 // Disney model rebuilds vertex l (shading normal, tangent frame) from its
 // stored triangle, barycentrics and directions and contracts the BRDF
 // Jacobian there with g * U_l * cos/pdf.
-template <bool kD>
+template <bool kD, class A>
 __device__ __forceinline__ void finish_path(const WfDev& w, const WfScene* e, const WfParams& lp, uint32_t slot,
-                                            uint32_t nv_slot, float3 gp, float* sacc, bool act) {
+                                            uint32_t nv_slot, float3 gp, const A& acc, bool act) {
   const uint32_t nv = act ? nv_slot : 0u;
   const uint32_t nmax = __reduce_max_sync(0xffffffffu, nv);
   for (uint32_t l = 0; l < nmax; ++l) {
     if constexpr (kD) {
       float g[kDisneyMat];
-      int base = -1;
+      int row = -1;
       if (l < nv) {
         const size_t ix = (size_t)l * w.cap + slot;
         const float4 T = w.aT[ix], U = w.aU[ix], Wi = w.aWi[ix], Wo = w.aWo[ix];
@@ -1095,15 +1195,15 @@ __device__ __forceinline__ void finish_path(const WfDev& w, const WfScene* e, co
           const int sg = __float_as_int(R.y);
           float m[kDisneyMat];
           load_disney(e->dis, sg, m);
-          if (disney_vjp(m, v.ns, X, Y, xyz(Wi), xyz(Wo), q, g)) base = acc_ix16(*e, lp, sg, 0);
+          if (disney_vjp(m, v.ns, X, Y, xyz(Wi), xyz(Wo), q, g)) row = acc_row(*e, lp, sg);
         }
       }
-      if (base < 0)
+      if (row < 0)
         for (int j = 0; j < kDisneyMat; ++j) g[j] = 0.0f;
-      warp_scatter<kDisneyMat>(sacc, base, g);
+      acc.material(row, g);
     } else {
       float g[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      int base = -1;
+      int row = -1;
       if (l < nv) {
         const size_t ix = (size_t)l * w.cap + slot;
         const float4 T = w.aT[ix], U = w.aU[ix];
@@ -1118,9 +1218,9 @@ __device__ __forceinline__ void finish_path(const WfDev& w, const WfScene* e, co
         g[4] = q.y * U.w;
         g[5] = q.z * U.w;
         g[6] = dot(q, f3(mb.x, mb.y, mb.z)) * R.x;
-        base = acc_ix(*e, lp, sg, 0);
+        row = acc_row(*e, lp, sg);
       }
-      warp_scatter<7>(sacc, base, g);
+      acc.material(row, g);
     }
   }
 }
@@ -1177,13 +1277,11 @@ __device__ __forceinline__ void scale_carry(const WfDev& w, uint32_t slot, uint3
 // Stage A: emission at the vertex, its contribution to the carry, and the
 // next-event candidate (with, for the Disney model, the material derivative
 // of its term, added if the shadow ray finds the light).
-template <bool kD>
+template <bool kD, bool kW>
 __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, WfParams lp, uint32_t p0, WfDev w,
                                                        int cur) {
-  extern __shared__ float sacc_sh[];
-  float* sacc = lp.gacc ? lp.gacc : sacc_sh;
-  const uint32_t np = (kD ? 16u : 10u) * lp.seg_n;
-  if (!lp.gacc) acc_zero(sacc, acc_shared_floats(kD ? 16u : 10u, lp.seg_n));
+  constexpr uint32_t P = kD ? 16u : 10u;
+  IPT_ACCUM(P, kW, acc);
   const uint32_t n = w.cnt[cur];
   const uint32_t si = set_iter(lp);
   const float inv_spp = 1.0f / (float)lp.spp;
@@ -1219,7 +1317,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, Wf
     float spec = 0.0f, dsdr = 0.0f;
     float gd[kDisneyMat];
     int vseg = 0;
-    int ebase = -1;  // accumulator of the emission found here
+    int erow = -1;  // accumulator row of the emission found here
     float3 ev = f3(0.f, 0.f, 0.f);
     float4 cq = make_float4(0.f, 0.f, 0.f, 0.f);
     Vtx cv;
@@ -1242,7 +1340,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, Wf
         if (wb > 0.0f) {
           const float f = wb * v.prof;
           add_to_carry<2>(w, slot, nv, xyz(__ldg(&e.t.emis[v.seg])) * f);
-          ebase = kD ? acc_ix16(e, lp, v.seg, kDisneyMat) : acc_ix(e, lp, v.seg, 7);
+          erow = acc_row(e, lp, v.seg);
           ev = gp * beta * (f * e.es);
         }
       }
@@ -1291,8 +1389,8 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, Wf
         }
       }
     }
-    warp_scatter3(sacc, ebase, ev);
-    finish_path<kD>(w, &e, lp, slot, nv, gp, sacc, finish);
+    acc.emission(erow, ev);
+    finish_path<kD>(w, &e, lp, slot, nv, gp, acc, finish);
     if (lp.cache_k != kNoCache) {
       const uint32_t qi = enqueue(&lp.cb.counts[0], query);
       if (query) {
@@ -1319,24 +1417,22 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, Wf
       }
     }
   }
-  if (!lp.gacc) acc_flush<kD ? 16u : 10u>(sacc, np, w.blk);
+  acc.flush(lp.seg_n, w.blk);
 }
 
 // Unoccluded next-event terms: light emission (Eq. 5), the vertex material
 // (Eq. 6 at this vertex) and the carry of the earlier vertices.  A launch
 // over one scene skips reading the slot's state word for its scene.
-template <bool kD>
+template <bool kD, bool kW>
 __global__ void __launch_bounds__(kWfThreads) wf_adj_connect(const WfScene* tab, WfParams lp, WfDev w) {
-  extern __shared__ float sacc_sh[];
-  float* sacc = lp.gacc ? lp.gacc : sacc_sh;
-  const uint32_t np = (kD ? 16u : 10u) * lp.seg_n;
-  if (!lp.gacc) acc_zero(sacc, acc_shared_floats(kD ? 16u : 10u, lp.seg_n));
+  constexpr uint32_t P = kD ? 16u : 10u;
+  IPT_ACCUM(P, kW, acc);
   const uint32_t n = w.cnt[2];
   const uint32_t lane = threadIdx.x & 31u;
   for (uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x - lane; i0 < n; i0 += gridDim.x * blockDim.x) {
     const uint32_t i = i0 + lane;
     const bool vis = i < n && w.sh_vis[i];
-    int lbase = -1, mbase = -1;  // accumulators of the light's emission and the vertex material
+    int lrow = -1, mrow = -1;  // accumulator rows of the light's emission and the vertex material
     float3 ge3 = f3(0.f, 0.f, 0.f);
     if constexpr (kD) {
       float g[kDisneyMat];
@@ -1345,52 +1441,50 @@ __global__ void __launch_bounds__(kWfThreads) wf_adj_connect(const WfScene* tab,
         const uint4 m = w.sh_meta[i];
         const WfScene& e = tab[lp.n_scenes == 1 ? 0u : state_scene(__float_as_uint(w.beta[m.x].w))];
         const float4 ge = w.sh_ge[i], cn = w.sh_n[i];
-        lbase = acc_ix16(e, lp, (int)m.w, kDisneyMat);
+        lrow = acc_row(e, lp, (int)m.w);
         ge3 = xyz(ge);
         const float4* dv = w.sh_dv + 4 * (size_t)i;
         const float4 d0 = dv[0], d1 = dv[1], d2 = dv[2], d3 = dv[3];
         const float gg[kDisneyMat] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w, d2.x, d2.y, d2.z, d2.w, d3.x};
         for (int j = 0; j < kDisneyMat; ++j) g[j] = gg[j];
-        mbase = acc_ix16(e, lp, (int)m.z, 0);
+        mrow = acc_row(e, lp, (int)m.z);
         add_to_carry<4>(w, m.x, w.nv[m.x], xyz(cn));
       }
-      warp_scatter3(sacc, lbase, ge3);
-      warp_scatter<kDisneyMat>(sacc, mbase, g);
-      continue;
+      acc.emission(lrow, ge3);
+      acc.material(mrow, g);
+    } else {
+      float g[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      if (vis) {
+        const uint4 m = w.sh_meta[i];
+        const WfScene& e = tab[lp.n_scenes == 1 ? 0u : state_scene(__float_as_uint(w.beta[m.x].w))];
+        const float4 ge = w.sh_ge[i], gm = w.sh_gm[i], cn = w.sh_n[i];
+        lrow = acc_row(e, lp, (int)m.w);
+        ge3 = xyz(ge);
+        const float3 q = xyz(gm);
+        const float4 mb = __ldg(&e.t.mat_b[m.z]);
+        g[0] = q.x * (1.0f / kPi);
+        g[1] = q.y * (1.0f / kPi);
+        g[2] = q.z * (1.0f / kPi);
+        g[3] = q.x * gm.w;
+        g[4] = q.y * gm.w;
+        g[5] = q.z * gm.w;
+        g[6] = dot(q, f3(mb.x, mb.y, mb.z)) * cn.w;
+        mrow = acc_row(e, lp, (int)m.z);
+        add_to_carry<4>(w, m.x, w.nv[m.x], xyz(cn));
+      }
+      acc.emission(lrow, ge3);
+      acc.material(mrow, g);
     }
-    float g[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (vis) {
-      const uint4 m = w.sh_meta[i];
-      const WfScene& e = tab[lp.n_scenes == 1 ? 0u : state_scene(__float_as_uint(w.beta[m.x].w))];
-      const float4 ge = w.sh_ge[i], gm = w.sh_gm[i], cn = w.sh_n[i];
-      lbase = acc_ix(e, lp, (int)m.w, 7);
-      ge3 = xyz(ge);
-      const float3 q = xyz(gm);
-      const float4 mb = __ldg(&e.t.mat_b[m.z]);
-      g[0] = q.x * (1.0f / kPi);
-      g[1] = q.y * (1.0f / kPi);
-      g[2] = q.z * (1.0f / kPi);
-      g[3] = q.x * gm.w;
-      g[4] = q.y * gm.w;
-      g[5] = q.z * gm.w;
-      g[6] = dot(q, f3(mb.x, mb.y, mb.z)) * cn.w;
-      mbase = acc_ix(e, lp, (int)m.z, 0);
-      add_to_carry<4>(w, m.x, w.nv[m.x], xyz(cn));
-    }
-    warp_scatter3(sacc, lbase, ge3);
-    warp_scatter<7>(sacc, mbase, g);
   }
-  if (!lp.gacc) acc_flush<kD ? 16u : 10u>(sacc, np, w.blk);
+  acc.flush(lp.seg_n, w.blk);
 }
 
 // Stage B: BRDF sampling; the new vertex joins the carry.
-template <bool kD>
+template <bool kD, bool kW>
 __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_b(const WfScene* tab, WfParams lp, uint32_t p0, WfDev w,
                                                        int cur) {
-  extern __shared__ float sacc_sh[];
-  float* sacc = lp.gacc ? lp.gacc : sacc_sh;
-  const uint32_t np = (kD ? 16u : 10u) * lp.seg_n;
-  if (!lp.gacc) acc_zero(sacc, acc_shared_floats(kD ? 16u : 10u, lp.seg_n));
+  constexpr uint32_t P = kD ? 16u : 10u;
+  IPT_ACCUM(P, kW, acc);
   if (blockIdx.x == 0 && threadIdx.x == 0) w.cnt[3] = 0;
   const uint32_t n = w.cnt[cur];
   const uint32_t si = set_iter(lp);
@@ -1484,7 +1578,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_b(const WfScene* tab, Wf
         w.beta[slot] = make_float4(bt.x, bt.y, bt.z, __uint_as_float(st | kDead));
       }
     }
-    finish_path<kD>(w, &e, lp, slot, nv, gfin, sacc, finish);
+    finish_path<kD>(w, &e, lp, slot, nv, gfin, acc, finish);
     const uint32_t ci = enqueue(nout, cont);
     if (cont) {
       qout[ci] = slot;
@@ -1494,17 +1588,15 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_b(const WfScene* tab, Wf
       w.beta[slot] = make_float4(beta.x, beta.y, beta.z, __uint_as_float(pack_state(k + 1, b)));
     }
   }
-  if (!lp.gacc) acc_flush<kD ? 16u : 10u>(sacc, np, w.blk);
+  acc.flush(lp.seg_n, w.blk);
 }
 
 // Paths closed by the cache: its prediction joins the earlier vertices'
 // carry (Eq. 6 through their BSDF factors), its parameter derivative goes to
 // the terminal segment's kd, ks and roughness, and the path finishes.
+template <bool kW>
 __global__ void __launch_bounds__(kWfThreads) wf_adj_cache(const WfScene* tab, WfParams lp, uint32_t p0, WfDev w) {
-  extern __shared__ float sacc_sh[];
-  float* sacc = lp.gacc ? lp.gacc : sacc_sh;
-  const uint32_t np = 10u * lp.seg_n;
-  if (!lp.gacc) acc_zero(sacc, acc_shared_floats(10u, lp.seg_n));
+  IPT_ACCUM(10u, kW, acc);
   const uint32_t n = lp.cb.counts[0];
   const float inv_spp = 1.0f / (float)lp.spp;
   const uint32_t lane = threadIdx.x & 31u;
@@ -1516,7 +1608,7 @@ __global__ void __launch_bounds__(kWfThreads) wf_adj_cache(const WfScene* tab, W
     const uint32_t nv = act ? w.nv[slot] : 0u;
     const WfScene& e = tab[lp.n_scenes == 1 ? 0u : state_scene(st)];
     float g[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int base = -1;
+    int row = -1;
     float3 gp = f3(0.f, 0.f, 0.f);
     if (act) {
       const int seg = __float_as_int(lp.cb.q.x[q].w);
@@ -1524,16 +1616,16 @@ __global__ void __launch_bounds__(kWfThreads) wf_adj_cache(const WfScene* tab, W
       const float* dp = lp.cb.qdp + 8 * (size_t)q;
 #pragma unroll
       for (int j = 0; j < 7; ++j) g[j] = dp[j];
-      base = acc_ix(e, lp, seg, 0);
+      row = acc_row(e, lp, seg);
       uint32_t pid, smp, ent;
       slot_pixel(e, p0, slot, lp.spp, lp.stride, pid, smp, ent);
       gp = pixel_grad(e, ent, inv_spp);
     }
-    warp_scatter<7>(sacc, base, g);
-    finish_path<false>(w, &e, lp, slot, nv, gp, sacc, act);
+    acc.material(row, g);
+    finish_path<false>(w, &e, lp, slot, nv, gp, acc, act);
     if (act) w.beta[slot].w = __uint_as_float(st | kDead);
   }
-  if (!lp.gacc) acc_flush<10u>(sacc, np, w.blk);
+  acc.flush(lp.seg_n, w.blk);
 }
 
 // grad_acc[i] += sum over block rows (FP64), for the chunk's parameters.
@@ -1556,6 +1648,16 @@ __global__ void __launch_bounds__(32 * kReduceWarps) wf_blk_reduce(const float* 
     double t = 0.0;
     for (int k = 0; k < kReduceWarps; ++k) t += part[k][lane];
     grad_acc[i] += t;
+  }
+}
+
+// grad_acc[P s + j] += value j of row s of the padded global accumulators.
+template <uint32_t P>
+__global__ void wf_wide_reduce(const float* gacc, uint32_t np, double* grad_acc) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < np; i += gridDim.x * blockDim.x) {
+    const uint32_t j = i % P;
+    const uint32_t at = P == 10u ? (j < 3u ? j : (j < 6u ? j + 1u : (j == 6u ? 3u : j + 1u))) : j;
+    grad_acc[i] += (double)gacc[(size_t)wide_stride(P) * (i / P) + at];
   }
 }
 
@@ -1921,10 +2023,10 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
   if (max_np > wb.blk_params) return cudaErrorInvalidValue;
   const size_t shmem = max_shared * sizeof(float);
   if (shmem > 48 * 1024) {
-    cudaFuncSetAttribute(wf_adj_a<kD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
-    cudaFuncSetAttribute(wf_adj_connect<kD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
-    cudaFuncSetAttribute(wf_adj_b<kD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
-    cudaFuncSetAttribute(wf_adj_cache, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
+    cudaFuncSetAttribute(wf_adj_a<kD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
+    cudaFuncSetAttribute(wf_adj_connect<kD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
+    cudaFuncSetAttribute(wf_adj_b<kD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
+    cudaFuncSetAttribute(wf_adj_cache<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
   }
   for (const WfChunk& c : chunks) {
     lp.seg_lo = c.seg_lo;
@@ -1934,14 +2036,19 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
     const bool global = c.seg_n > max_seg;
     lp.gacc = global ? wb.blk : nullptr;
     const size_t sm = global ? 0 : acc_shared_floats(P, c.seg_n) * sizeof(float);
+    const auto k_a = global ? wf_adj_a<kD, true> : wf_adj_a<kD, false>;
+    const auto k_c = global ? wf_adj_connect<kD, true> : wf_adj_connect<kD, false>;
+    const auto k_b = global ? wf_adj_b<kD, true> : wf_adj_b<kD, false>;
+    const auto k_q = global ? wf_adj_cache<true> : wf_adj_cache<false>;
     // each adjoint stage runs one wave at its own occupancy for this
     // accumulator size; block b of every stage adds into gradient row b
-    // (all blocks into row 0 in global mode)
-    const int g_a = one_wave(L, wf_adj_a<kD>, sm), g_c = one_wave(L, wf_adj_connect<kD>, sm);
-    const int g_b = one_wave(L, wf_adj_b<kD>, sm), g_q = one_wave(L, wf_adj_cache, sm);
+    // (all blocks into the padded global array in global mode)
+    const int g_a = one_wave(L, k_a, sm), g_c = one_wave(L, k_c, sm);
+    const int g_b = one_wave(L, k_b, sm), g_q = one_wave(L, k_q, sm);
     const int rows = global ? 1 : std::max(std::max(g_a, g_c), std::max(g_b, g_q));
     if (rows > wf_max_blocks(L)) return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(wb.blk, 0, (size_t)rows * np * sizeof(float), st);
+    cudaError_t e = cudaMemsetAsync(
+        wb.blk, 0, (global ? (size_t)wide_stride(P) * c.seg_n : (size_t)rows * np) * sizeof(float), st);
     if (e != cudaSuccess) return e;
     const uint32_t slots = c.n_pix * tp.spp;
     {
@@ -1961,7 +2068,7 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
       }
       {
         IPT_STAGE(11);
-        wf_adj_a<kD><<<g_a, kWfThreads, sm, st>>>(tab_dev, lp, c.p0, w, cur);
+        k_a<<<g_a, kWfThreads, sm, st>>>(tab_dev, lp, c.p0, w, cur);
       }
       if (k < last_k) {
         if (tp.nee) {
@@ -1970,10 +2077,10 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
             launch_trace<2>(width, grid, tab_dev, tab, w, cur, L.wf_steps, err, st);
           }
           IPT_STAGE(12);
-          wf_adj_connect<kD><<<g_c, kWfThreads, sm, st>>>(tab_dev, lp, w);
+          k_c<<<g_c, kWfThreads, sm, st>>>(tab_dev, lp, w);
         }
         IPT_STAGE(13);
-        wf_adj_b<kD><<<g_b, kWfThreads, sm, st>>>(tab_dev, lp, c.p0, w, cur);
+        k_b<<<g_b, kWfThreads, sm, st>>>(tab_dev, lp, c.p0, w, cur);
       }
       cur ^= 1;
     }
@@ -1988,10 +2095,13 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
         if (e != cudaSuccess) return e;
       }
       IPT_STAGE(13);
-      wf_adj_cache<<<g_q, kWfThreads, sm, st>>>(tab_dev, lp, c.p0, w);
+      k_q<<<g_q, kWfThreads, sm, st>>>(tab_dev, lp, c.p0, w);
     }
     IPT_STAGE(14);
-    wf_blk_reduce<<<(np + 31) / 32, 32 * kReduceWarps, 0, st>>>(wb.blk, rows, np, grad_acc + P * c.seg_lo);
+    if (global)
+      wf_wide_reduce<P><<<std::min<uint32_t>((np + 255u) / 256u, 2048u), 256, 0, st>>>(wb.blk, np, grad_acc + P * c.seg_lo);
+    else
+      wf_blk_reduce<<<(np + 31) / 32, 32 * kReduceWarps, 0, st>>>(wb.blk, rows, np, grad_acc + P * c.seg_lo);
   }
   return cudaGetLastError();
 }
@@ -2030,13 +2140,13 @@ cudaError_t wf_init(Launcher* L) {
   // gradient rows: the widest one-wave grid of an adjoint stage (accumulators
   // in dynamic shared memory only lower the occupancy)
   int rows = 0;
-  rows = std::max(rows, one_wave(*L, wf_adj_a<false>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_connect<false>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_b<false>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_a<true>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_connect<true>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_b<true>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_cache, 0));
+  rows = std::max(rows, one_wave(*L, wf_adj_a<false, false>, 0));
+  rows = std::max(rows, one_wave(*L, wf_adj_connect<false, false>, 0));
+  rows = std::max(rows, one_wave(*L, wf_adj_b<false, false>, 0));
+  rows = std::max(rows, one_wave(*L, wf_adj_a<true, false>, 0));
+  rows = std::max(rows, one_wave(*L, wf_adj_connect<true, false>, 0));
+  rows = std::max(rows, one_wave(*L, wf_adj_b<true, false>, 0));
+  rows = std::max(rows, one_wave(*L, wf_adj_cache<false>, 0));
   L->wf_max_rows = rows;
   return cudaSuccess;
 }
