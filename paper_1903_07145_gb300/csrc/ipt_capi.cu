@@ -574,8 +574,9 @@ ipt_status ipt_create(ipt_ctx** out, const ipt_options* opt) {
     ctx->stream = static_cast<cudaStream_t>(opt->stream);  // NULL: legacy default stream
   }
   if (e == cudaSuccess) e = ipt::init_launcher(&ctx->L, opt->device);
-  if (e == cudaSuccess) e = cudaMalloc(&ctx->err_dev, sizeof(uint32_t));
-  if (e == cudaSuccess) e = cudaMemset(ctx->err_dev, 0, sizeof(uint32_t));
+  // the error word, then the ray-casting kernel's two counters
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->err_dev, 3 * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMemset(ctx->err_dev, 0, 3 * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMallocHost(&ctx->loss_host, sizeof(double));
   if (e == cudaSuccess && (opt->flags & IPT_FLAG_COUNTERS)) {
     e = cudaMalloc(&ctx->counters_dev, 6 * sizeof(unsigned long long));
@@ -929,8 +930,8 @@ ipt_status ipt_trace_rays(ipt_ctx* ctx, int32_t scene, uint32_t n, const float* 
   if (n && (!orig || !dir || !tri_out)) return fail(ctx, IPT_ERR_INVALID_ARG, "null ray buffers");
   IPT_CK(cudaSetDevice(ctx->device));
   Timed tm(ctx, IPT_KERNEL_TRACE);
-  IPT_CK(ipt::launch_trace_rays(buffers(ctx, s), n, orig, dir, skip, tri_out, t_out, u_out, v_out, ctx->err_dev,
-                                ctx->stream));
+  const ipt::RayArrays rays{orig, dir, skip, tri_out, t_out, u_out, v_out, nullptr};
+  IPT_CK(ipt::launch_trace_rays(ctx->L, buffers(ctx, s), rays, n, ctx->err_dev + 1, ctx->err_dev, ctx->stream));
   return IPT_OK;
 }
 

@@ -236,10 +236,18 @@ cudaError_t launch_batch_losses(const double* rows, int n_rows, const BatchMembe
                                 uint32_t n_tab, double* loss, cudaStream_t st);
 cudaError_t launch_tick(uint32_t* counter, cudaStream_t st);
 
-cudaError_t launch_trace_rays(const SceneBuffers& s, uint32_t n, const float* orig,
-                              const float* dir, const int32_t* skip, int32_t* tri_out,
-                              float* t_out, float* u_out, float* v_out, uint32_t* err,
-                              cudaStream_t st);
+// Closest-hit rays given as arrays (see ipt_trace_rays); t, u, v may be null.
+struct RayArrays {
+  const float *orig, *dir;
+  const int32_t* skip;
+  int32_t* tri;
+  float *t, *u, *v;
+  const uint32_t* orig_to_internal;  // set by the launcher
+};
+
+// state: two device words, 0 before the first call (kept 0 between launches).
+cudaError_t launch_trace_rays(const Launcher& L, const SceneBuffers& s, const RayArrays& a, uint32_t n,
+                              uint32_t* state, uint32_t* err, cudaStream_t st);
 
 cudaError_t launch_philox(uint32_t n, const uint32_t* ctr, const uint32_t* key, uint32_t* out,
                           cudaStream_t st);

@@ -10,7 +10,7 @@
 //   k_finalize  loss and gradient reduction;
 //   k_adam      Adam + L1 emission regulariser + clamps (Sec. 4.4-4.5), then
 //               the tables for the next iteration;
-//   k_trace_rays, k_philox: the ray-casting and random-number primitives.
+//   k_philox    the random-number primitive (ray casting: ipt_wavefront.cu).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -712,22 +712,6 @@ static cudaError_t launch_tables_wide(const SceneBuffers& s, const SegBuffers& t
 }
 
 
-__global__ void k_trace_rays(SceneDev s, const uint32_t* orig_to_internal, uint32_t n, const float* orig,
-                             const float* dir, const int32_t* skip, int32_t* tri_out, float* t_out,
-                             float* u_out, float* v_out, uint32_t* err) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float3 o = f3(orig[3 * i], orig[3 * i + 1], orig[3 * i + 2]);
-  const float3 d = f3(dir[3 * i], dir[3 * i + 1], dir[3 * i + 2]);
-  int sk = -1;
-  if (skip && skip[i] >= 0 && (uint32_t)skip[i] < s.n_tri) sk = (int)orig_to_internal[skip[i]];
-  const Hit h = trace_closest(s, o, d, __int_as_float(0x7f800000), sk, err);
-  tri_out[i] = h.tri >= 0 ? tri_orig(s.tris, h.tri) : -1;
-  if (t_out) t_out[i] = h.t;
-  if (u_out) u_out[i] = h.u;
-  if (v_out) v_out[i] = h.v;
-}
-
 __global__ void k_philox(uint32_t n, const uint32_t* ctr, const uint32_t* key, uint32_t* out) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -943,17 +927,6 @@ cudaError_t launch_batch_losses(const double* rows, int n_rows, const BatchMembe
 
 cudaError_t launch_tick(uint32_t* counter, cudaStream_t st) {
   k_tick<<<1, 1, 0, st>>>(counter);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_trace_rays(const SceneBuffers& s, uint32_t n, const float* orig,
-                              const float* dir, const int32_t* skip, int32_t* tri_out,
-                              float* t_out, float* u_out, float* v_out, uint32_t* err,
-                              cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  const int block = 128;
-  k_trace_rays<<<(n + block - 1) / block, block, 0, st>>>(scene_dev(s), s.orig_to_internal, n, orig, dir, skip,
-                                                           tri_out, t_out, u_out, v_out, err);
   return cudaGetLastError();
 }
 

@@ -423,9 +423,10 @@ __device__ __forceinline__ uint2 st_pop(const Stack& S, Trav& T) {
 }
 
 template <int kWidth>
-__device__ __forceinline__ void trav_init(const WfScene& e, Trav& T, float3 o, float3 d, float tmax, int skip_a, int skip_b) {
+__device__ __forceinline__ void trav_init(const SceneDev& s, Trav& T, float3 o, float3 d, float tmax, int skip_a,
+                                          int skip_b) {
   T.r = ray_pre(o, d);
-  if constexpr (kWidth == kGrid4) T.g = grid_ray(e.s.grid_lo, e.s.grid_s, T.r);
+  if constexpr (kWidth == kGrid4) T.g = grid_ray(s.grid_lo, s.grid_s, T.r);
   T.oinv = f3(o.x * T.r.inv.x, o.y * T.r.inv.y, o.z * T.r.inv.z);
   T.tmax = tmax;
   T.skip_a = skip_a;
@@ -657,30 +658,83 @@ __device__ __forceinline__ bool node_step8(const SceneDev& s, Trav& T, const Sta
   return advance8(s, T, S);
 }
 
-// Stores a finished ray's result: the hit record (closest), the unoccluded
-// light contribution (forward shadow rays) or the visibility flag (adjoint
-// shadow rays).
-template <int kMode, bool kCount>
-__device__ __forceinline__ void trace_finish(const WfDev& w, const uint32_t* qsrc, uint32_t i, const Trav& T,
-                                             const SceneDev& sd) {
-  if constexpr (kCount) count_ray(sd, kMode != 0 ? 1 : 0, T.n_nodes, T.n_tests);
-  if (kMode == 0) {
-    const uint32_t slot = qsrc[i];
-    w.hit[slot] = make_float4(__int_as_float(T.best), T.bt, T.bu, T.bv);
-  } else if (kMode == 1) {
-    if (!T.occluded) {
-      const uint32_t slot = w.sh_meta[i].x;
-      const float4 c = w.sh_c[i];
-      float4 r = w.rad[slot];
-      r.x += c.x;
-      r.y += c.y;
-      r.z += c.z;
-      w.rad[slot] = r;
+// Rays of the wavefront: where they come from and where their results go.
+// kMode 0 takes queue `cur` (in the order of `order` when given), 1 and 2 the
+// shadow records.
+template <int kMode, int kWidth, bool kCount>
+struct QueueRays {
+  const WfScene* tab;
+  const WfDev& w;
+  const uint32_t* qsrc;
+  int one_scene;
+  SceneDev sd;
+
+  __device__ __forceinline__ const SceneDev& scene() const { return sd; }
+
+  __device__ __forceinline__ void load(uint32_t i, Trav& T) {
+    // a launch over one scene skips the lookup of the ray's scene
+    const uint32_t slot = kMode != 0 ? w.sh_meta[i].x : qsrc[i];
+    uint32_t b = 0;
+    if (!one_scene) {
+      b = state_scene(__float_as_uint(w.beta[slot].w));
+      sd = tab[b].s;
     }
-  } else {
-    w.sh_vis[i] = T.occluded ? 0u : 1u;
+    if (kMode != 0) {
+      const float4 o = w.sh_o[i], d = w.sh_d[i];
+      trav_init<kWidth>(tab[b].s, T, xyz(o), xyz(d), d.w, __float_as_int(o.w), (int)w.sh_meta[i].y);
+    } else {
+      const float4 o = w.ray_o[slot], d = w.ray_d[slot];
+      trav_init<kWidth>(tab[b].s, T, xyz(o), xyz(d), __int_as_float(0x7f800000), __float_as_int(o.w), -1);
+    }
   }
-}
+
+  // The hit record (closest), the unoccluded light contribution (forward
+  // shadow rays) or the visibility flag (adjoint shadow rays).
+  __device__ __forceinline__ void finish(uint32_t i, const Trav& T) const {
+    if constexpr (kCount) count_ray(sd, kMode != 0 ? 1 : 0, T.n_nodes, T.n_tests);
+    if (kMode == 0) {
+      const uint32_t slot = qsrc[i];
+      w.hit[slot] = make_float4(__int_as_float(T.best), T.bt, T.bu, T.bv);
+    } else if (kMode == 1) {
+      if (!T.occluded) {
+        const uint32_t slot = w.sh_meta[i].x;
+        const float4 c = w.sh_c[i];
+        float4 r = w.rad[slot];
+        r.x += c.x;
+        r.y += c.y;
+        r.z += c.z;
+        w.rad[slot] = r;
+      }
+    } else {
+      w.sh_vis[i] = T.occluded ? 0u : 1u;
+    }
+  }
+};
+
+// Rays given by the caller (ipt_trace_rays).
+template <int kWidth, bool kCount>
+struct ArrayRays {
+  const SceneDev& s;
+  const RayArrays& a;
+
+  __device__ __forceinline__ const SceneDev& scene() const { return s; }
+
+  __device__ __forceinline__ void load(uint32_t i, Trav& T) {
+    const float* o = a.orig + 3 * (size_t)i;
+    const float* d = a.dir + 3 * (size_t)i;
+    int sk = -1;
+    if (a.skip && a.skip[i] >= 0 && (uint32_t)a.skip[i] < s.n_tri) sk = (int)a.orig_to_internal[a.skip[i]];
+    trav_init<kWidth>(s, T, f3(o[0], o[1], o[2]), f3(d[0], d[1], d[2]), __int_as_float(0x7f800000), sk, -1);
+  }
+
+  __device__ __forceinline__ void finish(uint32_t i, const Trav& T) const {
+    if constexpr (kCount) count_ray(s, 0, T.n_nodes, T.n_tests);
+    a.tri[i] = T.best >= 0 ? tri_orig(s.tris, T.best) : -1;
+    if (a.t) a.t[i] = T.bt;
+    if (a.u) a.u[i] = T.bu;
+    if (a.v) a.v[i] = T.bv;
+  }
+};
 
 // Persistent traversal: each warp fetches rays for its idle lanes with one
 // atomic, then steps its lanes' traversals.
@@ -695,24 +749,19 @@ __device__ __forceinline__ void trace_finish(const WfDev& w, const uint32_t* qsr
 //    (with one or two lanes active).
 //  * Binary BVH: rounds of `steps` node visits, whole leaves at a time, and a
 //    refetch after each round.
-// Closest hit takes queue `cur`'s slots in the order of `order` when given
-// (the same slots reordered by bin), else in queue order.
+// kFew: a launch with no more rays than its grid has lanes.  Each warp takes
+// its rays by position (no fetch, no refill), and they are spread over all
+// warps: such a launch lasts as long as its slowest warp, and a warp takes
+// the steps of all its rays' phases.  A room's pixel batch of 64 (4096 rays a
+// launch, 11 launches a pass): closest hit 0.33 -> 0.24 ms, shadow rays 0.32
+// -> 0.23 ms; two rays a warp at least: 0.25 and 0.24, four: 0.25 and 0.25,
+// eight: 0.27 and 0.27, 32: 0.30 and 0.29.
 // kCount: counts node visits and triangle tests (a context with counters);
 // without it the two counters and their pointer stay out of the registers
 // (with the ray's permuted origin kept instead of selected per test: closest
 // hit 41.8 -> 39.8 ms, shadow rays 23.3 -> 22.1 ms on the 61k room).
-template <int kMode, int kWidth, bool kCount>
-__global__ void __launch_bounds__(kWfThreads, 8) wf_trace(const WfScene* tab, WfDev w, int cur, int steps,
-                                                       int one_scene, const uint32_t* order, uint32_t* err) {
-  constexpr bool kAny = kMode != 0;
-  if (!kAny && blockIdx.x == 0 && threadIdx.x == 0) {
-    w.cnt[cur ? 0 : 1] = 0;  // next queue, filled by the shading stage
-    w.cnt[2] = 0;            // shadow queue
-    w.cnt[4] = 0;            // shadow fetch counter
-  }
-  const uint32_t n = kAny ? w.cnt[2] : w.cnt[cur];
-  const uint32_t* qsrc = order ? order : queue(w, cur);
-  uint32_t* fetch = kAny ? &w.cnt[4] : &w.cnt[3];
+template <bool kAny, int kWidth, bool kFew, class Src>
+__device__ __forceinline__ void trace_loop(Src& src, uint32_t n, uint32_t* fetch, int steps, uint32_t* err) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t lt_mask = (1u << lane) - 1u;
   const int refill = min(max(steps, 1), 32);
@@ -720,48 +769,42 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_trace(const WfScene* tab, Wf
   uint2 deep[kStackSize - kShortStack];
   const Stack S{s_stack + threadIdx.x, deep};
   Trav T;
-  SceneDev sd = tab[0].s;
   constexpr uint32_t kNone = 0xffffffffu;
-  uint32_t item = kNone;  // the lane's queue entry
-  bool fin = false;      // wide BVHs: the lane's ray has ended, its result not yet stored
-  bool drained = false;  // warp-uniform: the queue has no rays left
+  uint32_t item = kNone;  // the lane's ray
+  bool fin = false;       // wide BVHs: the lane's ray has ended, its result not yet stored
+  bool drained = false;   // warp-uniform: no rays left to fetch
   for (;;) {
     if (fin) {  // results are stored at the refill, by all ended lanes together
-      trace_finish<kMode, kCount>(w, qsrc, item, T, sd);
+      src.finish(item, T);
       item = kNone;
       fin = false;
     }
     const bool need = item == kNone && !drained;
     const unsigned m = __ballot_sync(0xffffffffu, need);
     if (m) {
-      const int leader = __ffs(m) - 1;
-      uint32_t base = 0;
-      if ((int)lane == leader) base = atomicAdd(fetch, (uint32_t)__popc(m));
-      base = __shfl_sync(0xffffffffu, base, leader);
-      drained = base + (uint32_t)__popc(m) >= n;
-      const uint32_t i = base + (uint32_t)__popc(m & lt_mask);
+      uint32_t i;
+      if constexpr (kFew) {
+        const uint32_t warps = gridDim.x * (kWfThreads / 32u);
+        const uint32_t lanes = (n + warps - 1u) / warps;
+        i = lane < lanes ? (blockIdx.x * (kWfThreads / 32u) + (threadIdx.x >> 5)) * lanes + lane : n;
+        drained = true;
+      } else {
+        const int leader = __ffs(m) - 1;
+        uint32_t base = 0;
+        if ((int)lane == leader) base = atomicAdd(fetch, (uint32_t)__popc(m));
+        base = __shfl_sync(0xffffffffu, base, leader);
+        drained = base + (uint32_t)__popc(m) >= n;
+        i = base + (uint32_t)__popc(m & lt_mask);
+      }
       if (need && i < n) {
         item = i;
-        // a launch over one scene skips the lookup of the ray's scene
-        const uint32_t slot = kAny ? w.sh_meta[i].x : qsrc[i];
-        uint32_t b = 0;
-        if (!one_scene) {
-          b = state_scene(__float_as_uint(w.beta[slot].w));
-          sd = tab[b].s;
-        }
-        if (kAny) {
-          const float4 o = w.sh_o[i], d = w.sh_d[i];
-          trav_init<kWidth>(tab[b], T, xyz(o), xyz(d), d.w, __float_as_int(o.w), (int)w.sh_meta[i].y);
-        } else {
-          const float4 o = w.ray_o[slot], d = w.ray_d[slot];
-          trav_init<kWidth>(tab[b], T, xyz(o), xyz(d), __int_as_float(0x7f800000), __float_as_int(o.w), -1);
-        }
+        src.load(i, T);
       }
     }
     if (__all_sync(0xffffffffu, item == kNone)) break;
     if constexpr (kWidth == 2) {
-      if (item != kNone && trav_run2<kAny>(sd, T, S, steps, err)) {
-        trace_finish<kMode, kCount>(w, qsrc, item, T, sd);
+      if (item != kNone && trav_run2<kAny>(src.scene(), T, S, steps, err)) {
+        src.finish(item, T);
         item = kNone;
       }
     } else {
@@ -773,9 +816,44 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_trace(const WfScene* tab, Wf
         if (ml == 0u || (!drained && 32 - __popc(ml) >= refill)) break;
         const bool tri_phase = __popc(mt) >= __popc(ml & ~mt);
         if (live && at_tri == tri_phase)
-          fin = at_tri        ? tri_step<kAny, kWidth>(sd, T, S)
-                : kWidth == 8 ? node_step8<kAny>(sd, T, S, err)
-                              : node_step4<kAny, kWidth == kGrid4>(sd, T, S, err);
+          fin = at_tri        ? tri_step<kAny, kWidth>(src.scene(), T, S)
+                : kWidth == 8 ? node_step8<kAny>(src.scene(), T, S, err)
+                              : node_step4<kAny, kWidth == kGrid4>(src.scene(), T, S, err);
+      }
+    }
+  }
+}
+
+template <int kMode, int kWidth, bool kCount, bool kFew>
+__global__ void __launch_bounds__(kWfThreads, 8) wf_trace(const WfScene* tab, WfDev w, int cur, int steps,
+                                                       int one_scene, const uint32_t* order, uint32_t* err) {
+  constexpr bool kAny = kMode != 0;
+  if (!kAny && blockIdx.x == 0 && threadIdx.x == 0) {
+    w.cnt[cur ? 0 : 1] = 0;  // next queue, filled by the shading stage
+    w.cnt[2] = 0;            // shadow queue
+    w.cnt[4] = 0;            // shadow fetch counter
+  }
+  const uint32_t n = kAny ? w.cnt[2] : w.cnt[cur];
+  QueueRays<kMode, kWidth, kCount> src{tab, w, order ? order : queue(w, cur), one_scene, tab[0].s};
+  trace_loop<kAny, kWidth, kFew>(src, n, kAny ? &w.cnt[4] : &w.cnt[3], steps, err);
+}
+
+// Closest hits of rays given as arrays, by the same loops (one thread per ray
+// with whole leaves and its stack in local memory took 279 us for a million
+// random rays in the 61k room, 194 us here; 4099 rays 37.3 -> 31.5 us).
+// state: [0] rays fetched, [1] blocks done; both 0 before and after a launch.
+template <int kWidth, bool kCount, bool kFew>
+__global__ void __launch_bounds__(kWfThreads, 8) k_trace_rays(SceneDev s, RayArrays a, uint32_t n, int steps,
+                                                              uint32_t* state, uint32_t* err) {
+  ArrayRays<kWidth, kCount> src{s, a};
+  trace_loop<false, kWidth, kFew>(src, n, state, steps, err);
+  if constexpr (!kFew) {  // the last block clears the counters
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(&state[1], 1u) == gridDim.x - 1u) {
+        state[0] = 0u;
+        state[1] = 0u;
       }
     }
   }
@@ -1798,27 +1876,60 @@ static int table_width(const std::vector<WfScene>& tab) {
 // grid nodes serve closest hits only: shadow rays visit fewer nodes per ray
 // set-up and gained nothing (61k room 20.95 -> 20.7 ms, 516k room 30.9 -> 31.7
 // ms), where closest hit went 37.8 -> 35.7 and 56.2 -> 54.0 ms.
-template <int kMode, bool kCount>
+template <int kMode, bool kCount, bool kFew>
 static void launch_trace_w(int width, int grid, const WfScene* tab_dev, int one, const WfDev& w, int cur, int steps,
                            uint32_t* err, cudaStream_t st, const uint32_t* order) {
   if (width == 8)
-    wf_trace<kMode, 8, kCount><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
+    wf_trace<kMode, 8, kCount, kFew><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
   else if (kMode == 0 && width == kGrid4)
-    wf_trace<0, kGrid4, kCount><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
+    wf_trace<0, kGrid4, kCount, kFew><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
   else if (width == 4 || width == kGrid4)
-    wf_trace<kMode, 4, kCount><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
+    wf_trace<kMode, 4, kCount, kFew><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
   else
-    wf_trace<kMode, 2, kCount><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
+    wf_trace<kMode, 2, kCount, kFew><<<grid, kWfThreads, 0, st>>>(tab_dev, w, cur, steps, one, order, err);
 }
 
+// slots: path slots of the chunk, the most rays the launch can have.
 template <int kMode>
 static void launch_trace(int width, int grid, const WfScene* tab_dev, const std::vector<WfScene>& tab, const WfDev& w,
-                         int cur, int steps, uint32_t* err, cudaStream_t st, const uint32_t* order = nullptr) {
+                         int cur, uint32_t slots, int steps, uint32_t* err, cudaStream_t st,
+                         const uint32_t* order = nullptr) {
   const int one = tab.size() == 1 ? 1 : 0;
   if (tab[0].s.counters)  // a context's scenes all count, or none does
-    launch_trace_w<kMode, true>(width, grid, tab_dev, one, w, cur, steps, err, st, order);
+    launch_trace_w<kMode, true, false>(width, grid, tab_dev, one, w, cur, steps, err, st, order);
+  else if (slots <= (uint32_t)grid * kWfThreads)
+    launch_trace_w<kMode, false, true>(width, grid, tab_dev, one, w, cur, steps, err, st, order);
   else
-    launch_trace_w<kMode, false>(width, grid, tab_dev, one, w, cur, steps, err, st, order);
+    launch_trace_w<kMode, false, false>(width, grid, tab_dev, one, w, cur, steps, err, st, order);
+}
+
+template <bool kCount, bool kFew>
+static void launch_rays_w(int grid, const SceneDev& s, const RayArrays& a, uint32_t n, int steps, uint32_t* state,
+                          uint32_t* err, cudaStream_t st) {
+  switch (s.wide) {
+    case 0: k_trace_rays<2, kCount, kFew><<<grid, kWfThreads, 0, st>>>(s, a, n, steps, state, err); break;
+    case 2: k_trace_rays<8, kCount, kFew><<<grid, kWfThreads, 0, st>>>(s, a, n, steps, state, err); break;
+    case 3: k_trace_rays<kGrid4, kCount, kFew><<<grid, kWfThreads, 0, st>>>(s, a, n, steps, state, err); break;
+    default: k_trace_rays<4, kCount, kFew><<<grid, kWfThreads, 0, st>>>(s, a, n, steps, state, err);
+  }
+}
+
+cudaError_t launch_trace_rays(const Launcher& L, const SceneBuffers& s, const RayArrays& a, uint32_t n,
+                              uint32_t* state, uint32_t* err, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  const int most = wf_grid(L);
+  RayArrays r = a;
+  r.orig_to_internal = s.orig_to_internal;
+  const SceneDev sd = scene_dev(s);
+  if (s.counters) {
+    launch_rays_w<true, false>(most, sd, r, n, L.wf_steps, state, err, st);
+  } else if (n <= (uint32_t)most * kWfThreads) {
+    const int grid = (int)std::min<uint32_t>((n + kWfThreads / 32u - 1u) / (kWfThreads / 32u), (uint32_t)most);
+    launch_rays_w<false, true>(grid, sd, r, n, L.wf_steps, state, err, st);
+  } else {
+    launch_rays_w<false, false>(most, sd, r, n, L.wf_steps, state, err, st);
+  }
+  return cudaGetLastError();
 }
 
 // Secondary closest-hit rays are reordered when the launcher asks for it:
@@ -1938,7 +2049,7 @@ cudaError_t wf_forward(const Launcher& L, const WfScene* tab_dev, const std::vec
       }
       {
         IPT_STAGE(8);
-        launch_trace<0>(width, grid, tab_dev, tab, w, cur, L.wf_steps, err, st, order);
+        launch_trace<0>(width, grid, tab_dev, tab, w, cur, slots, L.wf_steps, err, st, order);
       }
       {
         IPT_STAGE(10);
@@ -1949,7 +2060,7 @@ cudaError_t wf_forward(const Launcher& L, const WfScene* tab_dev, const std::vec
       }
       if (k < last_k && k < tp.max_depth && tp.nee && !(record && k < lp.cache_k)) {
         IPT_STAGE(9);
-        launch_trace<1>(width, grid, tab_dev, tab, w, cur, L.wf_steps, err, st);
+        launch_trace<1>(width, grid, tab_dev, tab, w, cur, slots, L.wf_steps, err, st);
       }
       cur ^= 1;
     }
@@ -2064,7 +2175,7 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
       }
       {
         IPT_STAGE(8);
-        launch_trace<0>(width, grid, tab_dev, tab, w, cur, L.wf_steps, err, st, order);
+        launch_trace<0>(width, grid, tab_dev, tab, w, cur, slots, L.wf_steps, err, st, order);
       }
       {
         IPT_STAGE(11);
@@ -2074,7 +2185,7 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
         if (tp.nee) {
           {
             IPT_STAGE(9);
-            launch_trace<2>(width, grid, tab_dev, tab, w, cur, L.wf_steps, err, st);
+            launch_trace<2>(width, grid, tab_dev, tab, w, cur, slots, L.wf_steps, err, st);
           }
           IPT_STAGE(12);
           k_c<<<g_c, kWfThreads, sm, st>>>(tab_dev, lp, w);
@@ -2121,14 +2232,21 @@ cudaError_t wf_init(Launcher* L) {
   // width's persistent grid fits in one wave
   int b = 1 << 30;
   const void* variants[] = {
-      (const void*)wf_trace<0, 2, false>, (const void*)wf_trace<1, 2, false>, (const void*)wf_trace<2, 2, false>,
-      (const void*)wf_trace<0, 4, false>, (const void*)wf_trace<1, 4, false>, (const void*)wf_trace<2, 4, false>,
-      (const void*)wf_trace<0, kGrid4, false>,
-      (const void*)wf_trace<0, 8, false>, (const void*)wf_trace<1, 8, false>, (const void*)wf_trace<2, 8, false>,
-      (const void*)wf_trace<0, 2, true>, (const void*)wf_trace<1, 2, true>, (const void*)wf_trace<2, 2, true>,
-      (const void*)wf_trace<0, 4, true>, (const void*)wf_trace<1, 4, true>, (const void*)wf_trace<2, 4, true>,
-      (const void*)wf_trace<0, kGrid4, true>,
-      (const void*)wf_trace<0, 8, true>, (const void*)wf_trace<1, 8, true>, (const void*)wf_trace<2, 8, true>};
+      (const void*)wf_trace<0, 2, false, false>, (const void*)wf_trace<1, 2, false, false>,
+      (const void*)wf_trace<2, 2, false, false>, (const void*)wf_trace<0, 4, false, false>,
+      (const void*)wf_trace<1, 4, false, false>, (const void*)wf_trace<2, 4, false, false>,
+      (const void*)wf_trace<0, kGrid4, false, false>, (const void*)wf_trace<0, 8, false, false>,
+      (const void*)wf_trace<1, 8, false, false>, (const void*)wf_trace<2, 8, false, false>,
+      (const void*)wf_trace<0, 2, false, true>, (const void*)wf_trace<1, 2, false, true>,
+      (const void*)wf_trace<2, 2, false, true>, (const void*)wf_trace<0, 4, false, true>,
+      (const void*)wf_trace<1, 4, false, true>, (const void*)wf_trace<2, 4, false, true>,
+      (const void*)wf_trace<0, kGrid4, false, true>, (const void*)wf_trace<0, 8, false, true>,
+      (const void*)wf_trace<1, 8, false, true>, (const void*)wf_trace<2, 8, false, true>,
+      (const void*)wf_trace<0, 2, true, false>, (const void*)wf_trace<1, 2, true, false>,
+      (const void*)wf_trace<2, 2, true, false>, (const void*)wf_trace<0, 4, true, false>,
+      (const void*)wf_trace<1, 4, true, false>, (const void*)wf_trace<2, 4, true, false>,
+      (const void*)wf_trace<0, kGrid4, true, false>, (const void*)wf_trace<0, 8, true, false>,
+      (const void*)wf_trace<1, 8, true, false>, (const void*)wf_trace<2, 8, true, false>};
   for (const void* k : variants) {
     int bk = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bk, k, kWfThreads, 0);

@@ -77,3 +77,23 @@ def test_bvh_forms_give_the_same_hits(name):
         hit = ref[0][ref[0] >= 0].numpy()
         assert (hit < 600).all()
     tr.close()
+
+
+@pytest.mark.parametrize("n", [1, 31, 4863, 4865, 155647, 155649, 400001])
+def test_ray_counts_around_the_launch_forms(n):
+    """A launch with at most as many rays as lanes spreads them over its warps,
+    a larger one refills: the same hits for a ray wherever it stands, with and
+    without skipped triangles, and twice in a row (the counters are cleared)."""
+    sc = scenes.indoor_room(3, n_cuboids=6, cuboid_sub=4, room_sub=4, n_lights=2, n_views=1, width=8, height=8)
+    tr = Tracer(sc, seed=1)
+    o, d = scenes.random_rays(sc, 997, 4)
+    skip = np.random.default_rng(5).integers(-1, sc.n_tri, 997).astype(np.int32)
+    pick = torch.from_numpy(np.random.default_rng(n).integers(0, 997, n))
+    o, d, skip = (torch.from_numpy(a) for a in (o, d, skip))
+    for sk in (None, skip):
+        ref = [v.cpu() for v in tr.trace_rays(o, d, sk)]
+        for _ in range(2):
+            got = [v.cpu() for v in tr.trace_rays(o[pick], d[pick], None if sk is None else sk[pick])]
+            for a, b in zip(ref, got):
+                assert torch.equal(a[pick], b)
+    tr.close()
