@@ -244,6 +244,40 @@ ipt_status ensure_wf(ipt_ctx* ctx, bool adjoint, uint32_t n_params, bool disney,
   return IPT_OK;
 }
 
+// Grows the radiance buffer of the megakernel's residual pass to n samples.
+// It stays as it is when n is above its limit or memory is short: the pass
+// then takes the form that needs none.
+void ensure_rad(ipt_ctx* ctx, uint64_t n) {
+  if (n <= ctx->L.rad_cap || n > ipt::kFewSamples) return;
+  uint32_t want = 1u << 16;
+  while (want < n) want *= 2;
+  if (ctx->L.rad) {
+    if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return;
+    cudaFree(ctx->L.rad);
+    ++ctx->alloc_gen;
+  }
+  ctx->L.rad = nullptr;
+  ctx->L.rad_cap = 0;
+  if (cudaMalloc(&ctx->L.rad, sizeof(float4) * want) == cudaSuccess)
+    ctx->L.rad_cap = want;
+  else
+    cudaGetLastError();
+}
+
+// The launcher of a residual pass of n samples.  A pass that the caller
+// captures gets no radiance buffer: its graph may outlive the buffer.
+static ipt::Launcher forward_launcher(ipt_ctx* ctx, uint64_t n) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const bool eager = cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  if (eager)
+    ensure_rad(ctx, n);
+  else
+    cudaGetLastError();
+  ipt::Launcher L = ctx->L;
+  if (!eager) L.rad_cap = 0;
+  return L;
+}
+
 bool use_wavefront_cap(const ipt_ctx* ctx, uint32_t spp) {
   const uint32_t cap = ctx->cfg.wavefront_slots ? ctx->cfg.wavefront_slots : (1u << 20);
   return spp <= cap;
@@ -329,8 +363,9 @@ ipt_status run_forward(ipt_ctx* ctx, int32_t scene_id, DeviceScene* s, uint32_t 
     }
     ipt::TraceParams tpk = tp;
     tpk.pick = pick;
+    const ipt::Launcher L = forward_launcher(ctx, (uint64_t)n * tp.spp);
     Timed tm(ctx, IPT_KERNEL_FORWARD);
-    IPT_CK(ipt::launch_forward(ctx->L, buffers(ctx, s), s->tab, s->views_dev, (uint32_t)s->views.size(), begin, n,
+    IPT_CK(ipt::launch_forward(L, buffers(ctx, s), s->tab, s->views_dev, (uint32_t)s->views.size(), begin, n,
                                tpk, img, msq, target, g_out, partials, g_scale, loss_kind, ctx->err_dev,
                                ctx->stream));
   }
@@ -610,6 +645,7 @@ ipt_status ipt_destroy(ipt_ctx* ctx) {
   for (cudaEvent_t e : ctx->spare_events) cudaEventDestroy(e);
   if (ctx->counters_dev) cudaFree(ctx->counters_dev);
   if (ctx->err_dev) cudaFree(ctx->err_dev);
+  if (ctx->L.rad) cudaFree(ctx->L.rad);
   if (ctx->loss_host) cudaFreeHost(ctx->loss_host);
   if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
   delete ctx;

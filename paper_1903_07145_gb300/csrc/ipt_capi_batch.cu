@@ -215,6 +215,8 @@ ipt_status ipt_batch_step(ipt_ctx* ctx, int32_t batch, const ipt_trace_opts* opt
     batch_table(ctx, b, opts->pixel_batch);
     IPT_CK(cudaMemcpyAsync(b->mem_dev, b->mem_host.data(), b->mem_host.size() * sizeof(ipt::BatchMember),
                            cudaMemcpyHostToDevice, ctx->stream));
+    if (ctx->cfg.integrator == 0)
+      ensure_rad(ctx, (uint64_t)(b->tab_host.back().pix_begin + b->tab_host.back().n_pix) * opts->spp_r);
     uint32_t max_seg = 0;
     for (const ipt::WfChunk& c : ipt::wf_plan(b->tab_host, cap, opts->spp_d, ipt::wf_max_segments()))
       max_seg = std::max(max_seg, c.seg_n);

@@ -238,6 +238,7 @@ void wf_release(ipt_ctx* c);
 // the S x 10 (or S x 16) parameters of its widest chunk.  Capacities only
 // grow.
 ipt_status ensure_wf(ipt_ctx* ctx, bool adjoint, uint32_t n_params, bool disney = false, uint32_t depth = 0);
+void ensure_rad(ipt_ctx* ctx, uint64_t n);
 bool use_wavefront_cap(const ipt_ctx* ctx, uint32_t spp);
 bool use_wavefront(const ipt_ctx* ctx, uint32_t spp);
 ipt::WfScene wf_entry(const ipt_ctx* ctx, int32_t scene_id, const DeviceScene* s, uint32_t pix_base, uint32_t n);

@@ -131,10 +131,13 @@ struct Launcher {
   int fwd_blocks_per_sm = 0;
   int adj_blocks_per_sm[4] = {0, 0, 0, 0};
   int wf_blocks_per_sm = 0;  // traversal kernels
+  int wf_occ = 0, wf_row_occ = 0;  // by occupancy: traversal kernels (the fewest), adjoint stages (the most)
   int wf_fixed_blocks = 0;   // configured blocks per SM for every wavefront kernel (0: by occupancy)
   int wf_max_rows = 0;       // gradient rows any adjoint stage may use (blocks of its widest grid)
   int wf_steps = 16;  // refill point of the persistent traversal (idle lanes; binary BVH: steps)
   int sort_cells = 0; // secondary closest-hit rays reordered by origin cell (cells per axis; 0: off)
+  float4* rad = nullptr;  // radiances of the megakernel's samples
+  uint32_t rad_cap = 0;   //   and how many it holds (at most kFewSamples)
   int sort_dirs = 0;  //   and direction (divisions of each cube-map face side; 0: none)
 };
 
@@ -170,6 +173,10 @@ constexpr int kMaxForwardDepth = 64;
 constexpr int kBlockThreads = 128;
 
 int loss_partials_capacity(const Launcher& L);
+// Most samples of a megakernel residual pass that runs one sample a thread
+// (their radiances, 16 bytes each, go through Launcher::rad, grown on demand;
+// a launch that it cannot hold keeps a pixel's samples in one warp).
+constexpr uint32_t kFewSamples = 1u << 20;
 
 cudaError_t launch_prepare(const SceneBuffers& s, const SegBuffers& t, const float* params,
                            const float* sparams, cudaStream_t st);

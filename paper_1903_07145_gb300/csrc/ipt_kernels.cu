@@ -28,51 +28,72 @@ __global__ void k_prepare(const float* params, const float* sparams, uint32_t S,
   build_tables(params, sparams, S, es, seg_area, t);
 }
 
-// Radiance estimate of one camera path.
-__device__ float3 forward_path(const SceneDev& s, const SegDev& t, const ViewDev& vw, uint32_t px, uint32_t py,
-                               uint32_t pid, uint32_t sample, const PathParams& pp, bool light,
-                               uint32_t* err) {
+// A camera path of the forward pass between two vertices.
+struct FwdPath {
   PathRng rng;
-  rng.base = make_uint4(pid, sample, pp.set_iter, 0);
-  rng.key = pp.key;
-  float3 o;
-  float3 d = camera_ray(vw, px, py, rng, o);
-  float3 beta = f3(1.0f, 1.0f, 1.0f), L = f3(0.0f, 0.0f, 0.0f);
-  const bool light_on = pp.nee && light;
-  int skip = -1;
-  float prev_pdf = 0.0f;
-  for (uint32_t k = 0;; ++k) {
-    const Hit h = trace_closest(s, o, d, __int_as_float(0x7f800000), skip, err);
-    if (h.tri < 0) break;
-    const Vtx v = make_vertex(s, h, d, pp.profile);
-    if (v.prof > 0.0f) {
-      const float wb = emission_weight(t, v, h.t, k > 0, light_on, prev_pdf, pp.mis);
-      if (wb > 0.0f) L = L + beta * xyz(__ldg(&t.emis[v.seg])) * (wb * v.prof);
-    }
-    if (k == pp.max_depth) break;
-    const float4 ua = rng.draw(k, 0), ub = rng.draw(k, 1);
-    const float4 ma = __ldg(&t.mat_a[v.seg]), mb = __ldg(&t.mat_b[v.seg]);
-    const float4 sa = __ldg(&t.samp[v.seg]);
-    if (light_on) {
-      const NeeResult ne = next_event(s, t, v, ua, ub, pp.profile, pp.mis, sa.y, sa.x, err);
-      if (ne.valid) {
-        const BrdfVal bv = brdf_eval(ma, mb, v.ns, v.wi, ne.wl);
-        L = L + beta * bv.f * xyz(__ldg(&t.emis[ne.seg])) * ne.k;
-      }
-    }
-    if (!(dot(v.wi, v.ns) > 0.0f)) break;
-    const float3 wo = bsdf_sample(sa.w, sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
-    const float pdf = bsdf_pdf(sa.y, sa.x, v.ns, v.wi, wo);
-    const float co = dot(wo, v.ns);
-    if (!(dot(wo, v.ng) > 0.0f) || !(co > 0.0f) || !(pdf > 0.0f)) break;
-    const BrdfVal bv = brdf_eval(ma, mb, v.ns, v.wi, wo);
-    beta = beta * bv.f * (co / pdf);
-    prev_pdf = pdf;
-    o = v.x + v.ng * s.eps;
-    d = wo;
-    skip = h.tri;
+  float3 o, d, beta, L;
+  float prev_pdf;
+  int skip;
+  uint32_t k;
+};
+
+__device__ __forceinline__ void forward_start(FwdPath& p, const ViewDev& vw, uint32_t px, uint32_t py, uint32_t pid,
+                                              uint32_t sample, const PathParams& pp) {
+  p.rng.base = make_uint4(pid, sample, pp.set_iter, 0);
+  p.rng.key = pp.key;
+  p.d = camera_ray(vw, px, py, p.rng, p.o);
+  p.beta = f3(1.0f, 1.0f, 1.0f);
+  p.L = f3(0.0f, 0.0f, 0.0f);
+  p.prev_pdf = 0.0f;
+  p.skip = -1;
+  p.k = 0;
+}
+
+// Traces to the next vertex and shades it; false when the path ends there.
+__device__ __forceinline__ bool forward_vertex(const SceneDev& s, const SegDev& t, const PathParams& pp, bool light_on,
+                                               FwdPath& p, uint32_t* err) {
+  const Hit h = trace_closest(s, p.o, p.d, __int_as_float(0x7f800000), p.skip, err);
+  if (h.tri < 0) return false;
+  const Vtx v = make_vertex(s, h, p.d, pp.profile);
+  if (v.prof > 0.0f) {
+    const float wb = emission_weight(t, v, h.t, p.k > 0, light_on, p.prev_pdf, pp.mis);
+    if (wb > 0.0f) p.L = p.L + p.beta * xyz(__ldg(&t.emis[v.seg])) * (wb * v.prof);
   }
-  return L;
+  if (p.k == pp.max_depth) return false;
+  const float4 ua = p.rng.draw(p.k, 0), ub = p.rng.draw(p.k, 1);
+  const float4 ma = __ldg(&t.mat_a[v.seg]), mb = __ldg(&t.mat_b[v.seg]);
+  const float4 sa = __ldg(&t.samp[v.seg]);
+  if (light_on) {
+    const NeeResult ne = next_event(s, t, v, ua, ub, pp.profile, pp.mis, sa.y, sa.x, err);
+    if (ne.valid) {
+      const BrdfVal bv = brdf_eval(ma, mb, v.ns, v.wi, ne.wl);
+      p.L = p.L + p.beta * bv.f * xyz(__ldg(&t.emis[ne.seg])) * ne.k;
+    }
+  }
+  if (!(dot(v.wi, v.ns) > 0.0f)) return false;
+  const float3 wo = bsdf_sample(sa.w, sa.x, v.ns, v.wi, ua.x, ua.y, ua.z);
+  const float pdf = bsdf_pdf(sa.y, sa.x, v.ns, v.wi, wo);
+  const float co = dot(wo, v.ns);
+  if (!(dot(wo, v.ng) > 0.0f) || !(co > 0.0f) || !(pdf > 0.0f)) return false;
+  const BrdfVal bv = brdf_eval(ma, mb, v.ns, v.wi, wo);
+  p.beta = p.beta * bv.f * (co / pdf);
+  p.prev_pdf = pdf;
+  p.o = v.x + v.ng * s.eps;
+  p.d = wo;
+  p.skip = h.tri;
+  ++p.k;
+  return true;
+}
+
+// Radiance estimate of one camera path.
+__device__ __forceinline__ float3 forward_path(const SceneDev& s, const SegDev& t, const ViewDev& vw, uint32_t px,
+                                               uint32_t py, uint32_t pid, uint32_t sample, const PathParams& pp,
+                                               bool light, uint32_t* err) {
+  FwdPath p;
+  forward_start(p, vw, px, py, pid, sample, pp);
+  while (forward_vertex(s, t, pp, pp.nee && light, p, err)) {
+  }
+  return p.L;
 }
 
 __device__ __forceinline__ void add3(float* acc, int i, float3 v) {
@@ -186,14 +207,17 @@ __device__ void adjoint_path(const SceneDev& s, const SegDev& t, const ViewDev& 
 // ---------------------------------------------------------------------------
 // Forward kernel: each pixel is handled by `group` lanes of one warp, each
 // lane tracing spp / group samples; the lanes' sums are combined with
-// butterfly shuffles, so the pixel estimate is deterministic.
+// butterfly shuffles, so the pixel estimate is deterministic.  kRad: the
+// samples' radiances were traced before (k_forward_samples) and are read from
+// `rad`; the sums are the same, in the same order.
 // ---------------------------------------------------------------------------
+template <bool kRad>
 __global__ void __launch_bounds__(kBlockThreads) k_forward(SceneDev s, SegDev t, const ViewDev* views,
                                                            uint32_t n_views, uint32_t pix_begin, uint32_t n_pix,
                                                            PathParams pp, float* img, float* msq,
                                                            const float* target, float* g_out,
                                                            double* loss_partials, float g_scale, int loss_kind,
-                                                           uint32_t* err) {
+                                                           const float4* rad, uint32_t* err) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t G = pp.group;
   const uint32_t ppw = 32u / G;
@@ -219,7 +243,11 @@ __global__ void __launch_bounds__(kBlockThreads) k_forward(SceneDev s, SegDev t,
       const uint32_t lp = pid - vw.offset;
       const uint32_t px = lp % vw.w, py = lp / vw.w;
       for (uint32_t smp = sub; smp < pp.spp; smp += G) {
-        const float3 L = forward_path(s, t, vw, px, py, pid, s0 + smp, pp, light, err);
+        float3 L;
+        if constexpr (kRad)
+          L = xyz(rad[local * pp.spp + smp]);
+        else
+          L = forward_path(s, t, vw, px, py, pid, s0 + smp, pp, light, err);
         a = a + L;
         a2 = a2 + L * L;
       }
@@ -276,13 +304,43 @@ __global__ void __launch_bounds__(kBlockThreads) k_forward(SceneDev s, SegDev t,
   }
 }
 
+// Small launches (a pixel batch of Sec. 4.5) leave most of the chip idle when a
+// pixel's samples share one warp, and last as long as one lane's chain of
+// paths in a diverging warp.  Here sample i (of pixel i / spp) is one thread's,
+// `lanes` samples to a warp, with the samples spread over all warps that fit.
+// Pixel batches on a Cornell box, 8 pixels of 128 samples: 141 -> 36 us
+// (derivative pass 52 -> 30 us); on a 4.8k-triangle room 657 -> 81 us, and 512
+// pixels of 33 samples, one lane a pixel before, 5.44 -> 0.18 ms.  The 64-scene
+// Cornell batch (64 pixels of 64 samples each, 262k samples) gains from the
+// blocks being scheduled as they end: a step 0.58 -> 0.34 ms.  kFewWarpsPerSm
+// 4, 8, 12, 16: 512 pixels of 33: 0.205, 0.177, 0.173, 0.175 ms; derivative
+// pass of 3000 paths: 0.127, 0.121, 0.185, 0.186 ms.
+__global__ void __launch_bounds__(kBlockThreads) k_forward_samples(SceneDev s, SegDev t, const ViewDev* views,
+                                                                   uint32_t n_views, uint32_t pix_begin, uint32_t n,
+                                                                   uint32_t lanes, PathParams pp, float4* rad,
+                                                                   uint32_t* err) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t i = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * lanes + lane;
+  if (lane >= lanes || i >= n) return;
+  const uint32_t local = i / pp.spp, smp = i - local * pp.spp;
+  uint32_t pid = pix_begin + local, s0 = 0;
+  if (pp.pick) {
+    pid = pp.pick[local];
+    s0 = local * pp.stride;
+  }
+  const ViewDev& vw = find_view(views, n_views, pid);
+  const uint32_t lp = pid - vw.offset;
+  const float3 L = forward_path(s, t, vw, lp % vw.w, lp / vw.w, pid, s0 + smp, pp, any_light(s, t), err);
+  rad[i] = make_float4(L.x, L.y, L.z, 0.0f);
+}
+
 // Pixels [pix_begin, pix_begin + n_pix) of the concatenated views; g_img is
 // indexed relative to pix_begin.
 template <int MAXD>
-__global__ void __launch_bounds__(kBlockThreads) k_adjoint(SceneDev s, SegDev t, const ViewDev* views,
+__global__ void __launch_bounds__(kBlockThreads, MAXD <= 4 ? 3 : 2) k_adjoint(SceneDev s, SegDev t, const ViewDev* views,
                                                            uint32_t n_views, uint32_t pix_begin, uint32_t n_pix,
-                                                           PathParams pp, const float* g_img, double* grad_acc,
-                                                           float* gacc, uint32_t* err) {
+                                                           PathParams pp, uint32_t lanes, const float* g_img,
+                                                           double* grad_acc, float* gacc, uint32_t* err) {
   // per-block accumulators in shared memory, or (scenes with too many
   // segments for it) one zeroed accumulator in global memory
   extern __shared__ float sgrad_sh[];
@@ -292,26 +350,33 @@ __global__ void __launch_bounds__(kBlockThreads) k_adjoint(SceneDev s, SegDev t,
     for (uint32_t i = threadIdx.x; i < n_par; i += blockDim.x) sgrad[i] = 0.0f;
   __syncthreads();
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t G = pp.group;
-  const uint32_t ppw = 32u / G;
-  const uint32_t sub = lane & (G - 1u);
-  const uint32_t warps_per_block = blockDim.x >> 5;
-  const uint32_t n_tasks = (n_pix + ppw - 1) / ppw;
-  const uint32_t stride = gridDim.x * warps_per_block;
   const bool light = any_light(s, t);
   const float inv_spp = 1.0f / (float)pp.spp;
-  for (uint32_t task = blockIdx.x * warps_per_block + (threadIdx.x >> 5); task < n_tasks; task += stride) {
-    const uint32_t local = task * ppw + lane / G;
-    if (local >= n_pix) continue;
+  const auto paths = [&](uint32_t local, uint32_t first, uint32_t step) {
     const uint32_t pid = pp.pick ? pp.pick[local] : pix_begin + local;
     const uint32_t s0 = pp.pick ? local * pp.stride : 0u;
     const float3 gp = f3(g_img[3 * local], g_img[3 * local + 1], g_img[3 * local + 2]) * inv_spp;
-    if (gp.x == 0.0f && gp.y == 0.0f && gp.z == 0.0f) continue;
+    if (gp.x == 0.0f && gp.y == 0.0f && gp.z == 0.0f) return;
     const ViewDev& vw = find_view(views, n_views, pid);
     const uint32_t lp = pid - vw.offset;
     const uint32_t px = lp % vw.w, py = lp / vw.w;
-    for (uint32_t smp = sub; smp < pp.spp; smp += G)
+    for (uint32_t smp = first; smp < pp.spp; smp += step)
       adjoint_path<MAXD>(s, t, vw, px, py, pid, s0 + smp, pp, light, gp, sgrad, err);
+  };
+  // lanes > 0 (few paths): path i is one thread's, `lanes` paths to a warp;
+  // otherwise `group` lanes of a warp share a pixel
+  uint32_t task = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_tasks, stride = 1u;
+  const uint32_t G = pp.group, ppw = 32u / G;
+  if (lanes) {
+    n_tasks = lane < lanes && task * lanes + lane < n_pix * pp.spp ? task + 1u : 0u;
+  } else {
+    n_tasks = (n_pix + ppw - 1) / ppw;
+    stride = gridDim.x * (blockDim.x >> 5);
+  }
+  for (; task < n_tasks; task += stride) {
+    const uint32_t i = task * lanes + lane;
+    const uint32_t local = lanes ? i / pp.spp : task * ppw + lane / G;
+    if (local < n_pix) paths(local, lanes ? i % pp.spp : lane & (G - 1u), lanes ? pp.spp : G);
   }
   __syncthreads();
   if (!gacc)
@@ -354,10 +419,12 @@ __device__ __forceinline__ PathParams scene_params(const PathParams& base, const
 // scene's loss sum (rows[block * n_scenes + scene], the layout of the
 // wavefront's reduction).
 // Four resident blocks per SM (at most 128 registers), as the single-scene
-// forward: the grid is one loss row per block of a full wave.
+// forward: the grid is one loss row per block of a full wave.  kRad: reads the
+// radiances that k_forward_samples_batch traced, as k_forward does.
+template <bool kRad>
 __global__ void __launch_bounds__(kBlockThreads, 4)
     k_forward_batch(const WfScene* tab, uint32_t n_scenes, uint32_t total, PathParams pp, uint32_t set,
-                    const uint32_t* iter_dev, int loss_kind, double* loss_rows, uint32_t* err) {
+                    const uint32_t* iter_dev, int loss_kind, double* loss_rows, const float4* rad, uint32_t* err) {
   extern __shared__ double sloss[];
   for (uint32_t i = threadIdx.x; i < n_scenes; i += blockDim.x) sloss[i] = 0.0;
   __syncthreads();
@@ -380,13 +447,18 @@ __global__ void __launch_bounds__(kBlockThreads, 4)
       const WfScene& e = tab[b];
       entry = p - e.pix_begin + e.pix_base;
       pid = e.pick ? e.pick[entry] : entry;
-      const uint32_t s0 = e.pick ? entry * pp.stride : 0u;
-      const PathParams q = scene_params(pp, e, set_iter);
-      const bool light = any_light(e.s, e.t);
-      const ViewDev& vw = find_view(e.views, e.n_views, pid);
-      const uint32_t lp = pid - vw.offset;
-      const uint32_t px = lp % vw.w, py = lp / vw.w;
-      for (uint32_t smp = sub; smp < pp.spp; smp += G) a = a + forward_path(e.s, e.t, vw, px, py, pid, s0 + smp, q, light, err);
+      if constexpr (kRad) {
+        for (uint32_t smp = sub; smp < pp.spp; smp += G) a = a + xyz(rad[p * pp.spp + smp]);
+      } else {
+        const uint32_t s0 = e.pick ? entry * pp.stride : 0u;
+        const PathParams q = scene_params(pp, e, set_iter);
+        const bool light = any_light(e.s, e.t);
+        const ViewDev& vw = find_view(e.views, e.n_views, pid);
+        const uint32_t lp = pid - vw.offset;
+        const uint32_t px = lp % vw.w, py = lp / vw.w;
+        for (uint32_t smp = sub; smp < pp.spp; smp += G)
+          a = a + forward_path(e.s, e.t, vw, px, py, pid, s0 + smp, q, light, err);
+      }
     }
     for (uint32_t off = G >> 1; off >= 1; off >>= 1) {
       a.x += __shfl_xor_sync(0xffffffffu, a.x, off);
@@ -416,12 +488,32 @@ __global__ void __launch_bounds__(kBlockThreads, 4)
   for (uint32_t i = threadIdx.x; i < n_scenes; i += blockDim.x) loss_rows[(size_t)blockIdx.x * n_scenes + i] = sloss[i];
 }
 
+// One sample of a launch pixel a thread (see k_forward_samples).
+__global__ void __launch_bounds__(kBlockThreads, 4)
+    k_forward_samples_batch(const WfScene* tab, uint32_t n_scenes, uint32_t n, uint32_t lanes, PathParams pp,
+                            uint32_t set, const uint32_t* iter_dev, float4* rad, uint32_t* err) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t i = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * lanes + lane;
+  if (lane >= lanes || i >= n) return;
+  const uint32_t p = i / pp.spp, smp = i - p * pp.spp;
+  const WfScene& e = tab[table_scene(tab, n_scenes, p)];
+  const uint32_t entry = p - e.pix_begin + e.pix_base;
+  const uint32_t pid = e.pick ? e.pick[entry] : entry;
+  const uint32_t s0 = e.pick ? entry * pp.stride : 0u;
+  const PathParams q = scene_params(pp, e, (set << 24) | (*iter_dev & 0xFFFFFFu));
+  const ViewDev& vw = find_view(e.views, e.n_views, pid);
+  const uint32_t lp = pid - vw.offset;
+  const float3 L =
+      forward_path(e.s, e.t, vw, lp % vw.w, lp / vw.w, pid, s0 + smp, q, any_light(e.s, e.t), err);
+  rad[i] = make_float4(L.x, L.y, L.z, 0.0f);
+}
+
 // Derivative pass: every entry's paths into the batch's packed segment
 // accumulators (shared per block, or global when they do not fit).
 template <int MAXD>
-__global__ void __launch_bounds__(kBlockThreads)
+__global__ void __launch_bounds__(kBlockThreads, MAXD <= 4 ? 3 : 2)
     k_adjoint_batch(const WfScene* tab, uint32_t n_scenes, uint32_t total, uint32_t n_par, PathParams pp,
-                    uint32_t set, const uint32_t* iter_dev, double* grad_acc, float* gacc, uint32_t* err) {
+                    uint32_t lanes, uint32_t set, const uint32_t* iter_dev, double* grad_acc, float* gacc, uint32_t* err) {
   extern __shared__ float bgrad_sh[];
   float* acc = gacc ? gacc : bgrad_sh;
   if (!gacc)
@@ -429,30 +521,36 @@ __global__ void __launch_bounds__(kBlockThreads)
   __syncthreads();
   const uint32_t set_iter = (set << 24) | (*iter_dev & 0xFFFFFFu);
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t G = pp.group;
-  const uint32_t ppw = 32u / G;
-  const uint32_t sub = lane & (G - 1u);
-  const uint32_t warps_per_block = blockDim.x >> 5;
-  const uint32_t n_tasks = (total + ppw - 1) / ppw;
-  const uint32_t stride = gridDim.x * warps_per_block;
   const float inv_spp = 1.0f / (float)pp.spp;
-  for (uint32_t task = blockIdx.x * warps_per_block + (threadIdx.x >> 5); task < n_tasks; task += stride) {
-    const uint32_t p = task * ppw + lane / G;
-    if (p >= total) continue;
+  const auto paths = [&](uint32_t p, uint32_t first, uint32_t step) {
     const WfScene& e = tab[table_scene(tab, n_scenes, p)];
     const uint32_t entry = p - e.pix_begin + e.pix_base;
     const uint32_t pid = e.pick ? e.pick[entry] : entry;
     const uint32_t s0 = e.pick ? entry * pp.stride : 0u;
     const float3 gp = f3(e.g_img[3 * entry], e.g_img[3 * entry + 1], e.g_img[3 * entry + 2]) * inv_spp;
-    if (gp.x == 0.0f && gp.y == 0.0f && gp.z == 0.0f) continue;
+    if (gp.x == 0.0f && gp.y == 0.0f && gp.z == 0.0f) return;
     const PathParams q = scene_params(pp, e, set_iter);
     const bool light = any_light(e.s, e.t);
     const ViewDev& vw = find_view(e.views, e.n_views, pid);
     const uint32_t lp = pid - vw.offset;
     const uint32_t px = lp % vw.w, py = lp / vw.w;
     float* sacc = acc + 10u * e.seg_offset;
-    for (uint32_t smp = sub; smp < pp.spp; smp += G)
+    for (uint32_t smp = first; smp < pp.spp; smp += step)
       adjoint_path<MAXD>(e.s, e.t, vw, px, py, pid, s0 + smp, q, light, gp, sacc, err);
+  };
+  // paths to threads as in k_adjoint
+  uint32_t task = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_tasks, stride = 1u;
+  const uint32_t G = pp.group, ppw = 32u / G;
+  if (lanes) {
+    n_tasks = lane < lanes && task * lanes + lane < total * pp.spp ? task + 1u : 0u;
+  } else {
+    n_tasks = (total + ppw - 1) / ppw;
+    stride = gridDim.x * (blockDim.x >> 5);
+  }
+  for (; task < n_tasks; task += stride) {
+    const uint32_t i = task * lanes + lane;
+    const uint32_t p = lanes ? i / pp.spp : task * ppw + lane / G;
+    if (p < total) paths(p, lanes ? i % pp.spp : lane & (G - 1u), lanes ? pp.spp : G);
   }
   __syncthreads();
   if (!gacc)
@@ -734,7 +832,7 @@ static void adjoint_occupancy(int* out) {
 cudaError_t init_launcher(Launcher* L, int device) {
   cudaError_t e = cudaDeviceGetAttribute(&L->num_sms, cudaDevAttrMultiProcessorCount, device);
   if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L->fwd_blocks_per_sm, k_forward, kBlockThreads, 0);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&L->fwd_blocks_per_sm, k_forward<false>, kBlockThreads, 0);
   if (e != cudaSuccess) return e;
   adjoint_occupancy<2>(&L->adj_blocks_per_sm[0]);
   adjoint_occupancy<4>(&L->adj_blocks_per_sm[1]);
@@ -758,6 +856,25 @@ static int grid_for(uint64_t n_tasks_warps, int blocks_cap) {
   return (int)g;
 }
 
+// Samples per warp of a launch of n samples that runs one sample a thread: as
+// few as kFewWarpsPerSm warps on each SM allow, 32 beyond that.
+constexpr uint32_t kFewWarpsPerSm = 8;
+static uint32_t few_lanes(const Launcher& L, uint64_t n) {
+  const uint32_t warps = kFewWarpsPerSm * (uint32_t)L.num_sms;
+  return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(32, (n + warps - 1u) / warps));
+}
+
+// The residual pass runs one sample a thread up to the capacity of the
+// radiance buffer; the derivative pass, whose blocks each clear and flush
+// their accumulators, up to one wave of warps.
+static bool few_forward(const Launcher& L, uint64_t n) { return n <= L.rad_cap; }
+static bool few_adjoint(const Launcher& L, uint64_t n) { return n <= 32ull * kFewWarpsPerSm * (uint32_t)L.num_sms; }
+
+static int few_grid(uint32_t n, uint32_t lanes) {
+  const uint32_t per_block = lanes * (kBlockThreads / 32u);
+  return (int)((n + per_block - 1u) / per_block);
+}
+
 cudaError_t launch_prepare(const SceneBuffers& s, const SegBuffers& t, const float* params,
                            const float* sparams, cudaStream_t st) {
   if (s.n_seg > kWideSegments) return launch_tables_wide(s, t, params, sparams ? sparams : params, nullptr, nullptr, st);
@@ -775,9 +892,19 @@ cudaError_t launch_forward(const Launcher& L, const SceneBuffers& s, const SegBu
   const int cap = L.num_sms * L.fwd_blocks_per_sm;
   // with a loss the grid is fixed, so the partial sums reduce in a fixed order
   const int grid = loss_partials ? cap : grid_for(tasks, cap);
-  k_forward<<<grid, kBlockThreads, 0, st>>>(scene_dev(s), seg_dev(t), reinterpret_cast<const ViewDev*>(views_dev),
-                                             n_views, pix_begin, n_pix, pp, img, msq, target, g_out,
-                                             loss_partials, g_scale, loss_kind, err);
+  const SceneDev sd = scene_dev(s);
+  const SegDev td = seg_dev(t);
+  const ViewDev* vd = reinterpret_cast<const ViewDev*>(views_dev);
+  if (few_forward(L, (uint64_t)n_pix * tp.spp)) {
+    const uint32_t n = n_pix * tp.spp, lanes = few_lanes(L, n);
+    k_forward_samples<<<few_grid(n, lanes), kBlockThreads, 0, st>>>(sd, td, vd, n_views, pix_begin, n, lanes, pp, L.rad,
+                                                                  err);
+    k_forward<true><<<grid, kBlockThreads, 0, st>>>(sd, td, vd, n_views, pix_begin, n_pix, pp, img, msq, target, g_out,
+                                                    loss_partials, g_scale, loss_kind, L.rad, err);
+    return cudaGetLastError();
+  }
+  k_forward<false><<<grid, kBlockThreads, 0, st>>>(sd, td, vd, n_views, pix_begin, n_pix, pp, img, msq, target, g_out,
+                                                   loss_partials, g_scale, loss_kind, nullptr, err);
   return cudaGetLastError();
 }
 
@@ -797,14 +924,17 @@ cudaError_t launch_adjoint(const Launcher& L, const SceneBuffers& s, const SegBu
     if (e != cudaSuccess) return e;
   }
   const ViewDev* vd = reinterpret_cast<const ViewDev*>(views_dev);
+  const uint64_t n_paths = (uint64_t)n_pix * tp.spp;
+  const uint32_t lanes = few_adjoint(L, n_paths) ? few_lanes(L, n_paths) : 0u;
   const int md = tp.max_depth < 1 ? 1 : (int)tp.max_depth;
 #define IPT_LAUNCH_ADJ(D, I)                                                                         \
   {                                                                                                  \
     if (shmem > 48 * 1024)                                                                           \
       cudaFuncSetAttribute(k_adjoint<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);  \
-    const int grid = grid_for(tasks, L.num_sms * L.adj_blocks_per_sm[I]);                            \
+    const int grid = lanes ? few_grid(n_pix * tp.spp, lanes)                                         \
+                           : grid_for(tasks, L.num_sms * L.adj_blocks_per_sm[I]);                    \
     k_adjoint<D><<<grid, kBlockThreads, shmem, st>>>(scene_dev(s), seg_dev(t), vd, n_views, pix_begin, n_pix, pp, \
-                                                     g_img, grad_acc, gacc, err);                    \
+                                                     lanes, g_img, grad_acc, gacc, err);             \
   }
   if (md <= 2)
     IPT_LAUNCH_ADJ(2, 0)
@@ -835,8 +965,19 @@ cudaError_t launch_forward_batch(const Launcher& L, const WfScene* tab_dev, uint
                                  const TraceParams& tp, const uint32_t* iter_dev, int loss_kind, double* loss_rows,
                                  uint32_t* err, cudaStream_t st) {
   // one block per loss row: every row of the batch's loss reduction is written
-  k_forward_batch<<<loss_partials_capacity(L), kBlockThreads, sizeof(double) * n_scenes, st>>>(
-      tab_dev, n_scenes, total, batch_path_params(tp), tp.set, iter_dev, loss_kind, loss_rows, err);
+  const PathParams pp = batch_path_params(tp);
+  const size_t sm = sizeof(double) * n_scenes;
+  if (few_forward(L, (uint64_t)total * tp.spp)) {
+    const uint32_t n = total * tp.spp, lanes = few_lanes(L, n);
+    if (n)
+      k_forward_samples_batch<<<few_grid(n, lanes), kBlockThreads, 0, st>>>(tab_dev, n_scenes, n, lanes, pp, tp.set,
+                                                                          iter_dev, L.rad, err);
+    k_forward_batch<true><<<loss_partials_capacity(L), kBlockThreads, sm, st>>>(
+        tab_dev, n_scenes, total, pp, tp.set, iter_dev, loss_kind, loss_rows, L.rad, err);
+    return cudaGetLastError();
+  }
+  k_forward_batch<false><<<loss_partials_capacity(L), kBlockThreads, sm, st>>>(
+      tab_dev, n_scenes, total, pp, tp.set, iter_dev, loss_kind, loss_rows, nullptr, err);
   return cudaGetLastError();
 }
 
@@ -856,14 +997,17 @@ cudaError_t launch_adjoint_batch(const Launcher& L, const WfScene* tab_dev, uint
     if (e != cudaSuccess) return e;
   }
   const uint64_t tasks = ((uint64_t)total + (32 / pp.group) - 1) / (32 / pp.group);
+  const uint64_t n_paths = (uint64_t)total * tp.spp;
+  const uint32_t lanes = few_adjoint(L, n_paths) ? few_lanes(L, n_paths) : 0u;
   const int md = tp.max_depth < 1 ? 1 : (int)tp.max_depth;
 #define IPT_LAUNCH_ADJB(D, I)                                                                              \
   {                                                                                                        \
     if (shmem > 48 * 1024)                                                                                 \
       cudaFuncSetAttribute(k_adjoint_batch<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);  \
-    const int grid = grid_for(tasks, L.num_sms * L.adj_blocks_per_sm[I]);                                  \
-    k_adjoint_batch<D><<<grid, kBlockThreads, shmem, st>>>(tab_dev, n_scenes, total, n_par, pp, tp.set,    \
-                                                           iter_dev, grad_acc, gacc, err);                 \
+    const int grid = lanes ? few_grid((uint32_t)n_paths, lanes)                                            \
+                           : grid_for(tasks, L.num_sms * L.adj_blocks_per_sm[I]);                          \
+    k_adjoint_batch<D><<<grid, kBlockThreads, shmem, st>>>(tab_dev, n_scenes, total, n_par, pp, lanes,     \
+                                                           tp.set, iter_dev, grad_acc, gacc, err);         \
   }
   if (md <= 2)
     IPT_LAUNCH_ADJB(2, 0)

@@ -2227,7 +2227,9 @@ cudaError_t wf_pick(const WfScene* tab_dev, const std::vector<WfScene>& tab, con
   return cudaGetLastError();
 }
 
-cudaError_t wf_init(Launcher* L) {
+// Resident blocks per SM, asked once per context (a configuration only
+// overrides them).
+static cudaError_t wf_occupancy(Launcher* L) {
   // the fewest resident blocks of any traversal variant, so that every
   // width's persistent grid fits in one wave
   int b = 1 << 30;
@@ -2253,19 +2255,31 @@ cudaError_t wf_init(Launcher* L) {
     if (e != cudaSuccess) return e;
     b = std::min(b, bk);
   }
-  L->wf_blocks_per_sm = b < 1 ? 1 : b;
-  if (L->wf_fixed_blocks > 0) L->wf_blocks_per_sm = L->wf_fixed_blocks;
-  // gradient rows: the widest one-wave grid of an adjoint stage (accumulators
-  // in dynamic shared memory only lower the occupancy)
-  int rows = 0;
-  rows = std::max(rows, one_wave(*L, wf_adj_a<false, false>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_connect<false, false>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_b<false, false>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_a<true, false>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_connect<true, false>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_b<true, false>, 0));
-  rows = std::max(rows, one_wave(*L, wf_adj_cache<false>, 0));
-  L->wf_max_rows = rows;
+  L->wf_occ = b < 1 ? 1 : b;
+  // the adjoint stage with the most blocks (accumulators in dynamic shared
+  // memory only lower the occupancy)
+  const void* stages[] = {(const void*)wf_adj_a<false, false>, (const void*)wf_adj_connect<false, false>,
+                          (const void*)wf_adj_b<false, false>, (const void*)wf_adj_a<true, false>,
+                          (const void*)wf_adj_connect<true, false>, (const void*)wf_adj_b<true, false>,
+                          (const void*)wf_adj_cache<false>};
+  L->wf_row_occ = 1;
+  for (const void* k : stages) {
+    int bk = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bk, k, kWfThreads, 0);
+    if (e != cudaSuccess) return e;
+    L->wf_row_occ = std::max(L->wf_row_occ, bk);
+  }
+  return cudaSuccess;
+}
+
+cudaError_t wf_init(Launcher* L) {
+  if (L->wf_occ == 0) {
+    const cudaError_t e = wf_occupancy(L);
+    if (e != cudaSuccess) return e;
+  }
+  L->wf_blocks_per_sm = L->wf_fixed_blocks > 0 ? L->wf_fixed_blocks : L->wf_occ;
+  // gradient rows: the widest one-wave grid of an adjoint stage
+  L->wf_max_rows = L->num_sms * (L->wf_fixed_blocks > 0 ? L->wf_fixed_blocks : L->wf_row_occ);
   return cudaSuccess;
 }
 
