@@ -292,9 +292,7 @@ ipt_status ipt_batch_params_get(ipt_ctx* ctx, int32_t batch, uint32_t member, fl
   if (member >= b->members.size() || !params_out) return fail(ctx, IPT_ERR_INVALID_ARG, "bad member or output");
   const ipt::BatchMember& m = b->mem_host[member];
   IPT_CK(cudaSetDevice(ctx->device));
-  IPT_CK(cudaMemcpyAsync(params_out, b->params + 10 * (size_t)m.seg_offset, 10 * sizeof(float) * m.n_seg,
-                         cudaMemcpyDeviceToHost, ctx->stream));
-  return ipt_synchronize(ctx);
+  return read_back(ctx, params_out, b->params + 10 * (size_t)m.seg_offset, 10 * sizeof(float) * m.n_seg);
 }
 
 ipt_status ipt_batch_destroy(ipt_ctx* ctx, int32_t batch) {

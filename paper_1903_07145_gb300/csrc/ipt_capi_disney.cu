@@ -120,9 +120,7 @@ ipt_status ipt_disney_params_get(ipt_ctx* ctx, int32_t scene, float* params_out)
   if (st != IPT_OK) return st;
   if (!params_out) return fail(ctx, IPT_ERR_INVALID_ARG, "null output");
   IPT_CK(cudaSetDevice(ctx->device));
-  IPT_CK(cudaMemcpyAsync(params_out, d->params, kDisneyValues * sizeof(float) * s->n_seg, cudaMemcpyDeviceToHost,
-                         ctx->stream));
-  return ipt_synchronize(ctx);
+  return read_back(ctx, params_out, d->params, kDisneyValues * sizeof(float) * s->n_seg);
 }
 
 ipt_status ipt_disney_render(ipt_ctx* ctx, int32_t scene, int32_t view, const ipt_trace_opts* opts, uint32_t set,

@@ -195,7 +195,12 @@ struct ipt_ctx {
   std::vector<ipt_capi::DeviceScene*> scenes;
   std::string last_error;
   uint32_t* err_dev = nullptr;
-  double* loss_host = nullptr;  // pinned
+  // pinned host words: the loss, the error word (at err_host) and a staging
+  // area for small results (stage_host), so that a call that returns them
+  // queues its copies and waits once
+  double* loss_host = nullptr;
+  uint32_t* err_host = nullptr;
+  unsigned char* stage_host = nullptr;
   unsigned long long* counters_dev = nullptr;
   std::vector<ipt_capi::PendingTiming> pending;
   std::vector<cudaEvent_t> spare_events;
@@ -239,6 +244,9 @@ void wf_release(ipt_ctx* c);
 // grow.
 ipt_status ensure_wf(ipt_ctx* ctx, bool adjoint, uint32_t n_params, bool disney = false, uint32_t depth = 0);
 void ensure_rad(ipt_ctx* ctx, uint64_t n);
+// Copies n bytes of device memory to `dst` in stream order and waits for the
+// stream (as ipt_synchronize: returns any device-side error).
+ipt_status read_back(ipt_ctx* ctx, void* dst, const void* src, size_t n);
 bool use_wavefront_cap(const ipt_ctx* ctx, uint32_t spp);
 bool use_wavefront(const ipt_ctx* ctx, uint32_t spp);
 ipt::WfScene wf_entry(const ipt_ctx* ctx, int32_t scene_id, const DeviceScene* s, uint32_t pix_base, uint32_t n);
