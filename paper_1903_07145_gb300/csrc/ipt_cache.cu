@@ -187,7 +187,7 @@ __device__ __forceinline__ float3 unit_pos(const CacheNet& net, float4 x) {
 // table's FP16 copy (queries) instead of the FP32 master (training and the
 // input VJP, whose result depends on the table only through the ReLU
 // decisions, which the FP16 rounding would move near their kinks).
-template <bool kHalf, class Tile>
+template <bool kHalf, int kUnroll, class Tile>
 __device__ __forceinline__ void encode_rows(const CacheNet& net, const int* res, const CacheRows& rows, const float4* mat_a,
                             const float4* mat_b, uint32_t r0, uint32_t end, Tile X, float4* meta, int lane) {
   const int row = lane & 15;
@@ -223,32 +223,62 @@ __device__ __forceinline__ void encode_rows(const CacheNet& net, const int* res,
     for (int i = 0; i < 8; ++i) X(row, w0 + i) = valid ? pack2(sh[2 * i], sh[2 * i + 1]) : 0u;
   }
   __syncwarp();
+  // Two lanes take a row's level, one the cell's corners at x, one those at
+  // x + 1, so that the neighbours are gathered by one instruction: they lie in
+  // one line nearly always (dense levels: adjacent; hashed levels: the index
+  // differs in the low bits in which x and x + 1 differ), and the L1 pays per
+  // line.  The lanes then exchange features and each sums one of them over
+  // the corners in order.  kUnroll levels at a time: their gathers are all
+  // issued before the first word is stored.  Rows past the end gather too
+  // (their position is in the cube) and store 0.  Input
+  // VJP of 500k random rows 0.249 -> 0.214 ms, of the 61k room's 4.9M rows 1.98
+  // -> 1.66 ms; queries of those 1.44 -> 1.37 ms.  (Fetching the aligned group
+  // of four entries with one wide load per neighbour pair was slower.)
+  const int er = lane >> 1;
+  const bool odd = lane & 1;
+  const float4 m = meta[er];
 #pragma unroll 1
-  for (int i = 0; i < 8; ++i) {
-    const int item = lane + 32 * i;
-    const int rr = item & 15, l = item >> 4;
-    const float4 m = meta[rr];
-    uint32_t word = 0u;
-    if (m.w != 0.0f) {
-      uint32_t idx[8];
-      float w[8];
-      level_corners(res, net.dense, l, make_float3(m.x, m.y, m.z), idx, w);
-      float f0 = 0.0f, f1 = 0.0f;
+  for (int l0 = 0; l0 < kCacheLevels; l0 += kUnroll) {
+    uint32_t word[kUnroll];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        float2 v;
+    for (int u = 0; u < kUnroll; ++u) {
+      const int l = l0 + u, nr = res[l];
+      const float px = m.x * (float)nr, py = m.y * (float)nr, pz = m.z * (float)nr;
+      const float gx = floorf(px), gy = floorf(py), gz = floorf(pz);
+      const int ix = (int)gx, iy = (int)gy, iz = (int)gz;
+      const float fx = px - gx, fy = py - gy, fz = pz - gz;
+      const bool dense = (net.dense >> l) & 1u;
+      const uint32_t s1 = (uint32_t)nr + 1u, base = (uint32_t)l * kCacheT;
+      const uint32_t cx = (uint32_t)min(ix + (odd ? 1 : 0), nr);
+      float2 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t cy = (uint32_t)min(iy + (k & 1), nr), cz = (uint32_t)min(iz + (k >> 1), nr);
+        const uint32_t h = dense ? cx + cy * s1 + cz * s1 * s1 : (cx ^ (cy * 2654435761u) ^ (cz * 805459861u));
+        const uint32_t at = base + (h & (kCacheT - 1u));
         if (kHalf) {
-          const uint32_t hv = __ldg(&net.table_h[idx[c]]);
-          v = __half22float2(*reinterpret_cast<const __half2*>(&hv));
+          const uint32_t hv = __ldg(&net.table_h[at]);
+          v[k] = __half22float2(*reinterpret_cast<const __half2*>(&hv));
         } else {
-          v = __ldg(&net.table[idx[c]]);
+          v[k] = __ldg(&net.table[at]);
         }
-        f0 += w[c] * v.x;
-        f1 += w[c] * v.y;
       }
-      word = pack2(f0, f1);
+      float f = 0.0f;  // feature 0 in the even lane, 1 in the odd one
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float own = odd ? v[k].y : v[k].x;
+        const float got = __shfl_xor_sync(0xffffffffu, odd ? v[k].x : v[k].y, 1);
+        const float w0 = (1.0f - fx) * ((k & 1) ? fy : 1.0f - fy) * ((k & 2) ? fz : 1.0f - fz);
+        const float w1 = fx * ((k & 1) ? fy : 1.0f - fy) * ((k & 2) ? fz : 1.0f - fz);
+        f += w0 * (odd ? got : own);
+        f += w1 * (odd ? own : got);
+      }
+      const float other = __shfl_xor_sync(0xffffffffu, f, 1);
+      word[u] = m.w != 0.0f ? pack2(f, other) : 0u;
     }
-    X(rr, l) = word;
+    if (!odd)
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) X(er, l0 + u) = word[u];
   }
   __syncwarp();
 }
@@ -508,7 +538,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32, 2) cache_vjp_k(CacheNet net, C
        tile += gridDim.x * (uint32_t)kVjpWarps) {
     const uint32_t r0 = tile * 16u;
     __syncwarp();
-    encode_rows<false>(net, res, rows, mat_a, mat_b, r0, n, X, meta, lane);
+    encode_rows<false, 2>(net, res, rows, mat_a, mat_b, r0, n, X, meta, lane);
     float y[2][4];
     uint32_t mask[4];
     net_forward_mask(Wt, X, y, mask, lane);
@@ -721,7 +751,7 @@ __global__ void __launch_bounds__(kThreads) cache_grad_k(CacheNet net, CacheRows
       }
     }
     const uint32_t r0 = begin + tile * kTileRows + 16u * (uint32_t)warp;
-    encode_rows<false>(net, res, rows, mat_a, mat_b, r0, end, X, meta, lane);
+    encode_rows<false, 2>(net, res, rows, mat_a, mat_b, r0, end, X, meta, lane);
     float y[2][4];
     net_forward<true>(Wt, X, H, hstride, y, lane);
     // relative L2: d/dy_c of (y_c - t_c)^2 / (sg(y_c)^2 + 0.01), mean over rows and channels
@@ -813,33 +843,37 @@ __global__ void __launch_bounds__(kThreads) cache_grad_k(CacheNet net, CacheRows
 }
 
 // ---------------------------------------------------------------------------
-// Inference on the fifth-generation tensor cores: 128-row tiles per block of
-// four warps, one row per thread.  Each warp encodes its 32 rows into the
-// block's input tile; per layer one thread issues the MMAs (A = the tile,
-// K-major: the rows' features in 128-byte chunks; B = the layer's weights in
-// the same blocked layout, K-major: each output's inputs in chunks) into a
-// 128 x 64 FP32 accumulator in TMEM; every thread then reads its row back
-// with tcgen05.ld, applies the ReLU and writes the next layer's BF16 tile
-// (over the layer's own input tile, whose MMAs have completed).  Two blocks
-// per SM: one block's gathers overlap the other's MMA round trips, and the
-// 74 KB of shared memory a block takes leave most of the SM's L1 to the
-// hash-table gathers (three blocks per SM, with 28 KB of L1 left, were 36%
-// slower).
+// Inference on the fifth-generation tensor cores: 128-row tiles, one row per
+// thread, kQGroups groups of four warps per block.  Each warp encodes its 32
+// rows into the group's tile; per layer one thread of the group issues the
+// MMAs (A = the tile, K-major: the rows' features in 128-byte chunks; B = the
+// layer's weights in the same blocked layout, K-major: each output's inputs
+// in chunks) into a 128 x 64 FP32 accumulator in TMEM; every thread then reads
+// its row back with tcgen05.ld, applies the ReLU and writes the next layer's
+// BF16 row over the layer's own input tile (whose MMAs have completed).  The
+// groups run on their own (named barriers, an mbarrier and 128 TMEM columns
+// each) and share one image of the weights: one block per SM, whose groups'
+// gathers overlap the others' MMA round trips, and whose 130 KB leave the
+// rest of the SM's 256 KB to the L1 that the gathers go through.  The L1's
+// lookups bound the kernel (one for every line a gather touches).  4.9M rows
+// of the 61k room's paths: 1.89 ms with two blocks of one group (148 KB, input
+// and activation tiles apart), 1.78 with a row's gathers of four levels issued
+// together, 1.44 with four groups (three: 1.55).
 // ---------------------------------------------------------------------------
 constexpr int kQRows = 128;
+constexpr int kQGroups = 4;
 constexpr int kQLboX = 10 * 128, kQLboH = 8 * 128;  // bytes between 8-row groups (activation tiles, weights)
 constexpr int kQW1 = 0;                               // 64 outputs x 80 inputs
 constexpr int kQW2 = kQW1 + 8 * kQLboX;               // W2..W4: 64 x 64 each
 constexpr int kQW5 = kQW2 + 3 * 8 * kQLboH;           // 16 outputs x 64 inputs
-constexpr int kQX = kQW5 + 2 * kQLboH;
-constexpr int kQH = kQX + (kQRows / 8) * kQLboX;      // one 128 x 64 tile
-constexpr int kQMeta = kQH + (kQRows / 8) * kQLboH;
-constexpr int kQBar = kQMeta + kQRows * 16;
-constexpr int kSmemInferTc = kQBar + 16;
-constexpr uint32_t kQCols = 128;                      // TMEM columns of a block
-static_assert(kQX % 128 == 0 && kQH % 128 == 0 && kQMeta % 16 == 0 && kQBar % 16 == 0, "tile alignment");
-static_assert(2 * kSmemInferTc <= 227 * 1024, "two inference blocks per SM");
-static_assert(2 * kQCols <= 512, "two inference blocks' TMEM per SM");
+constexpr int kQX = kQW5 + 2 * kQLboH;                // the groups: tile, then row metadata
+constexpr int kQTile = (kQRows / 8) * kQLboX;         // 128 x 80 inputs, then 128 x 64 activations in their place
+constexpr int kQGroup = kQTile + kQRows * 16;
+constexpr int kQBar = kQX + kQGroups * kQGroup;       // mbarriers (8 bytes each), TMEM address
+constexpr int kSmemInferTc = kQBar + 8 * kQGroups + 16;
+constexpr uint32_t kQCols = 128;                      // TMEM columns of a group
+static_assert(kQX % 128 == 0 && kQTile % 128 == 0 && kQGroup % 128 == 0 && kQBar % 16 == 0, "tile alignment");
+static_assert(kSmemInferTc <= 227 * 1024 && kQGroups * kQCols <= 512, "one inference block per SM");
 
 // The out-major BF16 weight image (mma.sync layout, padded rows) re-laid in
 // the blocked K-major layout: output n, input chunk c (8 inputs, 16 bytes)
@@ -898,66 +932,81 @@ __device__ __forceinline__ void issue_layer(uint32_t tmem, uint32_t a, uint32_t 
     umma_bf16(tmem, umma_sdesc(a + 256u * k, 128, a_lbo), umma_sdesc(w + 256u * k, 128, w_lbo), idesc, k > 0 ? 1u : 0u);
 }
 
-__global__ void __launch_bounds__(128, 2) cache_infer_tc_k(CacheNet net, CacheRows rows, const float4* mat_a,
-                                                           const float4* mat_b, const uint32_t* count_dev,
-                                                           uint32_t n_max, CacheOut o) {
+// Barrier of a group's 128 threads (ids 1..kQGroups; 0 is __syncthreads), and
+// the same with the conjunction of a predicate.
+__device__ __forceinline__ void group_sync(int g) { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); }
+
+__device__ __forceinline__ bool group_and(int g, bool p) {
+  uint32_t r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.and.pred q, %2, 128, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"(p ? 1u : 0u), "r"(g + 1)
+      : "memory");
+  return r != 0u;
+}
+
+__global__ void __launch_bounds__(128 * kQGroups, 1)
+    cache_infer_tc_k(CacheNet net, CacheRows rows, const float4* mat_a, const float4* mat_b,
+                     const uint32_t* count_dev, uint32_t n_max, CacheOut o) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int res[kCacheLevels];
   load_weights_blocked(net, sm, res);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + kQBar + 8);
-  const uint32_t mbar = smem_addr(sm + kQBar);
-  if (warp == 0) {
+  const int g = threadIdx.x >> 7;  // group
+  const int warp = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + kQBar + 8 * kQGroups);
+  const uint32_t mbar = smem_addr(sm + kQBar + 8 * g);
+  if (threadIdx.x < 32) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
-                 "r"(kQCols)
+                 "r"(kQCols * kQGroups)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar), "r"(1) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
+  if (threadIdx.x < kQGroups)
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(sm + kQBar + 8 * threadIdx.x)), "r"(1)
+                 : "memory");
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = *tmem_slot + kQCols * (uint32_t)g;
   const uint32_t tlane = tmem + ((uint32_t)(32 * warp) << 16);  // this warp's 32 TMEM lanes
   const uint32_t n = count_dev ? min(*count_dev, n_max) : n_max;
-  const uint32_t base = smem_addr(sm);
-  const BlockTile X{reinterpret_cast<uint32_t*>(sm + kQX), kQLboX / 4};
-  float4* meta = reinterpret_cast<float4*>(sm + kQMeta);
+  const uint32_t base = smem_addr(sm), tile_addr = base + (uint32_t)(kQX + g * kQGroup);
+  unsigned char* tile_sm = sm + kQX + g * kQGroup;
+  const BlockTile X{reinterpret_cast<uint32_t*>(tile_sm), kQLboX / 4};
+  const BlockTile H{reinterpret_cast<uint32_t*>(tile_sm), kQLboH / 4};
+  float4* meta = reinterpret_cast<float4*>(tile_sm + kQTile);
   const int row = 32 * warp + lane;  // this thread's row of the tile
   uint32_t phase = 0;
   bool ok = true;
   const uint32_t n_tiles = (n + kQRows - 1u) / kQRows;
-  for (uint32_t tile = blockIdx.x; tile < n_tiles && ok; tile += gridDim.x) {
+  // a launch of few tiles takes the blocks' first groups first
+  for (uint32_t tile = blockIdx.x + gridDim.x * (uint32_t)g; tile < n_tiles && ok; tile += gridDim.x * kQGroups) {
     const uint32_t r0 = tile * kQRows;
-    encode_rows<true>(net, res, rows, mat_a, mat_b, r0 + 32u * warp, n, X.rows_from(32 * warp), meta + 32 * warp, lane);
-    encode_rows<true>(net, res, rows, mat_a, mat_b, r0 + 32u * warp + 16u, n, X.rows_from(32 * warp + 16),
-                meta + 32 * warp + 16, lane);
+    encode_rows<true, 4>(net, res, rows, mat_a, mat_b, r0 + 32u * warp, n, X.rows_from(32 * warp), meta + 32 * warp, lane);
+    encode_rows<true, 4>(net, res, rows, mat_a, mat_b, r0 + 32u * warp + 16u, n, X.rows_from(32 * warp + 16),
+                         meta + 32 * warp + 16, lane);
     float y[3] = {0.f, 0.f, 0.f};
 #pragma unroll 1
     for (int l = 0; l < 5 && ok; ++l) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       tc_fence_before();
-      __syncthreads();
-      if (threadIdx.x == 0) {
+      group_sync(g);
+      if ((threadIdx.x & 127u) == 0u) {
         tc_fence_after();
-        const uint32_t a = base + (uint32_t)(l == 0 ? kQX : kQH);
-        const uint32_t a_lbo = l == 0 ? kQLboX : kQLboH;
         const uint32_t w = base + (uint32_t)(l == 0 ? kQW1 : (l < 4 ? kQW2 + (l - 1) * 8 * kQLboH : kQW5));
-        const uint32_t w_lbo = l == 0 ? kQLboX : kQLboH;
-        issue_layer(tmem, a, a_lbo, w, w_lbo, l == 0 ? 80 : 64, l < 4 ? 64 : 16);
+        const uint32_t lbo = l == 0 ? kQLboX : kQLboH;
+        issue_layer(tmem, tile_addr, lbo, w, lbo, l == 0 ? 80 : 64, l < 4 ? 64 : 16);
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
                      : "memory");
       }
-      ok = __syncthreads_and(mbar_wait(mbar, phase, kWaitLimit)) != 0;
+      ok = group_and(g, mbar_wait(mbar, phase, kWaitLimit));
       phase ^= 1u;
       tc_fence_after();
       if (!ok) break;
       if (l < 4) {
         // ReLU, BF16, this row of the next tile
-        const BlockTile H{reinterpret_cast<uint32_t*>(sm + kQH), kQLboH / 4};
 #pragma unroll
         for (int c0 = 0; c0 < 64; c0 += 16) {
           float v[16];
@@ -991,21 +1040,23 @@ __global__ void __launch_bounds__(128, 2) cache_infer_tc_k(CacheNet net, CacheRo
         *dst = make_float4(v.x + b.x * y[0], v.y + b.y * y[1], v.z + b.z * y[2], v.w);
       }
     }
-    // the next tile's encoding overwrites X (read by layer 1, done) and meta
+    // the next tile's encoding overwrites the tile (read by the last layer,
+    // done) and its accumulators are read back
     tc_fence_before();
-    __syncthreads();
+    group_sync(g);
     tc_fence_after();
   }
   // MMAs in flight after a failed wait must finish before the TMEM goes back
   bool drained = ok;
   if (!ok) {
-    drained = __syncthreads_and(mbar_wait(mbar, phase ^ 1u, kWaitLimit)) != 0;
-    if (threadIdx.x == 0 && o.err) atomicOr(o.err, kErrTimeout);
+    drained = group_and(g, mbar_wait(mbar, phase ^ 1u, kWaitLimit));
+    if ((threadIdx.x & 127u) == 0u && o.err) atomicOr(o.err, kErrTimeout);
   }
   tc_fence_before();
-  __syncthreads();
-  if (warp == 0 && drained)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kQCols) : "memory");
+  drained = __syncthreads_and(drained) != 0;
+  if (threadIdx.x < 32 && drained)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(*tmem_slot), "r"(kQCols * kQGroups)
+                 : "memory");
 }
 
 // Position of FP32 master weight i in the BF16 image (out-major rows).
@@ -1131,14 +1182,14 @@ static cudaError_t launch_infer_tc(const CacheNet& net, const CacheRows& rows, c
                                    int num_sms, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(cache_infer_tc_k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemInferTc);
   if (e != cudaSuccess) return e;
-  // the smallest shared-memory carveout that holds two blocks (with the 1 KB
+  // the smallest shared-memory carveout that holds the block (with the 1 KB
   // the system reserves per block): the rest of the 256 KB stays L1
-  const int carveout = (2 * (kSmemInferTc + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024);
+  const int carveout = ((kSmemInferTc + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024);
   e = cudaFuncSetAttribute(cache_infer_tc_k, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
   if (e != cudaSuccess) return e;
   const uint32_t tiles = (n + kQRows - 1u) / kQRows;
-  const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(tiles, (uint32_t)(2 * num_sms)));
-  cache_infer_tc_k<<<grid, 128, kSmemInferTc, st>>>(net, rows, mat_a, mat_b, count_dev, n, out);
+  const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(tiles, (uint32_t)num_sms));
+  cache_infer_tc_k<<<grid, 128 * kQGroups, kSmemInferTc, st>>>(net, rows, mat_a, mat_b, count_dev, n, out);
   return cudaGetLastError();
 }
 
