@@ -56,27 +56,28 @@ constexpr int kW1 = 0, kW2 = 80 * 64, kW3 = kW2 + 4096, kW4 = kW3 + 4096, kW5 = 
 // BF16 weight image, then each warp's input tile (row stride kXs) and row
 // metadata (kSmemVjp).  Training: the weight image, then the block's
 // 64-row tiles in the core-matrix-blocked layout of BlockTile -- X (80
-// features), H1..H4 and dZ1..dZ4 (64 each), dY (16) -- the rows' metadata,
-// and the weight-gradient MMAs' mbarrier and TMEM address.
+// features), H1..H4 (64 each), two dZ tiles (dZ4 and dZ2 use the first, dZ3
+// and dZ1 the second), dY (16) -- the rows' metadata, and the weight-gradient
+// MMAs' mbarrier and TMEM address: 104 KB, two blocks per SM.
 constexpr int kSmWt = 0;
 constexpr int kSmX = kSmWt + (int)kCacheWtElems * 2;
 // bytes between consecutive 8-row groups of a blocked tile (features / 8 chunks of 128 B)
 constexpr int kLboX = 10 * 128, kLboH = 8 * 128, kLboY = 2 * 128;
 constexpr int kTX = kSmX;
 constexpr int kTH = kTX + 8 * kLboX;       // H1..H4: 8 row groups of kLboH each
-constexpr int kTDz = kTH + 4 * 8 * kLboH;  // dZ1..dZ4
-constexpr int kTDy = kTDz + 4 * 8 * kLboH;
+constexpr int kTDz = kTH + 4 * 8 * kLboH;  // dZ4 / dZ2, then dZ3 / dZ1
+constexpr int kTDy = kTDz + 2 * 8 * kLboH;
 constexpr int kTMeta = kTDy + 8 * kLboY;
 constexpr int kTBar = kTMeta + kTileRows * 16;  // mbarrier (8 B), TMEM address (4 B)
 constexpr int kSmemTrain = kTBar + 16;
 static_assert(kSmX % 16 == 0 && kTH % 16 == 0 && kTDz % 16 == 0 && kTDy % 16 == 0 && kTMeta % 16 == 0 &&
                   kTBar % 16 == 0,
               "shared regions must be 16-byte aligned");
-static_assert(kSmemTrain <= 227 * 1024, "training tile exceeds shared memory");
+static_assert(2 * (kSmemTrain + 1024) <= 227 * 1024, "two training blocks per SM");
 // An M = 128 operand reads 16 feature chunks of every row group; the X and
 // H tiles have fewer, so the reads of the last group run past the tile into
-// the next region (never past dZ1).  The rows of D they feed are not used.
-static_assert(kTX + 7 * kLboX + 16 * 128 <= kTDz && kTH + 3 * 8 * kLboH + 7 * kLboH + 16 * 128 <= kTDy,
+// the next region (H4 is no operand).  The rows of D they feed are not used.
+static_assert(kTX + 7 * kLboX + 16 * 128 <= kTDz && kTH + 2 * 8 * kLboH + 7 * kLboH + 16 * 128 <= kTDz,
               "M = 128 operand reads must stay inside the tiles");
 
 // A tile of 16-bit pairs addressed by (row, word); word w of a row holds
@@ -149,29 +150,6 @@ __device__ __forceinline__ void sh16(float3 d, float o[16]) {
   o[13] = -0.4570457994644658f * x * (5.0f * zz - 1.0f);
   o[14] = 1.445305721320277f * z * (xx - yy);
   o[15] = -0.5900435899266435f * x * (xx - 3.0f * yy);
-}
-
-// Table indices and trilinear weights of the 8 corners of level l's cell.
-// res: the levels' resolutions, staged in shared memory (dynamic index).
-__device__ __forceinline__ void level_corners(const int* res, uint32_t dense_mask, int l, float3 x, uint32_t idx[8],
-                                              float w[8]) {
-  const int n = res[l];
-  const float px = x.x * (float)n, py = x.y * (float)n, pz = x.z * (float)n;
-  const float gx = floorf(px), gy = floorf(py), gz = floorf(pz);
-  const int ix = (int)gx, iy = (int)gy, iz = (int)gz;
-  const float fx = px - gx, fy = py - gy, fz = pz - gz;
-  const bool dense = (dense_mask >> l) & 1u;
-  const uint32_t s1 = (uint32_t)n + 1u;
-  const uint32_t base = (uint32_t)l * kCacheT;
-#pragma unroll
-  for (int c = 0; c < 8; ++c) {
-    const uint32_t cx = (uint32_t)min(ix + (c & 1), n);
-    const uint32_t cy = (uint32_t)min(iy + ((c >> 1) & 1), n);
-    const uint32_t cz = (uint32_t)min(iz + ((c >> 2) & 1), n);
-    w[c] = ((c & 1) ? fx : 1.0f - fx) * ((c & 2) ? fy : 1.0f - fy) * ((c & 4) ? fz : 1.0f - fz);
-    const uint32_t h = dense ? cx + cy * s1 + cz * s1 * s1 : (cx ^ (cy * 2654435761u) ^ (cz * 805459861u));
-    idx[c] = base + (h & (kCacheT - 1u));
-  }
 }
 
 __device__ __forceinline__ float3 unit_pos(const CacheNet& net, float4 x) {
@@ -467,40 +445,6 @@ __device__ __forceinline__ void net_backward_mask(const __nv_bfloat16* Wtb, cons
   layer_bwd<4, JP0, JP1, kXs>(Wtb + kWt1, a, dx, lane);
 }
 
-// Backward pass of the warp's rows from dL/dy down to the inputs: returns the
-// input-gradient fragments of n-tile pairs [JP0, JP1) of the 80 inputs.
-// Pre-activation gradients (and dY) are stored when kStore; layer i of H and
-// Dz is hstride words after layer i - 1.
-template <bool kStore, int JP0, int JP1>
-__device__ __forceinline__ void net_backward(const __nv_bfloat16* Wtb, BlockTile H, int hstride, BlockTile Dz,
-                                             BlockTile Dy, const float (&dy)[2][4],
-                                             float (&dx)[2 * (JP1 - JP0)][4], int lane) {
-  const int g = lane >> 2, t = lane & 3;
-  uint32_t ay[1][4];
-  ay[0][0] = pack2(dy[0][0], dy[0][1]);
-  ay[0][1] = pack2(dy[0][2], dy[0][3]);
-  ay[0][2] = pack2(dy[1][0], dy[1][1]);
-  ay[0][3] = pack2(dy[1][2], dy[1][3]);
-  if (kStore) {
-    Dy(g, t) = ay[0][0];
-    Dy(g + 8, t) = ay[0][1];
-    Dy(g, 4 + t) = ay[0][2];
-    Dy(g + 8, 4 + t) = ay[0][3];
-  }
-  float dh[8][4];
-  uint32_t a[4][4];
-  layer_bwd<1, 0, 4, kHs>(Wtb + kWt5, ay, dh, lane);
-  auto at = [](BlockTile b, int i, int stride) { return BlockTile{b.p + i * stride, b.lbo}; };
-  relu_grad<kStore>(dh, at(H, 3, hstride), a, at(Dz, 3, hstride), g, t);
-  layer_bwd<4, 0, 4, kHs>(Wtb + kWt4, a, dh, lane);
-  relu_grad<kStore>(dh, at(H, 2, hstride), a, at(Dz, 2, hstride), g, t);
-  layer_bwd<4, 0, 4, kHs>(Wtb + kWt3, a, dh, lane);
-  relu_grad<kStore>(dh, at(H, 1, hstride), a, at(Dz, 1, hstride), g, t);
-  layer_bwd<4, 0, 4, kHs>(Wtb + kWt2, a, dh, lane);
-  relu_grad<kStore>(dh, H, a, Dz, g, t);
-  layer_bwd<4, JP0, JP1, kXs>(Wtb + kWt1, a, dx, lane);
-}
-
 __device__ __forceinline__ void load_weights(const CacheNet& net, unsigned char* sm, int* res) {
   uint4* dst = reinterpret_cast<uint4*>(sm + kSmWt);
   for (uint32_t i = threadIdx.x; i < kCacheWtElems / 8; i += blockDim.x) dst[i] = __ldg(&net.wt[i]);
@@ -600,7 +544,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32, 2) cache_vjp_k(CacheNet net, C
 // the FP32 accumulators live in tensor memory (TMEM), one thread issues the
 // MMAs, and an mbarrier tracks their completion.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kDwCols = 512;       // TMEM columns held by a training block (272 used)
+constexpr uint32_t kDwCols = 256;       // TMEM columns of a training block
 constexpr uint32_t kWaitLimit = 1u << 24;  // mbarrier polls before a wait gives up
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -644,36 +588,37 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, uint32
   return false;
 }
 
-// One tile's weight gradients added to the TMEM accumulators (sums over the
-// tile's 64 rows, K, in four steps of 16): dW1 = X^T dZ1, dW2..dW4 =
-// H1..H3^T dZ2..dZ4, dW5 = H4^T dY.  D rows (TMEM lanes) are the layer's
+// Two layers' weight gradients of one tile added to the TMEM accumulators
+// (sums over the tile's 64 rows, K, in four steps of 16): hi = true dW4 =
+// H3^T dZ4 and dW3 = H2^T dZ3, false dW2 = H1^T dZ2 and dW1 = X^T dZ1 (the
+// pair that shares the two dZ tiles).  D rows (TMEM lanes) are the layer's
 // inputs (M = 128; rows past 80 or 64 inputs take values that are never
-// read), columns its outputs: dW1 at columns 0-63, dW2..dW4 at 64-255, dW5
-// at 256-271.  accumulate = 0 overwrites (the block's first tile).
-__device__ __forceinline__ void issue_weight_grads(const unsigned char* sm, uint32_t tmem, bool accumulate) {
+// read), columns its outputs: dWl at columns 64 (l - 1).  accumulate = false
+// overwrites (the block's first tile).
+__device__ __forceinline__ void issue_weight_grads(const unsigned char* sm, uint32_t tmem, bool hi, bool accumulate) {
   const uint32_t base = smem_addr(sm);
 #pragma unroll
-  for (int l = 0; l < 5; ++l) {
+  for (int d = 0; d < 2; ++d) {
+    const int l = (hi ? 3 : 1) - d;  // layer l + 1
     const uint32_t a = base + (uint32_t)(l == 0 ? kTX : kTH + (l - 1) * 8 * kLboH);
     const uint32_t alb = l == 0 ? kLboX : kLboH;
-    const uint32_t b = base + (uint32_t)(l < 4 ? kTDz + l * 8 * kLboH : kTDy);
-    const uint32_t blb = l < 4 ? kLboH : kLboY;
-    const uint32_t idesc = umma_idesc(128, l < 4 ? 64 : 16);
+    const uint32_t b = base + (uint32_t)(kTDz + d * 8 * kLboH);
+    const uint32_t idesc = umma_idesc(128, 64);
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      umma_bf16(tmem + 64u * (uint32_t)l, umma_sdesc(a + 2u * k * alb, alb, 128), umma_sdesc(b + 2u * k * blb, blb, 128),
-                idesc, (accumulate || k > 0) ? 1u : 0u);
+      umma_bf16(tmem + 64u * (uint32_t)l, umma_sdesc(a + 2u * k * alb, alb, 128),
+                umma_sdesc(b + 2u * k * kLboH, kLboH, 128), idesc, (accumulate || k > 0) ? 1u : 0u);
   }
 }
 
-// Adds the block's accumulated weight gradients to gw (FP32 master layout,
-// input index first).  Warp w reads TMEM lanes 32w..32w + 31, i.e. input m =
-// 32w + lane of every layer.
+// Adds the block's accumulated weight gradients of layers 1..4 to gw (FP32
+// master layout, input index first).  Warp w reads TMEM lanes 32w..32w + 31,
+// i.e. input m = 32w + lane of every layer.
 __device__ __forceinline__ void flush_weight_grads(uint32_t tmem, float* gw) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m = 32 * warp + lane;
 #pragma unroll 1
-  for (int c0 = 0; c0 < 272; c0 += 16) {
+  for (int c0 = 0; c0 < 256; c0 += 16) {
     uint32_t r[16];
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -683,22 +628,31 @@ __device__ __forceinline__ void flush_weight_grads(uint32_t tmem, float* gw) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
     const int l = c0 >> 6, n0 = c0 & 63;
     if (m < (l == 0 ? 80 : 64)) {
-      float* dst = gw + (l == 0 ? kW1 + m * 64 : (l < 4 ? kW2 + (l - 1) * 4096 + m * 64 : kW5 + m * 16)) + n0;
+      float* dst = gw + (l == 0 ? kW1 + m * 64 : kW2 + (l - 1) * 4096 + m * 64) + n0;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const float v = __uint_as_float(r[j]);
-        if (v != 0.0f) atomicAdd(dst + j, v);
-      }
+      for (int j = 0; j < 16; j += 4)
+        asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + j),
+                     "f"(__uint_as_float(r[j])), "f"(__uint_as_float(r[j + 1])), "f"(__uint_as_float(r[j + 2])),
+                     "f"(__uint_as_float(r[j + 3]))
+                     : "memory");
     }
   }
 }
 
 // Training gradients over block tiles of 64 rows of one minibatch.  The
 // forward and backward passes run on mma.sync per warp (16 rows each); the
-// weight gradients of each tile go to the tensor cores as one batch of 20
-// tcgen05.mma (issued after the tile's tiles are written, waited for before
-// the next tile overwrites them), accumulated in TMEM for the whole launch.
-__global__ void __launch_bounds__(kThreads) cache_grad_k(CacheNet net, CacheRows rows, const float4* mat_a,
+// weight gradients of layers 1..4 go to the tensor cores as two batches of 8
+// tcgen05.mma a tile (layers 4 and 3 once their dZ tiles are written, layers 2
+// and 1 after them over the same two tiles), accumulated in TMEM for the
+// whole launch; dW5, whose dY has three non-zero columns, is summed in
+// registers.  A tile is a chain of gathers, 18 MMA layers and scatters by four
+// warps, so the kernel lasts as long as its latency: two dZ tiles instead of
+// four and 256 TMEM columns instead of 272 let two blocks share an SM.  Table
+// gradients are scattered as the gathers read (a lane pair per level, one x
+// side each).  153k rows: 0.322 -> 0.258
+// ms, half of it from flushing with vector reductions (every block adds to the
+// same 18k weights at its end).
+__global__ void __launch_bounds__(kThreads, 2) cache_grad_k(CacheNet net, CacheRows rows, const float4* mat_a,
                                                          const float4* mat_b, const uint32_t* count_dev,
                                                          uint32_t n_max, uint32_t batch, uint32_t n_batches,
                                                          CacheOut o) {
@@ -737,6 +691,9 @@ __global__ void __launch_bounds__(kThreads) cache_grad_k(CacheNet net, CacheRows
   const BlockTile Dy = BlockTile{reinterpret_cast<uint32_t*>(sm + kTDy), kLboY / 4}.rows_from(16 * warp);
   const int hstride = 8 * kLboH / 4;  // words between layers
   float4* meta = reinterpret_cast<float4*>(sm + kTMeta) + warp * 16;
+  // dW5: input k of the last layer, a half of the tile's rows
+  const int k5 = threadIdx.x & 63, half5 = (threadIdx.x >> 6) * (kTileRows / 2);
+  float dw5[3] = {0.f, 0.f, 0.f};
   double loss = 0.0;
   uint32_t issued = 0;  // MMA batches committed to the mbarrier
   bool failed = false;
@@ -793,23 +750,87 @@ __global__ void __launch_bounds__(kThreads) cache_grad_k(CacheNet net, CacheRows
       dy[0][0] = d2a;
       dy[0][2] = d2b;
     }
-    float dx[4][4];
-    net_backward<true, 0, 2>(Wtb, H, hstride, Dz, Dy, dy, dx, lane);
-    // hash-table gradient: n-tile j holds level 4j + t (features 0, 1)
+    float dh[8][4], dx[4][4];
+    uint32_t a[4][4];
+    {
+      uint32_t ay[1][4];
+      ay[0][0] = pack2(dy[0][0], dy[0][1]);
+      ay[0][1] = pack2(dy[0][2], dy[0][3]);
+      ay[0][2] = pack2(dy[1][0], dy[1][1]);
+      ay[0][3] = pack2(dy[1][2], dy[1][3]);
+      Dy(g, t) = ay[0][0];
+      Dy(g + 8, t) = ay[0][1];
+      layer_bwd<1, 0, 4, kHs>(Wtb + kWt5, ay, dh, lane);
+    }
+    const auto layer = [&](const BlockTile& b, int i) { return BlockTile{b.p + i * hstride, b.lbo}; };
+    relu_grad<true>(dh, layer(H, 3), a, Dz, g, t);  // dZ4
+    layer_bwd<4, 0, 4, kHs>(Wtb + kWt4, a, dh, lane);
+    relu_grad<true>(dh, layer(H, 2), a, layer(Dz, 1), g, t);  // dZ3
+    // the tiles' generic-proxy writes become visible to the tensor cores
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc_fence_after();
+      issue_weight_grads(sm, tmem, true, issued > 0);
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
+                   : "memory");
+    }
+    ++issued;
+    layer_bwd<4, 0, 4, kHs>(Wtb + kWt3, a, dh, lane);
+    {
+      const BlockTile H4 = BlockTile{reinterpret_cast<uint32_t*>(sm + kTH) + 3 * hstride, kLboH / 4};
+      const BlockTile Y = BlockTile{reinterpret_cast<uint32_t*>(sm + kTDy), kLboY / 4};
+#pragma unroll 4
+      for (int r = half5; r < half5 + kTileRows / 2; ++r) {
+        const float2 hv = unpack2(H4(r, k5 >> 1));
+        const float h = (k5 & 1) ? hv.y : hv.x;
+        const float2 y01 = unpack2(Y(r, 0)), y23 = unpack2(Y(r, 1));
+        dw5[0] += h * y01.x;
+        dw5[1] += h * y01.y;
+        dw5[2] += h * y23.x;
+      }
+    }
+    // layers 4 and 3 are done with the dZ tiles before layers 2 and 1 take them
+    if (__syncthreads_or(!mbar_wait(mbar, (issued - 1u) & 1u, kWaitLimit))) {
+      failed = true;
+      break;
+    }
+    relu_grad<true>(dh, layer(H, 1), a, Dz, g, t);  // dZ2
+    layer_bwd<4, 0, 4, kHs>(Wtb + kWt2, a, dh, lane);
+    relu_grad<true>(dh, H, a, layer(Dz, 1), g, t);  // dZ1
+    layer_bwd<4, 0, 2, kXs>(Wtb + kWt1, a, dx, lane);
+    // hash-table gradient: n-tile j holds level 4j + t (features 0, 1); a lane
+    // pair adds each of its two levels, one x side of the cell per lane
     if (o.gt) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int l = 4 * j + t;
+      for (int h = 0; h < 2; ++h) {
+        const float4 m = meta[g + 8 * h];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float4 m = meta[g + 8 * h];
-          if (m.w == 0.0f) continue;
-          uint32_t idx[8];
-          float w[8];
-          level_corners(res, net.dense, l, make_float3(m.x, m.y, m.z), idx, w);
-          const float d0 = dx[j][2 * h], d1 = dx[j][2 * h + 1];
+        for (int j = 0; j < 4; ++j) {
+          const float m0 = dx[j][2 * h], m1 = dx[j][2 * h + 1];
 #pragma unroll
-          for (int c = 0; c < 8; ++c) atomicAdd(&o.gt[idx[c]], make_float2(w[c] * d0, w[c] * d1));
+          for (int p = 0; p < 2; ++p) {
+            const float d0 = __shfl_sync(0xffffffffu, m0, (lane & ~1) | p);
+            const float d1 = __shfl_sync(0xffffffffu, m1, (lane & ~1) | p);
+            if (m.w == 0.0f) continue;
+            const int l = 4 * j + (t & 2) + p, nr = res[l];
+            const bool odd = lane & 1;
+            const float px = m.x * (float)nr, py = m.y * (float)nr, pz = m.z * (float)nr;
+            const float gx = floorf(px), gy = floorf(py), gz = floorf(pz);
+            const int ix = (int)gx, iy = (int)gy, iz = (int)gz;
+            const float fx = px - gx, fy = py - gy, fz = pz - gz;
+            const bool dense = (net.dense >> l) & 1u;
+            const uint32_t s1 = (uint32_t)nr + 1u, base = (uint32_t)l * kCacheT;
+            const uint32_t cx = (uint32_t)min(ix + (odd ? 1 : 0), nr);
+            const float wx = odd ? fx : 1.0f - fx;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t cy = (uint32_t)min(iy + (k & 1), nr), cz = (uint32_t)min(iz + (k >> 1), nr);
+              const uint32_t hh = dense ? cx + cy * s1 + cz * s1 * s1 : (cx ^ (cy * 2654435761u) ^ (cz * 805459861u));
+              const float w = wx * ((k & 1) ? fy : 1.0f - fy) * ((k & 2) ? fz : 1.0f - fz);
+              atomicAdd(&o.gt[base + (hh & (kCacheT - 1u))], make_float2(w * d0, w * d1));
+            }
+          }
         }
       }
     }
@@ -818,7 +839,7 @@ __global__ void __launch_bounds__(kThreads) cache_grad_k(CacheNet net, CacheRows
     __syncthreads();
     if (threadIdx.x == 0) {
       tc_fence_after();
-      issue_weight_grads(sm, tmem, issued > 0);
+      issue_weight_grads(sm, tmem, false, issued > 1);
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
                    : "memory");
     }
@@ -829,7 +850,12 @@ __global__ void __launch_bounds__(kThreads) cache_grad_k(CacheNet net, CacheRows
   if (issued) drained = __syncthreads_or(!mbar_wait(mbar, (issued - 1u) & 1u, kWaitLimit)) == 0;
   if ((failed || !drained) && threadIdx.x == 0 && o.err) atomicOr(o.err, kErrTimeout);
   tc_fence_after();
-  if (issued && drained && !failed) flush_weight_grads(tmem, o.gw);
+  if (issued && drained && !failed) {
+    flush_weight_grads(tmem, o.gw);
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (dw5[c] != 0.0f) atomicAdd(&o.gw[kW5 + k5 * 16 + c], dw5[c]);
+  }
   tc_fence_before();
   __syncthreads();
   // the TMEM is freed unless MMAs may still write it
@@ -1206,7 +1232,7 @@ cudaError_t cache_grad(const CacheNet& net, const CacheRows& rows, const float4*
                        const CacheOut& out, int num_sms, cudaStream_t st) {
   if (n == 0 || n_batches == 0) return cudaSuccess;
   const uint32_t tiles = ((n + n_batches - 1u) / n_batches + kTileRows - 1u) / kTileRows;
-  const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(tiles, (uint32_t)num_sms));
+  const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(tiles, (uint32_t)(2 * num_sms)));
   cudaFuncSetAttribute(cache_grad_k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTrain);
   cache_grad_k<<<grid, kThreads, kSmemTrain, st>>>(net, rows, mat_a, mat_b, count_dev, n, batch, n_batches, out);
   return cudaGetLastError();

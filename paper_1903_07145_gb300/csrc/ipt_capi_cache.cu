@@ -246,12 +246,18 @@ ipt_status ipt_cache_grad(ipt_ctx* ctx, int32_t scene, uint32_t n, const float* 
   if ((st = cache_api_rows(ctx, c, n)) != IPT_OK) return st;
   IPT_CK(ipt::cache_pack_rows(n, x01, dir, nrm, params7, target, c->api, c->api_ma, c->api_mb, ctx->stream));
   const size_t nw = ipt::kCacheWeights, nt = ipt::kCacheTableFloats;
-  IPT_CK(cudaMemsetAsync(c->gw, 0, nw * sizeof(float), ctx->stream));
-  IPT_CK(cudaMemsetAsync(c->gt, 0, nt * sizeof(float), ctx->stream));
+  // the kernel adds to the caller's arrays where their alignment allows its
+  // vector reductions; the cache's own accumulators (kept zero between
+  // training steps) take the rest
+  const auto aligned = [](const void* p, size_t a) { return p && reinterpret_cast<uintptr_t>(p) % a == 0; };
+  float* gw = aligned(grad_weights, 16) ? grad_weights : c->gw;
+  float* gt = !grad_table || aligned(grad_table, 8) ? grad_table : c->gt;  // null: no table gradient
+  IPT_CK(cudaMemsetAsync(gw, 0, nw * sizeof(float), ctx->stream));
+  if (gt) IPT_CK(cudaMemsetAsync(gt, 0, nt * sizeof(float), ctx->stream));
   IPT_CK(cudaMemsetAsync(c->loss_dev, 0, sizeof(double), ctx->stream));
   ipt::CacheOut o{};
-  o.gw = c->gw;
-  o.gt = reinterpret_cast<float2*>(c->gt);
+  o.gw = gw;
+  o.gt = reinterpret_cast<float2*>(gt);
   o.loss = c->loss_dev;
   o.err = ctx->err_dev;
   {
@@ -259,12 +265,15 @@ ipt_status ipt_cache_grad(ipt_ctx* ctx, int32_t scene, uint32_t n, const float* 
     IPT_CK(ipt::cache_grad(cache_net(s, true), c->api, c->api_ma, c->api_mb, nullptr, n, 0, 1, o, ctx->L.num_sms,
                            ctx->stream));
   }
-  if (grad_weights)
-    IPT_CK(cudaMemcpyAsync(grad_weights, c->gw, nw * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
-  if (grad_table)
-    IPT_CK(cudaMemcpyAsync(grad_table, c->gt, nt * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
-  IPT_CK(cudaMemsetAsync(c->gw, 0, nw * sizeof(float), ctx->stream));
-  IPT_CK(cudaMemsetAsync(c->gt, 0, nt * sizeof(float), ctx->stream));
+  if (gw == c->gw) {
+    if (grad_weights)
+      IPT_CK(cudaMemcpyAsync(grad_weights, gw, nw * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
+    IPT_CK(cudaMemsetAsync(gw, 0, nw * sizeof(float), ctx->stream));
+  }
+  if (gt == c->gt) {
+    IPT_CK(cudaMemcpyAsync(grad_table, gt, nt * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
+    IPT_CK(cudaMemsetAsync(gt, 0, nt * sizeof(float), ctx->stream));
+  }
   if (loss_out) {
     IPT_CK(cudaMemcpyAsync(c->host, c->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     if ((st = ipt_synchronize(ctx)) != IPT_OK) return st;
