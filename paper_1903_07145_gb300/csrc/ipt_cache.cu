@@ -158,6 +158,41 @@ __device__ __forceinline__ float3 unit_pos(const CacheNet& net, float4 x) {
                      fminf(fmaxf((x.z - net.lo.z) * net.inv_ext.z, 0.0f), 1.0f));
 }
 
+// Where a kernel's rows come from.  PackedRows: the wavefront's queries and
+// records (materials by segment).  RawRows: the caller's arrays of the
+// evaluation entry points (packing them first, and unpacking the results,
+// took 29 us of 289 for 500k rows).
+struct PackedRows {
+  CacheRows r;
+  const float4 *mat_a, *mat_b;
+  __device__ __forceinline__ void position(uint32_t i, float4& x, float4& ma, float4& mb) const {
+    x = r.x[i];
+    const int seg = __float_as_int(x.w);
+    ma = __ldg(&mat_a[seg]);
+    mb = __ldg(&mat_b[seg]);
+  }
+  __device__ __forceinline__ float4 direction(uint32_t i) const { return r.d[i]; }
+  __device__ __forceinline__ float4 normal(uint32_t i) const { return r.n[i]; }
+  __device__ __forceinline__ float4 u(uint32_t i) const { return r.u[i]; }
+};
+
+struct RawRows {
+  CacheRaw r;
+  static __device__ __forceinline__ float4 row3(const float* p, uint32_t i) {
+    p += 3 * (size_t)i;
+    return make_float4(p[0], p[1], p[2], 0.0f);
+  }
+  __device__ __forceinline__ void position(uint32_t i, float4& x, float4& ma, float4& mb) const {
+    x = row3(r.x, i);
+    const float* q = r.p7 + 7 * (size_t)i;
+    ma = make_float4(q[0], q[1], q[2], q[6]);
+    mb = make_float4(q[3], q[4], q[5], 0.0f);
+  }
+  __device__ __forceinline__ float4 direction(uint32_t i) const { return row3(r.d, i); }
+  __device__ __forceinline__ float4 normal(uint32_t i) const { return row3(r.n, i); }
+  __device__ __forceinline__ float4 u(uint32_t i) const { return row3(r.u, i); }
+};
+
 // Encodes rows [r0, r0 + 16) (valid below `end`) into the warp's input tile
 // X (16 rows of 80 BF16 features) and its row metadata (unit position, valid
 // flag).
@@ -165,22 +200,17 @@ __device__ __forceinline__ float3 unit_pos(const CacheNet& net, float4 x) {
 // table's FP16 copy (queries) instead of the FP32 master (training and the
 // input VJP, whose result depends on the table only through the ReLU
 // decisions, which the FP16 rounding would move near their kinks).
-template <bool kHalf, int kUnroll, class Tile>
-__device__ __forceinline__ void encode_rows(const CacheNet& net, const int* res, const CacheRows& rows, const float4* mat_a,
-                            const float4* mat_b, uint32_t r0, uint32_t end, Tile X, float4* meta, int lane) {
+template <bool kHalf, int kUnroll, class Rows, class Tile>
+__device__ __forceinline__ void encode_rows(const CacheNet& net, const int* res, const Rows& rows, uint32_t r0,
+                                            uint32_t end, Tile X, float4* meta, int lane) {
   const int row = lane & 15;
   const uint32_t r = r0 + (uint32_t)row;
   const bool valid = r < end;
   if (lane < 16) {
-    const float4 xq = valid ? rows.x[r] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 xq = make_float4(0.f, 0.f, 0.f, 0.f), ma = xq, mb = xq;
+    if (valid) rows.position(r, xq, ma, mb);
     const float3 p = unit_pos(net, xq);
     meta[row] = make_float4(p.x, p.y, p.z, valid ? 1.0f : 0.0f);
-    float4 ma = make_float4(0.f, 0.f, 0.f, 0.f), mb = ma;
-    if (valid) {
-      const int seg = __float_as_int(xq.w);
-      ma = __ldg(&mat_a[seg]);
-      mb = __ldg(&mat_b[seg]);
-    }
     X(row, 32) = pack2(ma.x, ma.y);  // kd r, g
     X(row, 33) = pack2(ma.z, mb.x);  // kd b, ks r
     X(row, 34) = pack2(mb.y, mb.z);  // ks g, b
@@ -191,7 +221,7 @@ __device__ __forceinline__ void encode_rows(const CacheNet& net, const int* res,
   {
     float3 dir = make_float3(0.f, 0.f, 1.f);
     if (valid) {
-      const float4 v = lane < 16 ? rows.d[r] : rows.n[r];
+      const float4 v = lane < 16 ? rows.direction(r) : rows.normal(r);
       dir = make_float3(v.x, v.y, v.z);
     }
     float sh[16];
@@ -454,6 +484,23 @@ __device__ __forceinline__ void load_weights(const CacheNet& net, unsigned char*
   }
 }
 
+// A row's prediction to the outputs that take it.
+template <class Rows>
+__device__ __forceinline__ void store_prediction(const CacheOut& o, const Rows& rows, uint32_t i, float3 C) {
+  if (o.c) o.c[i] = make_float4(C.x, C.y, C.z, 0.0f);
+  if (o.rgb) {
+    o.rgb[3 * (size_t)i] = C.x;
+    o.rgb[3 * (size_t)i + 1] = C.y;
+    o.rgb[3 * (size_t)i + 2] = C.z;
+  }
+  if (o.rad) {
+    const float4 b = rows.u(i);
+    float4* dst = &o.rad[__float_as_uint(rows.direction(i).w)];
+    const float4 v = *dst;
+    *dst = make_float4(v.x + b.x * C.x, v.y + b.y * C.y, v.z + b.z * C.z, v.w);
+  }
+}
+
 // Input VJP (with the query's outputs) over warp tiles of 16 rows; the warps
 // share one shared-memory weight image.  The hidden layers' ReLU masks stay
 // in registers, so a block holds only the weights and its warps' input
@@ -463,9 +510,9 @@ constexpr int kVjpWarps = 12;
 constexpr int kSmemVjp = kSmX + kVjpWarps * 16 * kXs * 2 + kVjpWarps * 16 * 16;
 static_assert(kSmX % 16 == 0 && (kSmX + kVjpWarps * 16 * kXs * 2) % 16 == 0, "VJP tiles must be aligned");
 
-__global__ void __launch_bounds__(kVjpWarps * 32, 2) cache_vjp_k(CacheNet net, CacheRows rows, const float4* mat_a,
-                                                         const float4* mat_b, const uint32_t* count_dev,
-                                                         uint32_t n_max, CacheOut o) {
+template <class Rows>
+__global__ void __launch_bounds__(kVjpWarps * 32, 2)
+    cache_vjp_k(CacheNet net, Rows rows, const uint32_t* count_dev, uint32_t n_max, CacheOut o) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int res[kCacheLevels];
   load_weights(net, sm, res);
@@ -482,7 +529,7 @@ __global__ void __launch_bounds__(kVjpWarps * 32, 2) cache_vjp_k(CacheNet net, C
        tile += gridDim.x * (uint32_t)kVjpWarps) {
     const uint32_t r0 = tile * 16u;
     __syncwarp();
-    encode_rows<false, 2>(net, res, rows, mat_a, mat_b, r0, n, X, meta, lane);
+    encode_rows<false, 2>(net, res, rows, r0, n, X, meta, lane);
     float y[2][4];
     uint32_t mask[4];
     net_forward_mask(Wt, X, y, mask, lane);
@@ -490,49 +537,39 @@ __global__ void __launch_bounds__(kVjpWarps * 32, 2) cache_vjp_k(CacheNet net, C
     const float y2a = __shfl_down_sync(0xffffffffu, y[0][0], 1);
     const float y2b = __shfl_down_sync(0xffffffffu, y[0][2], 1);
     const uint32_t ra = r0 + (uint32_t)g, rb = ra + 8u;
-    if (t == 0) {
+    // upstream u on outputs 0..2: lane t = 0 takes (u.x, u.y), t = 1 (u.z, 0)
+    float dy[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    if (t < 2) {
       if (ra < n) {
-        const float3 C = make_float3(y[0][0], y[0][1], y2a);
-        if (o.c) o.c[ra] = make_float4(C.x, C.y, C.z, 0.0f);
-        if (o.rad) {
-          const float4 b = rows.u[ra];
-          float4* dst = &o.rad[__float_as_uint(rows.d[ra].w)];
-          const float4 v = *dst;
-          *dst = make_float4(v.x + b.x * C.x, v.y + b.y * C.y, v.z + b.z * C.z, v.w);
-        }
+        const float4 u = rows.u(ra);
+        dy[0][0] = t == 0 ? u.x : u.z;
+        dy[0][1] = t == 0 ? u.y : 0.0f;
       }
       if (rb < n) {
-        const float3 C = make_float3(y[0][2], y[0][3], y2b);
-        if (o.c) o.c[rb] = make_float4(C.x, C.y, C.z, 0.0f);
-        if (o.rad) {
-          const float4 b = rows.u[rb];
-          float4* dst = &o.rad[__float_as_uint(rows.d[rb].w)];
-          const float4 v = *dst;
-          *dst = make_float4(v.x + b.x * C.x, v.y + b.y * C.y, v.z + b.z * C.z, v.w);
-        }
+        const float4 u = rows.u(rb);
+        dy[0][2] = t == 0 ? u.x : u.z;
+        dy[0][3] = t == 0 ? u.y : 0.0f;
       }
     }
+    if (t == 0) {
+      if (ra < n) store_prediction(o, rows, ra, make_float3(y[0][0], y[0][1], y2a));
+      if (rb < n) store_prediction(o, rows, rb, make_float3(y[0][2], y[0][3], y2b));
+    }
     {
-      // upstream u on outputs 0..2: lane t = 0 takes (u.x, u.y), t = 1 (u.z, 0)
-      float dy[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-      if (t < 2) {
-        if (ra < n) {
-          const float4 u = rows.u[ra];
-          dy[0][0] = t == 0 ? u.x : u.z;
-          dy[0][1] = t == 0 ? u.y : 0.0f;
-        }
-        if (rb < n) {
-          const float4 u = rows.u[rb];
-          dy[0][2] = t == 0 ? u.x : u.z;
-          dy[0][3] = t == 0 ? u.y : 0.0f;
-        }
-      }
       float dx[2][4];
       net_backward_mask<4, 5>(Wtb, mask, dy, dx, lane);
       // n-tile 8 = inputs 64..71: kd rgb, ks rgb, roughness, pad
       if (o.dp) {
         if (ra < n) *reinterpret_cast<float2*>(&o.dp[8 * (size_t)ra + 2 * t]) = make_float2(dx[0][0], dx[0][1]);
         if (rb < n) *reinterpret_cast<float2*>(&o.dp[8 * (size_t)rb + 2 * t]) = make_float2(dx[0][2], dx[0][3]);
+      }
+      if (o.dp7) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (2 * t + k == 7) break;
+          if (ra < n) o.dp7[7 * (size_t)ra + 2 * t + k] = dx[0][k];
+          if (rb < n) o.dp7[7 * (size_t)rb + 2 * t + k] = dx[0][2 + k];
+        }
       }
     }
   }
@@ -652,10 +689,10 @@ __device__ __forceinline__ void flush_weight_grads(uint32_t tmem, float* gw) {
 // side each).  153k rows: 0.322 -> 0.258
 // ms, half of it from flushing with vector reductions (every block adds to the
 // same 18k weights at its end).
-__global__ void __launch_bounds__(kThreads, 2) cache_grad_k(CacheNet net, CacheRows rows, const float4* mat_a,
-                                                         const float4* mat_b, const uint32_t* count_dev,
-                                                         uint32_t n_max, uint32_t batch, uint32_t n_batches,
-                                                         CacheOut o) {
+template <class Rows>
+__global__ void __launch_bounds__(kThreads, 2)
+    cache_grad_k(CacheNet net, Rows rows, const uint32_t* count_dev, uint32_t n_max, uint32_t batch,
+                 uint32_t n_batches, CacheOut o) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int res[kCacheLevels];
   load_weights(net, sm, res);
@@ -708,7 +745,7 @@ __global__ void __launch_bounds__(kThreads, 2) cache_grad_k(CacheNet net, CacheR
       }
     }
     const uint32_t r0 = begin + tile * kTileRows + 16u * (uint32_t)warp;
-    encode_rows<false, 2>(net, res, rows, mat_a, mat_b, r0, end, X, meta, lane);
+    encode_rows<false, 2>(net, res, rows, r0, end, X, meta, lane);
     float y[2][4];
     net_forward<true>(Wt, X, H, hstride, y, lane);
     // relative L2: d/dy_c of (y_c - t_c)^2 / (sg(y_c)^2 + 0.01), mean over rows and channels
@@ -718,7 +755,7 @@ __global__ void __launch_bounds__(kThreads, 2) cache_grad_k(CacheNet net, CacheR
     float da[3] = {0.f, 0.f, 0.f}, db[3] = {0.f, 0.f, 0.f};
     if (t == 0) {
       if (ra < end) {
-        const float4 tg = rows.u[ra];
+        const float4 tg = rows.u(ra);
         const float yy[3] = {y[0][0], y[0][1], y2a}, tt[3] = {tg.x, tg.y, tg.z};
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -728,7 +765,7 @@ __global__ void __launch_bounds__(kThreads, 2) cache_grad_k(CacheNet net, CacheR
         }
       }
       if (rb < end) {
-        const float4 tg = rows.u[rb];
+        const float4 tg = rows.u(rb);
         const float yy[3] = {y[0][2], y[0][3], y2b}, tt[3] = {tg.x, tg.y, tg.z};
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -972,9 +1009,9 @@ __device__ __forceinline__ bool group_and(int g, bool p) {
   return r != 0u;
 }
 
+template <class Rows>
 __global__ void __launch_bounds__(128 * kQGroups, 1)
-    cache_infer_tc_k(CacheNet net, CacheRows rows, const float4* mat_a, const float4* mat_b,
-                     const uint32_t* count_dev, uint32_t n_max, CacheOut o) {
+    cache_infer_tc_k(CacheNet net, Rows rows, const uint32_t* count_dev, uint32_t n_max, CacheOut o) {
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int res[kCacheLevels];
   load_weights_blocked(net, sm, res);
@@ -1010,8 +1047,8 @@ __global__ void __launch_bounds__(128 * kQGroups, 1)
   // a launch of few tiles takes the blocks' first groups first
   for (uint32_t tile = blockIdx.x + gridDim.x * (uint32_t)g; tile < n_tiles && ok; tile += gridDim.x * kQGroups) {
     const uint32_t r0 = tile * kQRows;
-    encode_rows<true, 4>(net, res, rows, mat_a, mat_b, r0 + 32u * warp, n, X.rows_from(32 * warp), meta + 32 * warp, lane);
-    encode_rows<true, 4>(net, res, rows, mat_a, mat_b, r0 + 32u * warp + 16u, n, X.rows_from(32 * warp + 16),
+    encode_rows<true, 4>(net, res, rows, r0 + 32u * warp, n, X.rows_from(32 * warp), meta + 32 * warp, lane);
+    encode_rows<true, 4>(net, res, rows, r0 + 32u * warp + 16u, n, X.rows_from(32 * warp + 16),
                          meta + 32 * warp + 16, lane);
     float y[3] = {0.f, 0.f, 0.f};
 #pragma unroll 1
@@ -1057,15 +1094,7 @@ __global__ void __launch_bounds__(128 * kQGroups, 1)
     }
     if (!ok) break;
     const uint32_t r = r0 + (uint32_t)row;
-    if (r < n) {
-      if (o.c) o.c[r] = make_float4(y[0], y[1], y[2], 0.0f);
-      if (o.rad) {
-        const float4 b = rows.u[r];
-        float4* dst = &o.rad[__float_as_uint(rows.d[r].w)];
-        const float4 v = *dst;
-        *dst = make_float4(v.x + b.x * y[0], v.y + b.y * y[1], v.z + b.z * y[2], v.w);
-      }
-    }
+    if (r < n) store_prediction(o, rows, r, make_float3(y[0], y[1], y[2]));
     // the next tile's encoding overwrites the tile (read by the last layer,
     // done) and its accumulators are read back
     tc_fence_before();
@@ -1134,32 +1163,6 @@ __global__ void cache_pack_k(const float* w, __nv_bfloat16* wt) {
     wt[image_index((int)i)] = __float2bfloat16_rn(w[i]);
 }
 
-__global__ void cache_pack_rows_k(uint32_t n, const float* x01, const float* dir, const float* nrm,
-                                  const float* p7, const float* u, CacheRows rows, float4* mat_a, float4* mat_b) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    rows.x[i] = make_float4(x01[3 * i], x01[3 * i + 1], x01[3 * i + 2], __int_as_float((int)i));
-    rows.d[i] = make_float4(dir[3 * i], dir[3 * i + 1], dir[3 * i + 2], __uint_as_float(i));
-    rows.n[i] = make_float4(nrm[3 * i], nrm[3 * i + 1], nrm[3 * i + 2], 0.0f);
-    rows.u[i] = u ? make_float4(u[3 * i], u[3 * i + 1], u[3 * i + 2], 0.0f) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float* q = p7 + 7 * (size_t)i;
-    mat_a[i] = make_float4(q[0], q[1], q[2], q[6]);
-    mat_b[i] = make_float4(q[3], q[4], q[5], 0.0f);
-  }
-}
-
-__global__ void cache_unpack_k(uint32_t n, const float4* c, const float* dp, float* rgb, float* dparams) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    if (rgb) {
-      const float4 v = c[i];
-      rgb[3 * i] = v.x;
-      rgb[3 * i + 1] = v.y;
-      rgb[3 * i + 2] = v.z;
-    }
-    if (dparams)
-      for (int k = 0; k < 7; ++k) dparams[7 * (size_t)i + k] = dp[8 * (size_t)i + k];
-  }
-}
-
 __global__ void cache_targets_k(CacheBuffers b, const float4* rad) {
   const uint32_t lo = b.counts[2], hi = min(b.counts[1], b.r_cap);
   for (uint32_t i = lo + blockIdx.x * blockDim.x + threadIdx.x; i < hi; i += gridDim.x * blockDim.x) {
@@ -1185,37 +1188,43 @@ void cache_grid(int res[kCacheLevels], uint32_t* dense) {
   }
 }
 
-static cudaError_t launch_vjp(const CacheNet& net, const CacheRows& rows, const float4* mat_a, const float4* mat_b,
-                              const uint32_t* count_dev, uint32_t n, const CacheOut& out, int num_sms,
-                              cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(cache_vjp_k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemVjp);
+template <class Rows>
+static cudaError_t launch_vjp(const CacheNet& net, const Rows& rows, const uint32_t* count_dev, uint32_t n,
+                              const CacheOut& out, int num_sms, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(cache_vjp_k<Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemVjp);
   if (e != cudaSuccess) return e;
-  static int per_sm = 0;  // resident blocks per SM at this shared-memory size (the same on every GB300)
-  if (per_sm == 0) {
-    int b = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, cache_vjp_k, kVjpWarps * 32, kSmemVjp);
-    if (e != cudaSuccess) return e;
-    per_sm = b < 1 ? 1 : b;
-  }
+  // two resident blocks per SM, as the kernel's launch bounds ask
   const uint32_t tiles = (n + 16u * kVjpWarps - 1u) / (16u * kVjpWarps);
-  const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(tiles, (uint32_t)(num_sms * per_sm)));
-  cache_vjp_k<<<grid, kVjpWarps * 32, kSmemVjp, st>>>(net, rows, mat_a, mat_b, count_dev, n, out);
+  const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(tiles, (uint32_t)(2 * num_sms)));
+  cache_vjp_k<<<grid, kVjpWarps * 32, kSmemVjp, st>>>(net, rows, count_dev, n, out);
   return cudaGetLastError();
 }
 
-static cudaError_t launch_infer_tc(const CacheNet& net, const CacheRows& rows, const float4* mat_a,
-                                   const float4* mat_b, const uint32_t* count_dev, uint32_t n, const CacheOut& out,
-                                   int num_sms, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(cache_infer_tc_k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemInferTc);
+template <class Rows>
+static cudaError_t launch_infer_tc(const CacheNet& net, const Rows& rows, const uint32_t* count_dev, uint32_t n,
+                                   const CacheOut& out, int num_sms, cudaStream_t st) {
+  cudaError_t e =
+      cudaFuncSetAttribute(cache_infer_tc_k<Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemInferTc);
   if (e != cudaSuccess) return e;
   // the smallest shared-memory carveout that holds the block (with the 1 KB
   // the system reserves per block): the rest of the 256 KB stays L1
   const int carveout = ((kSmemInferTc + 1024) * 100 + 228 * 1024 - 1) / (228 * 1024);
-  e = cudaFuncSetAttribute(cache_infer_tc_k, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
+  e = cudaFuncSetAttribute(cache_infer_tc_k<Rows>, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
   if (e != cudaSuccess) return e;
   const uint32_t tiles = (n + kQRows - 1u) / kQRows;
   const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(tiles, (uint32_t)num_sms));
-  cache_infer_tc_k<<<grid, 128 * kQGroups, kSmemInferTc, st>>>(net, rows, mat_a, mat_b, count_dev, n, out);
+  cache_infer_tc_k<<<grid, 128 * kQGroups, kSmemInferTc, st>>>(net, rows, count_dev, n, out);
+  return cudaGetLastError();
+}
+
+template <class Rows>
+static cudaError_t launch_grad(const CacheNet& net, const Rows& rows, const uint32_t* count_dev, uint32_t n,
+                               uint32_t batch, uint32_t n_batches, const CacheOut& out, int num_sms, cudaStream_t st) {
+  if (n == 0 || n_batches == 0) return cudaSuccess;
+  const uint32_t tiles = ((n + n_batches - 1u) / n_batches + kTileRows - 1u) / kTileRows;
+  const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(tiles, (uint32_t)(2 * num_sms)));
+  cudaFuncSetAttribute(cache_grad_k<Rows>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTrain);
+  cache_grad_k<<<grid, kThreads, kSmemTrain, st>>>(net, rows, count_dev, n, batch, n_batches, out);
   return cudaGetLastError();
 }
 
@@ -1223,19 +1232,26 @@ cudaError_t cache_infer(const CacheNet& net, const CacheRows& rows, const float4
                         const uint32_t* count_dev, uint32_t n, const CacheOut& out, bool vjp, int num_sms,
                         cudaStream_t st) {
   if (n == 0) return cudaSuccess;
-  if (vjp) return launch_vjp(net, rows, mat_a, mat_b, count_dev, n, out, num_sms, st);
-  return launch_infer_tc(net, rows, mat_a, mat_b, count_dev, n, out, num_sms, st);
+  const PackedRows r{rows, mat_a, mat_b};
+  return vjp ? launch_vjp(net, r, count_dev, n, out, num_sms, st) : launch_infer_tc(net, r, count_dev, n, out, num_sms, st);
+}
+
+cudaError_t cache_infer_raw(const CacheNet& net, const CacheRaw& rows, uint32_t n, const CacheOut& out, bool vjp,
+                            int num_sms, cudaStream_t st) {
+  if (n == 0) return cudaSuccess;
+  const RawRows r{rows};
+  return vjp ? launch_vjp(net, r, nullptr, n, out, num_sms, st) : launch_infer_tc(net, r, nullptr, n, out, num_sms, st);
 }
 
 cudaError_t cache_grad(const CacheNet& net, const CacheRows& rows, const float4* mat_a, const float4* mat_b,
                        const uint32_t* count_dev, uint32_t n, uint32_t batch, uint32_t n_batches,
                        const CacheOut& out, int num_sms, cudaStream_t st) {
-  if (n == 0 || n_batches == 0) return cudaSuccess;
-  const uint32_t tiles = ((n + n_batches - 1u) / n_batches + kTileRows - 1u) / kTileRows;
-  const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>(tiles, (uint32_t)(2 * num_sms)));
-  cudaFuncSetAttribute(cache_grad_k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemTrain);
-  cache_grad_k<<<grid, kThreads, kSmemTrain, st>>>(net, rows, mat_a, mat_b, count_dev, n, batch, n_batches, out);
-  return cudaGetLastError();
+  return launch_grad(net, PackedRows{rows, mat_a, mat_b}, count_dev, n, batch, n_batches, out, num_sms, st);
+}
+
+cudaError_t cache_grad_raw(const CacheNet& net, const CacheRaw& rows, uint32_t n, const CacheOut& out, int num_sms,
+                           cudaStream_t st) {
+  return launch_grad(net, RawRows{rows}, nullptr, n, 0, 1, out, num_sms, st);
 }
 
 cudaError_t cache_adam(float* w, float* mw, float* vw, float* gw, float* table, float* mt, float* vt, float* gt,
@@ -1254,20 +1270,6 @@ cudaError_t cache_pack_table(const float* table, uint32_t* table_h, cudaStream_t
 
 cudaError_t cache_pack_weights(const float* w, uint4* wt, cudaStream_t st) {
   cache_pack_k<<<grid_of(kCacheWeights, 256), 256, 0, st>>>(w, reinterpret_cast<__nv_bfloat16*>(wt));
-  return cudaGetLastError();
-}
-
-cudaError_t cache_pack_rows(uint32_t n, const float* x01, const float* dir, const float* nrm, const float* params7,
-                            const float* u, const CacheRows& rows, float4* mat_a, float4* mat_b, cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  cache_pack_rows_k<<<grid_of(n, 256), 256, 0, st>>>(n, x01, dir, nrm, params7, u, rows, mat_a, mat_b);
-  return cudaGetLastError();
-}
-
-cudaError_t cache_unpack_out(uint32_t n, const float4* c, const float* dp, float* rgb, float* dparams,
-                             cudaStream_t st) {
-  if (n == 0) return cudaSuccess;
-  cache_unpack_k<<<grid_of(n, 256), 256, 0, st>>>(n, c, dp, rgb, dparams);
   return cudaGetLastError();
 }
 

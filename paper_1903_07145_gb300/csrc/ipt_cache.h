@@ -43,6 +43,11 @@ struct CacheRows {
   float4* u;
 };
 
+// Rows given as plain arrays: x01, d, n, u (n x 3), p7 (n x 7: kd, ks, r).
+struct CacheRaw {
+  const float *x, *d, *n, *p7, *u;
+};
+
 // Device error word bit: a bounded wait for the tensor cores gave up (the
 // pass's results are incomplete).
 constexpr uint32_t kErrTimeout = 4u;
@@ -51,6 +56,8 @@ constexpr uint32_t kErrTimeout = 4u;
 struct CacheOut {
   float4* c;      // prediction per row (nullable)
   float4* rad;    // nullable: rad[slot] += u * prediction
+  float* rgb;     // nullable: prediction per row, 3 floats
+  float* dp7;     // nullable: as dp, 7 floats per row
   float* dp;      // nullable: 8 floats per row, d(u . prediction) / d(kd, ks, r), 8th = 0
   float* gw;      // training: weight gradients (accumulated)
   float2* gt;     // training: hash-table gradients (accumulated)
@@ -97,14 +104,12 @@ cudaError_t cache_pack_weights(const float* w, uint4* wt, cudaStream_t st);
 // FP16 copy of the hash table (kCacheTableFloats halves), from the FP32 master.
 cudaError_t cache_pack_table(const float* table, uint32_t* table_h, cudaStream_t st);
 
-// Rows of the evaluation entry points: row i gets x = x01[i], segment i,
-// and per-row parameter tables (kd, r) / (ks, 0) from params7[i].
-cudaError_t cache_pack_rows(uint32_t n, const float* x01, const float* dir, const float* nrm, const float* params7,
-                            const float* u, const CacheRows& rows, float4* mat_a, float4* mat_b, cudaStream_t st);
-
-// Per-row outputs of the evaluation entry points back to n x 3 / n x 7.
-cudaError_t cache_unpack_out(uint32_t n, const float4* c, const float* dp, float* rgb, float* dparams,
-                             cudaStream_t st);
+// The same for rows given as plain arrays (outputs rgb and dp7, or gw and gt,
+// must not share memory with them).
+cudaError_t cache_infer_raw(const CacheNet& net, const CacheRaw& rows, uint32_t n, const CacheOut& out, bool vjp,
+                            int num_sms, cudaStream_t st);
+cudaError_t cache_grad_raw(const CacheNet& net, const CacheRaw& rows, uint32_t n, const CacheOut& out, int num_sms,
+                           cudaStream_t st);
 
 // Targets of the records appended since the chunk began: u = rad[slot].
 cudaError_t cache_targets(const CacheBuffers& b, const float4* rad, cudaStream_t st);

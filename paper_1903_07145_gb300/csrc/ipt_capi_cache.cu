@@ -122,33 +122,28 @@ ipt_status cache_create(ipt_ctx* ctx, DeviceScene* s, const ipt_cache_opts* o) {
   return IPT_OK;
 }
 
-// Evaluation rows for n inputs.
-ipt_status cache_api_rows(ipt_ctx* ctx, CacheState* c, uint32_t n) {
+// Room for n rows' results.
+ipt_status cache_api_out(ipt_ctx* ctx, CacheState* c, uint32_t n) {
   if (c->api_cap >= n) return IPT_OK;
   IPT_CK(cudaStreamSynchronize(ctx->stream));
-  for (void* p : c->api_owned) cudaFree(p);
-  c->api_owned.clear();
+  cudaFree(c->api_out);
+  c->api_out = nullptr;
   c->api_cap = 0;
-  cudaError_t e = cudaSuccess;
-  auto A = [&](auto** p, size_t k) {
-    void* q = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc(&q, k * sizeof(**p));
-    if (e == cudaSuccess) {
-      c->api_owned.push_back(q);
-      *p = static_cast<std::remove_reference_t<decltype(*p)>>(q);
-    }
-  };
-  A(&c->api.x, n);
-  A(&c->api.d, n);
-  A(&c->api.n, n);
-  A(&c->api.u, n);
-  A(&c->api_ma, n);
-  A(&c->api_mb, n);
-  A(&c->api_c, n);
-  A(&c->api_dp, 8 * (size_t)n);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "cache evaluation rows");
+  IPT_CK(cudaMalloc(&c->api_out, 10 * sizeof(float) * (size_t)n));
   c->api_cap = n;
   return IPT_OK;
+}
+
+bool overlap(const void* a, size_t na, const void* b, size_t nb) {
+  const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+  return a && b && x < y + nb && y < x + na;
+}
+
+// Whether `out` (bytes) shares memory with any of the rows' arrays.
+bool touches_rows(const void* out, size_t bytes, const ipt::CacheRaw& r, uint32_t n) {
+  const size_t n3 = 3 * sizeof(float) * (size_t)n, n7 = 7 * sizeof(float) * (size_t)n;
+  return overlap(out, bytes, r.x, n3) || overlap(out, bytes, r.d, n3) || overlap(out, bytes, r.n, n3) ||
+         overlap(out, bytes, r.u, n3) || overlap(out, bytes, r.p7, n7);
 }
 
 }  // namespace
@@ -218,18 +213,27 @@ ipt_status ipt_cache_eval(ipt_ctx* ctx, int32_t scene, uint32_t n, const float* 
   if (!x01 || !dir || !nrm || !params7 || !rgb_out) return fail(ctx, IPT_ERR_INVALID_ARG, "null input or output");
   CacheState* c = s->cache;
   IPT_CK(cudaSetDevice(ctx->device));
-  if ((st = cache_api_rows(ctx, c, n)) != IPT_OK) return st;
-  IPT_CK(ipt::cache_pack_rows(n, x01, dir, nrm, params7, upstream, c->api, c->api_ma, c->api_mb, ctx->stream));
   const bool vjp = upstream && dparams_out;
+  const ipt::CacheRaw rows{x01, dir, nrm, params7, upstream};
+  const size_t n3 = 3 * sizeof(float) * (size_t)n, n7 = 7 * sizeof(float) * (size_t)n;
+  // rows are read while others' results are stored
+  const bool apart = !touches_rows(rgb_out, n3, rows, n) && !(vjp && touches_rows(dparams_out, n7, rows, n));
   ipt::CacheOut o{};
-  o.c = c->api_c;
-  o.dp = vjp ? c->api_dp : nullptr;
+  o.rgb = rgb_out;
+  o.dp7 = vjp ? dparams_out : nullptr;
+  if (!apart) {
+    if ((st = cache_api_out(ctx, c, n)) != IPT_OK) return st;
+    o.rgb = c->api_out;
+    o.dp7 = vjp ? c->api_out + 3 * (size_t)n : nullptr;
+  }
   {
     Timed tm(ctx, vjp ? IPT_KERNEL_CACHE_VJP : IPT_KERNEL_CACHE_INFER);
-    IPT_CK(ipt::cache_infer(cache_net(s, true), c->api, c->api_ma, c->api_mb, nullptr, n, o, vjp, ctx->L.num_sms,
-                            ctx->stream));
+    IPT_CK(ipt::cache_infer_raw(cache_net(s, true), rows, n, o, vjp, ctx->L.num_sms, ctx->stream));
   }
-  IPT_CK(ipt::cache_unpack_out(n, c->api_c, c->api_dp, rgb_out, vjp ? dparams_out : nullptr, ctx->stream));
+  if (!apart) {
+    IPT_CK(cudaMemcpyAsync(rgb_out, o.rgb, n3, cudaMemcpyDeviceToDevice, ctx->stream));
+    if (vjp) IPT_CK(cudaMemcpyAsync(dparams_out, o.dp7, n7, cudaMemcpyDeviceToDevice, ctx->stream));
+  }
   return IPT_OK;
 }
 
@@ -243,15 +247,16 @@ ipt_status ipt_cache_grad(ipt_ctx* ctx, int32_t scene, uint32_t n, const float* 
   if (!x01 || !dir || !nrm || !params7 || !target) return fail(ctx, IPT_ERR_INVALID_ARG, "null input");
   CacheState* c = s->cache;
   IPT_CK(cudaSetDevice(ctx->device));
-  if ((st = cache_api_rows(ctx, c, n)) != IPT_OK) return st;
-  IPT_CK(ipt::cache_pack_rows(n, x01, dir, nrm, params7, target, c->api, c->api_ma, c->api_mb, ctx->stream));
+  const ipt::CacheRaw rows{x01, dir, nrm, params7, target};
   const size_t nw = ipt::kCacheWeights, nt = ipt::kCacheTableFloats;
   // the kernel adds to the caller's arrays where their alignment allows its
-  // vector reductions; the cache's own accumulators (kept zero between
-  // training steps) take the rest
+  // vector reductions and they are apart from the rows; the cache's own
+  // accumulators (kept zero between training steps) take the rest
   const auto aligned = [](const void* p, size_t a) { return p && reinterpret_cast<uintptr_t>(p) % a == 0; };
-  float* gw = aligned(grad_weights, 16) ? grad_weights : c->gw;
-  float* gt = !grad_table || aligned(grad_table, 8) ? grad_table : c->gt;  // null: no table gradient
+  const bool own_w = !aligned(grad_weights, 16) || touches_rows(grad_weights, nw * sizeof(float), rows, n);
+  const bool own_t = grad_table && (!aligned(grad_table, 8) || touches_rows(grad_table, nt * sizeof(float), rows, n));
+  float* gw = own_w ? c->gw : grad_weights;
+  float* gt = own_t ? c->gt : grad_table;  // null: no table gradient
   IPT_CK(cudaMemsetAsync(gw, 0, nw * sizeof(float), ctx->stream));
   if (gt) IPT_CK(cudaMemsetAsync(gt, 0, nt * sizeof(float), ctx->stream));
   IPT_CK(cudaMemsetAsync(c->loss_dev, 0, sizeof(double), ctx->stream));
@@ -262,15 +267,14 @@ ipt_status ipt_cache_grad(ipt_ctx* ctx, int32_t scene, uint32_t n, const float* 
   o.err = ctx->err_dev;
   {
     Timed tm(ctx, IPT_KERNEL_CACHE_GRAD);
-    IPT_CK(ipt::cache_grad(cache_net(s, true), c->api, c->api_ma, c->api_mb, nullptr, n, 0, 1, o, ctx->L.num_sms,
-                           ctx->stream));
+    IPT_CK(ipt::cache_grad_raw(cache_net(s, true), rows, n, o, ctx->L.num_sms, ctx->stream));
   }
-  if (gw == c->gw) {
+  if (own_w) {
     if (grad_weights)
       IPT_CK(cudaMemcpyAsync(grad_weights, gw, nw * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
     IPT_CK(cudaMemsetAsync(gw, 0, nw * sizeof(float), ctx->stream));
   }
-  if (gt == c->gt) {
+  if (own_t) {
     IPT_CK(cudaMemcpyAsync(grad_table, gt, nt * sizeof(float), cudaMemcpyDeviceToDevice, ctx->stream));
     IPT_CK(cudaMemsetAsync(gt, 0, nt * sizeof(float), ctx->stream));
   }

@@ -50,14 +50,9 @@ struct CacheState {
   uint64_t steps_done = 0;
   uint32_t last_pass_steps = 0;
   ipt::CacheBuffers buf{};
-  // rows of the evaluation entry points
-  ipt::CacheRows api{};
-  float4* api_ma = nullptr;
-  float4* api_mb = nullptr;
-  float4* api_c = nullptr;
-  float* api_dp = nullptr;
+  // results of an evaluation call whose outputs share memory with its inputs
+  float* api_out = nullptr;  // 10 floats per row
   uint32_t api_cap = 0;
-  std::vector<void*> api_owned;
   std::vector<void*> owned;
   double image_bias = -1.0, grad_bias = -1.0;
 };
@@ -65,7 +60,7 @@ struct CacheState {
 inline void free_cache(CacheState* c) {
   if (!c) return;
   for (void* p : c->owned) cudaFree(p);
-  for (void* p : c->api_owned) cudaFree(p);
+  cudaFree(c->api_out);
   if (c->host) cudaFreeHost(c->host);
   delete c;
 }
