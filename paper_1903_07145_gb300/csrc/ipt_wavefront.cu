@@ -867,8 +867,15 @@ __global__ void __launch_bounds__(kWfThreads, 8) k_trace_rays(SceneDev s, RayArr
 // path-state loads, and the extra warps hide more of that latency.
 // kD: the Disney material model (sampler, BRDF and NEE pdf) in place of
 // Lambert + GGX; the rest of the stage is shared.
-template <bool kD>
-__global__ void __launch_bounds__(kWfThreads, 8) wf_shade_fwd(const WfScene* tab, WfParams lp, uint32_t p0,
+// kOne: a launch over one scene, whose table entry is the kernel parameter
+// `one` (constant memory: its pointers are operands, where the table's entry
+// is loaded again for nearly every use, a dependent load before each of a
+// vertex's ~20 scattered ones).  61k room: shading 8.25 -> 8.0 ms, first adjoint
+// stage 11.9 -> 11.5 ms (516k room 14.3 -> 13.4).  (The traversal, whose pointers
+// stay in registers, gained nothing from it.)
+template <bool kD, bool kOne>
+__global__ void __launch_bounds__(kWfThreads, 8) wf_shade_fwd(const WfScene* tab, const __grid_constant__ WfScene one,
+                                                           WfParams lp, uint32_t p0,
                                                            WfDev w, int cur) {
   if (blockIdx.x == 0 && threadIdx.x == 0) w.cnt[3] = 0;  // closest fetch counter of the next vertex
   const uint32_t n = w.cnt[cur];
@@ -893,7 +900,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_shade_fwd(const WfScene* tab
     float pdf = 0.0f;
     Vtx v;
     if (tri >= 0) {
-      const WfScene& e = tab[lp.n_scenes == 1 ? 0u : b];
+      const WfScene& e = kOne ? one : tab[b];
       const bool light_on = lp.nee && any_light(e.s, e.t);
       const float4 rd = w.ray_d[slot];
       Hit h;
@@ -997,7 +1004,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_shade_fwd(const WfScene* tab
     const uint32_t ci = enqueue(nout, cont);
     if (cont) {
       qout[ci] = slot;
-      if (lp.keys) lp.keys[ci] = (uint16_t)ray_bin(lp.bin, tab[lp.n_scenes == 1 ? 0u : b], b, org, wo);
+      if (lp.keys) lp.keys[ci] = (uint16_t)ray_bin(lp.bin, kOne ? one : tab[b], b, org, wo);
       w.ray_o[slot] = make_float4(org.x, org.y, org.z, __int_as_float(tri));
       w.ray_d[slot] = make_float4(wo.x, wo.y, wo.z, pdf);
       w.beta[slot] = make_float4(beta.x, beta.y, beta.z, __uint_as_float(pack_state(k + 1, b)));
@@ -1355,8 +1362,9 @@ __device__ __forceinline__ void scale_carry(const WfDev& w, uint32_t slot, uint3
 // Stage A: emission at the vertex, its contribution to the carry, and the
 // next-event candidate (with, for the Disney model, the material derivative
 // of its term, added if the shadow ray finds the light).
-template <bool kD, bool kW>
-__global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, WfParams lp, uint32_t p0, WfDev w,
+template <bool kD, bool kW, bool kOne>
+__global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, const __grid_constant__ WfScene one,
+                                                       WfParams lp, uint32_t p0, WfDev w,
                                                        int cur) {
   constexpr uint32_t P = kD ? 16u : 10u;
   IPT_ACCUM(P, kW, acc);
@@ -1382,7 +1390,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, Wf
     const int tri = __float_as_int(hh.x);
     const uint32_t st = __float_as_uint(bt.w);
     const uint32_t k = state_k(st), b = state_scene(st);
-    const WfScene& e = tab[lp.n_scenes == 1 ? 0u : b];
+    const WfScene& e = kOne ? one : tab[b];
     uint32_t pid = 0, smp = 0, ent = 0;
     float3 gp = f3(0.f, 0.f, 0.f);
     if (act) {
@@ -1501,8 +1509,9 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_a(const WfScene* tab, Wf
 // Unoccluded next-event terms: light emission (Eq. 5), the vertex material
 // (Eq. 6 at this vertex) and the carry of the earlier vertices.  A launch
 // over one scene skips reading the slot's state word for its scene.
-template <bool kD, bool kW>
-__global__ void __launch_bounds__(kWfThreads) wf_adj_connect(const WfScene* tab, WfParams lp, WfDev w) {
+template <bool kD, bool kW, bool kOne>
+__global__ void __launch_bounds__(kWfThreads) wf_adj_connect(const WfScene* tab, const __grid_constant__ WfScene one,
+                                                             WfParams lp, WfDev w) {
   constexpr uint32_t P = kD ? 16u : 10u;
   IPT_ACCUM(P, kW, acc);
   const uint32_t n = w.cnt[2];
@@ -1517,7 +1526,7 @@ __global__ void __launch_bounds__(kWfThreads) wf_adj_connect(const WfScene* tab,
       for (int j = 0; j < kDisneyMat; ++j) g[j] = 0.0f;
       if (vis) {
         const uint4 m = w.sh_meta[i];
-        const WfScene& e = tab[lp.n_scenes == 1 ? 0u : state_scene(__float_as_uint(w.beta[m.x].w))];
+        const WfScene& e = kOne ? one : tab[state_scene(__float_as_uint(w.beta[m.x].w))];
         const float4 ge = w.sh_ge[i], cn = w.sh_n[i];
         lrow = acc_row(e, lp, (int)m.w);
         ge3 = xyz(ge);
@@ -1534,7 +1543,7 @@ __global__ void __launch_bounds__(kWfThreads) wf_adj_connect(const WfScene* tab,
       float g[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       if (vis) {
         const uint4 m = w.sh_meta[i];
-        const WfScene& e = tab[lp.n_scenes == 1 ? 0u : state_scene(__float_as_uint(w.beta[m.x].w))];
+        const WfScene& e = kOne ? one : tab[state_scene(__float_as_uint(w.beta[m.x].w))];
         const float4 ge = w.sh_ge[i], gm = w.sh_gm[i], cn = w.sh_n[i];
         lrow = acc_row(e, lp, (int)m.w);
         ge3 = xyz(ge);
@@ -1558,8 +1567,9 @@ __global__ void __launch_bounds__(kWfThreads) wf_adj_connect(const WfScene* tab,
 }
 
 // Stage B: BRDF sampling; the new vertex joins the carry.
-template <bool kD, bool kW>
-__global__ void __launch_bounds__(kWfThreads, 8) wf_adj_b(const WfScene* tab, WfParams lp, uint32_t p0, WfDev w,
+template <bool kD, bool kW, bool kOne>
+__global__ void __launch_bounds__(kWfThreads, 8) wf_adj_b(const WfScene* tab, const __grid_constant__ WfScene one,
+                                                       WfParams lp, uint32_t p0, WfDev w,
                                                        int cur) {
   constexpr uint32_t P = kD ? 16u : 10u;
   IPT_ACCUM(P, kW, acc);
@@ -1590,7 +1600,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_b(const WfScene* tab, Wf
     float pdf = 0.0f;
     int tri = -1;
     const uint32_t k = state_k(st), b = state_scene(st);
-    const WfScene& e = tab[lp.n_scenes == 1 ? 0u : b];
+    const WfScene& e = kOne ? one : tab[b];
     float3 gfin = f3(0.f, 0.f, 0.f);
     if (!(st & kDead)) {
       tri = __float_as_int(hh.x);
@@ -1660,7 +1670,7 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_b(const WfScene* tab, Wf
     const uint32_t ci = enqueue(nout, cont);
     if (cont) {
       qout[ci] = slot;
-      if (lp.keys) lp.keys[ci] = (uint16_t)ray_bin(lp.bin, tab[lp.n_scenes == 1 ? 0u : b], b, org, wo);
+      if (lp.keys) lp.keys[ci] = (uint16_t)ray_bin(lp.bin, kOne ? one : tab[b], b, org, wo);
       w.ray_o[slot] = make_float4(org.x, org.y, org.z, __int_as_float(tri));
       w.ray_d[slot] = make_float4(wo.x, wo.y, wo.z, pdf);
       w.beta[slot] = make_float4(beta.x, beta.y, beta.z, __uint_as_float(pack_state(k + 1, b)));
@@ -1673,7 +1683,8 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_adj_b(const WfScene* tab, Wf
 // carry (Eq. 6 through their BSDF factors), its parameter derivative goes to
 // the terminal segment's kd, ks and roughness, and the path finishes.
 template <bool kW>
-__global__ void __launch_bounds__(kWfThreads) wf_adj_cache(const WfScene* tab, WfParams lp, uint32_t p0, WfDev w) {
+__global__ void __launch_bounds__(kWfThreads) wf_adj_cache(const __grid_constant__ WfScene e, WfParams lp, uint32_t p0,
+                                                           WfDev w) {
   IPT_ACCUM(10u, kW, acc);
   const uint32_t n = lp.cb.counts[0];
   const float inv_spp = 1.0f / (float)lp.spp;
@@ -1684,7 +1695,6 @@ __global__ void __launch_bounds__(kWfThreads) wf_adj_cache(const WfScene* tab, W
     const uint32_t slot = act ? __float_as_uint(lp.cb.q.d[q].w) : 0u;
     const uint32_t st = act ? __float_as_uint(w.beta[slot].w) : 0u;
     const uint32_t nv = act ? w.nv[slot] : 0u;
-    const WfScene& e = tab[lp.n_scenes == 1 ? 0u : state_scene(st)];
     float g[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     int row = -1;
     float3 gp = f3(0.f, 0.f, 0.f);
@@ -2028,7 +2038,9 @@ cudaError_t wf_forward(const Launcher& L, const WfScene* tab_dev, const std::vec
   const int width = table_width(tab);
   const int grid = wf_grid(L);
   const int grid_cam = one_wave(L, wf_camera, 0);
-  const int grid_sh = disney ? one_wave(L, wf_shade_fwd<true>, 0) : one_wave(L, wf_shade_fwd<false>, 0);
+  const auto k_sh = ns == 1 ? (disney ? wf_shade_fwd<true, true> : wf_shade_fwd<false, true>)
+                            : (disney ? wf_shade_fwd<true, false> : wf_shade_fwd<false, false>);
+  const int grid_sh = one_wave(L, k_sh, 0);
   const int red_grid = loss_partials_capacity(L);
   const size_t red_smem = sizeof(double) * ns;
   const std::vector<WfChunk> chunks = wf_plan(tab, wb.cap, tp.spp, 0xffffffffu);
@@ -2053,10 +2065,7 @@ cudaError_t wf_forward(const Launcher& L, const WfScene* tab_dev, const std::vec
       }
       {
         IPT_STAGE(10);
-        if (disney)
-          wf_shade_fwd<true><<<grid_sh, kWfThreads, 0, st>>>(tab_dev, lp, c.p0, w, cur);
-        else
-          wf_shade_fwd<false><<<grid_sh, kWfThreads, 0, st>>>(tab_dev, lp, c.p0, w, cur);
+        k_sh<<<grid_sh, kWfThreads, 0, st>>>(tab_dev, tab[0], lp, c.p0, w, cur);
       }
       if (k < last_k && k < tp.max_depth && tp.nee && !(record && k < lp.cache_k)) {
         IPT_STAGE(9);
@@ -2134,10 +2143,11 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
   if (max_np > wb.blk_params) return cudaErrorInvalidValue;
   const size_t shmem = max_shared * sizeof(float);
   if (shmem > 48 * 1024) {
-    cudaFuncSetAttribute(wf_adj_a<kD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
-    cudaFuncSetAttribute(wf_adj_connect<kD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
-    cudaFuncSetAttribute(wf_adj_b<kD, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
-    cudaFuncSetAttribute(wf_adj_cache<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
+    const void* shared[] = {(const void*)wf_adj_a<kD, false, true>, (const void*)wf_adj_a<kD, false, false>,
+                            (const void*)wf_adj_connect<kD, false, true>, (const void*)wf_adj_connect<kD, false, false>,
+                            (const void*)wf_adj_b<kD, false, true>, (const void*)wf_adj_b<kD, false, false>,
+                            (const void*)wf_adj_cache<false>};
+    for (const void* k : shared) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shmem);
   }
   for (const WfChunk& c : chunks) {
     lp.seg_lo = c.seg_lo;
@@ -2147,9 +2157,12 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
     const bool global = c.seg_n > max_seg;
     lp.gacc = global ? wb.blk : nullptr;
     const size_t sm = global ? 0 : acc_shared_floats(P, c.seg_n) * sizeof(float);
-    const auto k_a = global ? wf_adj_a<kD, true> : wf_adj_a<kD, false>;
-    const auto k_c = global ? wf_adj_connect<kD, true> : wf_adj_connect<kD, false>;
-    const auto k_b = global ? wf_adj_b<kD, true> : wf_adj_b<kD, false>;
+    const auto k_a = ns == 1 ? (global ? wf_adj_a<kD, true, true> : wf_adj_a<kD, false, true>)
+                             : (global ? wf_adj_a<kD, true, false> : wf_adj_a<kD, false, false>);
+    const auto k_c = ns == 1 ? (global ? wf_adj_connect<kD, true, true> : wf_adj_connect<kD, false, true>)
+                             : (global ? wf_adj_connect<kD, true, false> : wf_adj_connect<kD, false, false>);
+    const auto k_b = ns == 1 ? (global ? wf_adj_b<kD, true, true> : wf_adj_b<kD, false, true>)
+                             : (global ? wf_adj_b<kD, true, false> : wf_adj_b<kD, false, false>);
     const auto k_q = global ? wf_adj_cache<true> : wf_adj_cache<false>;
     // each adjoint stage runs one wave at its own occupancy for this
     // accumulator size; block b of every stage adds into gradient row b
@@ -2179,7 +2192,7 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
       }
       {
         IPT_STAGE(11);
-        k_a<<<g_a, kWfThreads, sm, st>>>(tab_dev, lp, c.p0, w, cur);
+        k_a<<<g_a, kWfThreads, sm, st>>>(tab_dev, tab[0], lp, c.p0, w, cur);
       }
       if (k < last_k) {
         if (tp.nee) {
@@ -2188,10 +2201,10 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
             launch_trace<2>(width, grid, tab_dev, tab, w, cur, slots, L.wf_steps, err, st);
           }
           IPT_STAGE(12);
-          k_c<<<g_c, kWfThreads, sm, st>>>(tab_dev, lp, w);
+          k_c<<<g_c, kWfThreads, sm, st>>>(tab_dev, tab[0], lp, w);
         }
         IPT_STAGE(13);
-        k_b<<<g_b, kWfThreads, sm, st>>>(tab_dev, lp, c.p0, w, cur);
+        k_b<<<g_b, kWfThreads, sm, st>>>(tab_dev, tab[0], lp, c.p0, w, cur);
       }
       cur ^= 1;
     }
@@ -2206,7 +2219,7 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
         if (e != cudaSuccess) return e;
       }
       IPT_STAGE(13);
-      k_q<<<g_q, kWfThreads, sm, st>>>(tab_dev, lp, c.p0, w);
+      k_q<<<g_q, kWfThreads, sm, st>>>(tab[0], lp, c.p0, w);
     }
     IPT_STAGE(14);
     if (global)
@@ -2258,10 +2271,14 @@ static cudaError_t wf_occupancy(Launcher* L) {
   L->wf_occ = b < 1 ? 1 : b;
   // the adjoint stage with the most blocks (accumulators in dynamic shared
   // memory only lower the occupancy)
-  const void* stages[] = {(const void*)wf_adj_a<false, false>, (const void*)wf_adj_connect<false, false>,
-                          (const void*)wf_adj_b<false, false>, (const void*)wf_adj_a<true, false>,
-                          (const void*)wf_adj_connect<true, false>, (const void*)wf_adj_b<true, false>,
-                          (const void*)wf_adj_cache<false>};
+  const void* stages[] = {
+      (const void*)wf_adj_a<false, false, false>, (const void*)wf_adj_connect<false, false, false>,
+      (const void*)wf_adj_b<false, false, false>, (const void*)wf_adj_a<false, false, true>,
+      (const void*)wf_adj_connect<false, false, true>, (const void*)wf_adj_b<false, false, true>,
+      (const void*)wf_adj_a<true, false, false>, (const void*)wf_adj_connect<true, false, false>,
+      (const void*)wf_adj_b<true, false, false>, (const void*)wf_adj_a<true, false, true>,
+      (const void*)wf_adj_connect<true, false, true>, (const void*)wf_adj_b<true, false, true>,
+      (const void*)wf_adj_cache<false>};
   L->wf_row_occ = 1;
   for (const void* k : stages) {
     int bk = 0;
