@@ -743,7 +743,13 @@ struct ArrayRays {
 //    triangle tests when at least as many lanes wait at a triangle as at a
 //    node, node tests otherwise (the other lanes sit the step out).  Letting
 //    both kinds run in one step serialises the two code paths with most
-//    lanes masked off in each.  The warp refetches once `steps` of its lanes
+//    lanes masked off in each.  Between two votes a lane takes up to three
+//    units of the kind (node tests of shadow rays and triangle tests: two):
+//    the votes cost more than the lanes that sit the further units out.  61k
+//    room, closest hit / shadow rays with (node, triangle) units per vote:
+//    (1, 1) 35.7 / 20.9 ms, (2, 1) 34.8 / 19.4, (3, 1) 33.7 / 19.6, (2, 2) 33.6
+//    / 18.1, (3, 2) 32.3 / 18.4, (4, 2) 32.9 / 18.6, (3, 3) 33.9 / 19.1, (2, 3)
+//    35.0 / 18.9, (5, 3) 36.0 / 20.4.  The warp refetches once `steps` of its lanes
 //    are idle (or all are); the lanes whose rays have ended store their
 //    results then, together, rather than each in the step its ray ends
 //    (with one or two lanes active).
@@ -815,10 +821,22 @@ __device__ __forceinline__ void trace_loop(Src& src, uint32_t n, uint32_t* fetch
         const unsigned mt = __ballot_sync(0xffffffffu, at_tri);
         if (ml == 0u || (!drained && 32 - __popc(ml) >= refill)) break;
         const bool tri_phase = __popc(mt) >= __popc(ml & ~mt);
-        if (live && at_tri == tri_phase)
-          fin = at_tri        ? tri_step<kAny, kWidth>(src.scene(), T, S)
-                : kWidth == 8 ? node_step8<kAny>(src.scene(), T, S, err)
-                              : node_step4<kAny, kWidth == kGrid4>(src.scene(), T, S, err);
+        if (tri_phase) {
+          if (at_tri) {
+            fin = tri_step<kAny, kWidth>(src.scene(), T, S);
+            if (!fin && T.tri < T.tri_end) fin = tri_step<kAny, kWidth>(src.scene(), T, S);
+          }
+        } else if (live && !at_tri) {
+          if constexpr (kWidth == 8) {
+            fin = node_step8<kAny>(src.scene(), T, S, err);
+          } else {
+            constexpr bool kGrid = kWidth == kGrid4;
+            fin = node_step4<kAny, kGrid>(src.scene(), T, S, err);
+            if (!fin && T.tri >= T.tri_end) fin = node_step4<kAny, kGrid>(src.scene(), T, S, err);
+            if constexpr (!kAny)
+              if (!fin && T.tri >= T.tri_end) fin = node_step4<kAny, kGrid>(src.scene(), T, S, err);
+          }
+        }
       }
     }
   }
