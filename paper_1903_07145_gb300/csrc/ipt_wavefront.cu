@@ -1041,10 +1041,20 @@ __global__ void __launch_bounds__(kWfThreads) wf_reduce(const WfScene* tab, WfPa
   const float inv = 1.0f / (float)lp.spp;
   for (uint32_t l = blockIdx.x * blockDim.x + threadIdx.x; l < n_pix; l += gridDim.x * blockDim.x) {
     float3 a = f3(0.f, 0.f, 0.f), a2 = f3(0.f, 0.f, 0.f);
-    for (uint32_t smp = 0; smp < lp.spp; ++smp) {
-      const float3 L = xyz(w.rad[l * lp.spp + smp]);
-      a = a + L;
-      a2 = a2 + L * L;
+    // eight samples' loads at a time, added in order (64 samples of 64 pixels:
+    // one load at a time was a chain of 64 misses)
+    for (uint32_t smp = 0; smp < lp.spp; smp += 8) {
+      float4 r[8];
+#pragma unroll
+      for (uint32_t j = 0; j < 8; ++j)
+        if (smp + j < lp.spp) r[j] = w.rad[l * lp.spp + smp + j];
+#pragma unroll
+      for (uint32_t j = 0; j < 8; ++j)
+        if (smp + j < lp.spp) {
+          const float3 L = xyz(r[j]);
+          a = a + L;
+          a2 = a2 + L * L;
+        }
     }
     const uint32_t b = state_scene(__float_as_uint(w.beta[l * lp.spp].w));
     const WfScene& e = tab[b];
@@ -1735,24 +1745,26 @@ __global__ void __launch_bounds__(kWfThreads) wf_adj_cache(const __grid_constant
 }
 
 // grad_acc[i] += sum over block rows (FP64), for the chunk's parameters.
-// Block b covers parameters 32b .. 32b+31: warp w sums rows w, w+32, ...
-// (lane l reads parameter 32b+l, so a warp reads 128 contiguous bytes per
-// row), then warp 0 adds the 32 warp sums in a fixed order: the result does
-// not depend on scheduling.
-constexpr int kReduceWarps = 32;
-__global__ void __launch_bounds__(32 * kReduceWarps) wf_blk_reduce(const float* blk, int rows, uint32_t np,
-                                                                    double* grad_acc) {
-  __shared__ double part[kReduceWarps][33];
-  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-  const uint32_t i = blockIdx.x * 32u + lane;
+// Block b covers parameters 8b .. 8b+7: group g of 8 lanes (128 groups) sums
+// rows g, g + 128, ... (a group reads 32 contiguous bytes per row), then 8
+// threads add the 128 sums in a fixed order: the result does not depend on
+// scheduling.  32 parameters a block left the FP64 additions (an SM's FP64 unit
+// takes 16 cycles for a warp's) to a few SMs: 31 us for the 160 parameters of
+// 1216 rows, 7 now, and 3 with the 32 rows of a pixel batch of 4096 paths.
+constexpr int kReduceCols = 8, kReduceGroups = 128;
+__global__ void __launch_bounds__(kReduceCols * kReduceGroups) wf_blk_reduce(const float* blk, int rows, uint32_t np,
+                                                                             double* grad_acc) {
+  __shared__ double part[kReduceGroups][kReduceCols];
+  const uint32_t c = threadIdx.x % kReduceCols, g = threadIdx.x / kReduceCols;
+  const uint32_t i = blockIdx.x * kReduceCols + c;
   double s = 0.0;
   if (i < np)
-    for (int r = (int)warp; r < rows; r += kReduceWarps) s += (double)blk[(size_t)r * np + i];
-  part[warp][lane] = s;
+    for (int r = (int)g; r < rows; r += kReduceGroups) s += (double)blk[(size_t)r * np + i];
+  part[g][c] = s;
   __syncthreads();
-  if (warp == 0 && i < np) {
+  if (threadIdx.x < kReduceCols && i < np) {
     double t = 0.0;
-    for (int k = 0; k < kReduceWarps; ++k) t += part[k][lane];
+    for (int k = 0; k < min(kReduceGroups, rows); ++k) t += part[k][c];
     grad_acc[i] += t;
   }
 }
@@ -1836,6 +1848,15 @@ static int one_wave(const Launcher& L, K kernel, size_t smem) {
   int b = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, kWfThreads, smem) != cudaSuccess || b < 1) b = 1;
   return L.num_sms * b;
+}
+
+// Blocks of an adjoint stage over a chunk of `slots` path slots: one wave, but
+// none without a slot.  A pixel batch of 4096 slots takes 32: gradient rows of
+// those alone are cleared and reduced (see wf_blk_reduce).  One-warp blocks,
+// which would reach more SMs, were measured and gave nothing.
+template <typename K>
+static int adjoint_blocks(const Launcher& L, K kernel, size_t smem, uint32_t slots) {
+  return (int)std::min<uint32_t>((uint32_t)one_wave(L, kernel, smem), (slots + kWfThreads - 1u) / kWfThreads);
 }
 
 int wf_max_blocks(const Launcher& L) { return std::max(wf_grid(L), L.wf_max_rows); }
@@ -2185,14 +2206,14 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
     // each adjoint stage runs one wave at its own occupancy for this
     // accumulator size; block b of every stage adds into gradient row b
     // (all blocks into the padded global array in global mode)
-    const int g_a = one_wave(L, k_a, sm), g_c = one_wave(L, k_c, sm);
-    const int g_b = one_wave(L, k_b, sm), g_q = one_wave(L, k_q, sm);
+    const uint32_t slots = c.n_pix * tp.spp;
+    const int g_a = adjoint_blocks(L, k_a, sm, slots), g_c = adjoint_blocks(L, k_c, sm, slots);
+    const int g_b = adjoint_blocks(L, k_b, sm, slots), g_q = adjoint_blocks(L, k_q, sm, slots);
     const int rows = global ? 1 : std::max(std::max(g_a, g_c), std::max(g_b, g_q));
     if (rows > wf_max_blocks(L)) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(
         wb.blk, 0, (global ? (size_t)wide_stride(P) * c.seg_n : (size_t)rows * np) * sizeof(float), st);
     if (e != cudaSuccess) return e;
-    const uint32_t slots = c.n_pix * tp.spp;
     {
       IPT_STAGE(7);
       wf_camera<<<grid_cam, kWfThreads, 0, st>>>(tab_dev, lp, c.p0, slots, w);
@@ -2243,7 +2264,8 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
     if (global)
       wf_wide_reduce<P><<<std::min<uint32_t>((np + 255u) / 256u, 2048u), 256, 0, st>>>(wb.blk, np, grad_acc + P * c.seg_lo);
     else
-      wf_blk_reduce<<<(np + 31) / 32, 32 * kReduceWarps, 0, st>>>(wb.blk, rows, np, grad_acc + P * c.seg_lo);
+      wf_blk_reduce<<<(np + kReduceCols - 1) / kReduceCols, kReduceCols * kReduceGroups, 0, st>>>(wb.blk, rows, np,
+                                                                                              grad_acc + P * c.seg_lo);
   }
   return cudaGetLastError();
 }
