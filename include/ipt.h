@@ -109,7 +109,12 @@ typedef struct {
  * identical paths).
  *   integrator: 0 = megakernel (one thread per path, every stage inline),
  *     1 = wavefront (chunks of path slots; persistent traversal kernels over
- *     compacted ray queues).
+ *     compacted ray queues).  A context whose program never calls
+ *     ipt_config_set reports 1 and runs the passes of ipt_render,
+ *     ipt_backward, ipt_loss_grad(_shard), ipt_step and ipt_batch_step that
+ *     have too few paths for the wavefront on the megakernel (the same paths;
+ *     the timings of such a pass are IPT_KERNEL_FORWARD and
+ *     IPT_KERNEL_ADJOINT).
  *   wavefront_slots: path slots per wavefront chunk (0 = 1 << 20); rounded
  *     down to whole pixels.  The context keeps 162 bytes of device memory
  *     per slot, and once it has run an adjoint 52 + 40 D more (D: the

@@ -290,6 +290,25 @@ bool use_wavefront(const ipt_ctx* ctx, uint32_t spp) {
   return ctx->cfg.integrator == 1 && spp <= cap;
 }
 
+// Whether a pass of n paths of a context whose program has set no integrator
+// runs the megakernel.  The paths are the same, and a small pass is a chain of
+// latencies: one launch of one path a thread has one where the wavefront's
+// 3-4 launches a vertex have one each, until the paths fill the chip and the
+// wavefront's compaction and refills win.  Furnished rooms of 3k and 61k
+// triangles, depth 5, a whole call, ms (wavefront | megakernel):
+//   paths                    4096        16384        65536       131072       262144
+//   ipt_render    3k    .34 | .13    .42 | .19    .52 | .29    .59 | .49    .80 | .86
+//                61k    .46 | .16    .56 | .27    .71 | .36    .82 | .65   1.05 | 1.20
+//   ipt_backward  3k    .52 | .16    .60 | .23    .72 | .54    .80 | 1.01  1.13 | 1.85
+//                61k    .63 | .19    .74 | .28    .91 | .71   1.01 | 1.27  1.42 | 2.36
+// Hence 28 and 14 warps of paths an SM (136192 and 68096 paths on 152).  A
+// context with traversal counters keeps the wavefront, which counts.
+static bool picks_megakernel(const ipt_ctx* ctx, uint64_t n, uint32_t warps_per_sm) {
+  return !ctx->cfg_set && !ctx->counters_dev && n <= 32ull * warps_per_sm * (uint32_t)ctx->L.num_sms;
+}
+bool picks_megakernel_forward(const ipt_ctx* ctx, uint64_t n) { return picks_megakernel(ctx, n, 28); }
+bool picks_megakernel_adjoint(const ipt_ctx* ctx, uint64_t n) { return picks_megakernel(ctx, n, 14); }
+
 // Scene-table entry of one scene for a launch over its pixels
 // [pix_base, pix_base + n) (launch pixels 0..n-1).
 ipt::WfScene wf_entry(const ipt_ctx* ctx, int32_t scene_id, const DeviceScene* s, uint32_t pix_base, uint32_t n) {
@@ -339,7 +358,15 @@ ipt_status run_forward(ipt_ctx* ctx, int32_t scene_id, DeviceScene* s, uint32_t 
                        uint32_t* pick) {
   if (cache && !use_wavefront_cap(ctx, tp.spp))
     return fail(ctx, IPT_ERR_INVALID_ARG, "cached passes need spp <= wavefront_slots");
-  if (cache || use_wavefront(ctx, tp.spp)) {
+  // a pass without the radiance buffer (under capture, or memory short) would
+  // run a pixel's samples in one warp: the wavefront is quicker then
+  ipt::Launcher L = ctx->L;
+  bool wavefront = cache || use_wavefront(ctx, tp.spp);
+  if (!wavefront || (!cache && picks_megakernel_forward(ctx, (uint64_t)n * tp.spp))) {
+    L = forward_launcher(ctx, (uint64_t)n * tp.spp);
+    wavefront = wavefront && L.rad_cap < (uint64_t)n * tp.spp;
+  }
+  if (wavefront) {
     ipt_status st = ensure_wf(ctx, false, 10u * s->n_seg);
     if (st != IPT_OK) return st;
     ipt::WfScene e = wf_entry(ctx, scene_id, s, begin, n);
@@ -365,7 +392,7 @@ ipt_status run_forward(ipt_ctx* ctx, int32_t scene_id, DeviceScene* s, uint32_t 
     }
     ipt::TraceParams tpk = tp;
     tpk.pick = pick;
-    const ipt::Launcher L = forward_launcher(ctx, (uint64_t)n * tp.spp);
+    tpk.serial_sums = ctx->cfg.integrator != 0;  // picked: the wavefront's image
     Timed tm(ctx, IPT_KERNEL_FORWARD);
     IPT_CK(ipt::launch_forward(L, buffers(ctx, s), s->tab, s->views_dev, (uint32_t)s->views.size(), begin, n,
                                tpk, img, msq, target, g_out, partials, g_scale, loss_kind, ctx->err_dev,
@@ -381,7 +408,7 @@ ipt_status run_adjoint(ipt_ctx* ctx, int32_t scene_id, DeviceScene* s, uint32_t 
                        const ipt::CachePass* cache, uint32_t* pick) {
   if (cache && !use_wavefront_cap(ctx, tp.spp))
     return fail(ctx, IPT_ERR_INVALID_ARG, "cached passes need spp <= wavefront_slots");
-  if (cache || use_wavefront(ctx, tp.spp)) {
+  if (cache || (use_wavefront(ctx, tp.spp) && !picks_megakernel_adjoint(ctx, (uint64_t)n * tp.spp))) {
     ipt_status st = ensure_wf(ctx, true, 10u * s->n_seg, false, tp.max_depth);
     if (st != IPT_OK) return st;
     ipt::WfScene e = wf_entry(ctx, scene_id, s, begin, n);
@@ -1069,6 +1096,7 @@ ipt_status ipt_config_set(ipt_ctx* ctx, const ipt_config* cfg) {
     wf_release(ctx);
   }
   ctx->cfg = *cfg;
+  ctx->cfg_set = true;
   ctx->L.wf_steps = cfg->trace_steps ? (int)cfg->trace_steps : 16;
   ctx->L.wf_fixed_blocks = (int)cfg->blocks_per_sm;
   ctx->L.sort_cells = (int)cfg->sort_cells;

@@ -144,6 +144,12 @@ static bool same_opts(const ipt_trace_opts& a, const ipt_trace_opts& b) { return
 static bool same_adam(const ipt_adam_opts& a, const ipt_adam_opts& b) { return std::memcmp(&a, &b, sizeof(a)) == 0; }
 static bool same_cfg(const ipt_config& a, const ipt_config& b) { return std::memcmp(&a, &b, sizeof(a)) == 0; }
 
+// Whether a batch's residual pass of n samples runs the megakernel: as
+// configured, or picked for its size when the radiance buffer holds it.
+static bool batch_mk_forward(const ipt_ctx* ctx, uint64_t n) {
+  return ctx->cfg.integrator == 0 || (picks_megakernel_forward(ctx, n) && n <= ctx->L.rad_cap);
+}
+
 // The iteration of a batch, queued on stream `st` (captured into the graph).
 static ipt_status batch_enqueue(ipt_ctx* ctx, Batch* b, const ipt_trace_opts* opts, const ipt_adam_opts* adam,
                                 cudaStream_t st) {
@@ -159,13 +165,13 @@ static ipt_status batch_enqueue(ipt_ctx* ctx, Batch* b, const ipt_trace_opts* op
   tp.mis = opts->mis;
   tp.profile = opts->emission_profile;
   if (opts->pixel_batch) IPT_CK(ipt::wf_pick(b->tab_dev, b->tab_host, b->iter_dev, 0u, st));
-  // the megakernel runs each pass as one launch over the whole table
-  const bool mk = ctx->cfg.integrator == 0;
   const uint32_t ns = (uint32_t)b->tab_host.size();
   const uint32_t total = ns ? b->tab_host.back().pix_begin + b->tab_host.back().n_pix : 0u;
   uint32_t n_seg_active = 0;
   for (const ipt::WfScene& e : b->tab_host) n_seg_active = std::max(n_seg_active, e.seg_offset + e.n_seg);
-  if (mk)
+  // the megakernel runs each pass as one launch over the whole table
+  tp.serial_sums = ctx->cfg.integrator != 0;  // picked: the wavefront's sums
+  if (batch_mk_forward(ctx, (uint64_t)total * opts->spp_r))
     IPT_CK(ipt::launch_forward_batch(ctx->L, b->tab_dev, ns, total, tp, b->iter_dev, opts->loss, b->loss_rows,
                                      ctx->err_dev, st));
   else
@@ -175,7 +181,7 @@ static ipt_status batch_enqueue(ipt_ctx* ctx, Batch* b, const ipt_trace_opts* op
   tp.set = opts->gradcheck_same_set ? IPT_SET_RESIDUAL : IPT_SET_DERIVATIVE;
   tp.spp = opts->spp_d;
   if (opts->gradcheck_same_set) tp.sample_stride = opts->spp_r;
-  if (mk)
+  if (ctx->cfg.integrator == 0 || picks_megakernel_adjoint(ctx, (uint64_t)total * opts->spp_d))
     IPT_CK(ipt::launch_adjoint_batch(ctx->L, b->tab_dev, ns, total, n_seg_active, tp, b->iter_dev, b->grad_acc,
                                      b->gacc, ctx->err_dev, st));
   else
@@ -207,7 +213,7 @@ ipt_status ipt_batch_step(ipt_ctx* ctx, int32_t batch, const ipt_trace_opts* opt
     return IPT_OK;
   }
   if (!b->exec || !same_opts(*opts, b->g_opts) || !same_adam(*adam, b->g_adam) || !same_cfg(ctx->cfg, b->g_cfg) ||
-      b->g_alloc_gen != ctx->alloc_gen) {
+      b->g_cfg_set != ctx->cfg_set || b->g_alloc_gen != ctx->alloc_gen) {
     // everything the graph touches is allocated before the capture
     if (opts->pixel_batch)
       for (int32_t id : b->members)
@@ -215,8 +221,8 @@ ipt_status ipt_batch_step(ipt_ctx* ctx, int32_t batch, const ipt_trace_opts* opt
     batch_table(ctx, b, opts->pixel_batch);
     IPT_CK(cudaMemcpyAsync(b->mem_dev, b->mem_host.data(), b->mem_host.size() * sizeof(ipt::BatchMember),
                            cudaMemcpyHostToDevice, ctx->stream));
-    if (ctx->cfg.integrator == 0)
-      ensure_rad(ctx, (uint64_t)(b->tab_host.back().pix_begin + b->tab_host.back().n_pix) * opts->spp_r);
+    const uint64_t n_fwd = (uint64_t)(b->tab_host.back().pix_begin + b->tab_host.back().n_pix) * opts->spp_r;
+    if (ctx->cfg.integrator == 0 || picks_megakernel_forward(ctx, n_fwd)) ensure_rad(ctx, n_fwd);
     uint32_t max_seg = 0;
     for (const ipt::WfChunk& c : ipt::wf_plan(b->tab_host, cap, opts->spp_d, ipt::wf_max_segments()))
       max_seg = std::max(max_seg, c.seg_n);
@@ -241,6 +247,7 @@ ipt_status ipt_batch_step(ipt_ctx* ctx, int32_t batch, const ipt_trace_opts* opt
     b->g_opts = *opts;
     b->g_adam = *adam;
     b->g_cfg = ctx->cfg;
+    b->g_cfg_set = ctx->cfg_set;
     b->g_alloc_gen = ctx->alloc_gen;
   }
   // the members' parameter tables (shared with the single-scene calls) hold

@@ -169,6 +169,7 @@ struct Batch {
   ipt_trace_opts g_opts{};
   ipt_adam_opts g_adam{};
   ipt_config g_cfg{};
+  bool g_cfg_set = false;
   uint64_t g_alloc_gen = 0;  // the context's alloc_gen when the graph was captured
 };
 
@@ -202,6 +203,7 @@ struct ipt_ctx {
   double kernel_ms[IPT_KERNEL_COUNT] = {0};
   uint64_t kernel_n[IPT_KERNEL_COUNT] = {0};
   ipt_config cfg = {1, 1u << 20, 32, 0, 4};
+  bool cfg_set = false;  // ipt_config_set was called: every pass runs the integrator it names
   ipt::WfBuffers wf;
   std::vector<void*> wf_owned;
   bool wf_adjoint = false;
@@ -244,6 +246,8 @@ void ensure_rad(ipt_ctx* ctx, uint64_t n);
 ipt_status read_back(ipt_ctx* ctx, void* dst, const void* src, size_t n);
 bool use_wavefront_cap(const ipt_ctx* ctx, uint32_t spp);
 bool use_wavefront(const ipt_ctx* ctx, uint32_t spp);
+bool picks_megakernel_forward(const ipt_ctx* ctx, uint64_t n);
+bool picks_megakernel_adjoint(const ipt_ctx* ctx, uint64_t n);
 ipt::WfScene wf_entry(const ipt_ctx* ctx, int32_t scene_id, const DeviceScene* s, uint32_t pix_base, uint32_t n);
 ipt_status upload_entry(ipt_ctx* ctx, const ipt::WfScene& e);
 ipt_status draw_picks(ipt_ctx* ctx, int32_t scene_id, const DeviceScene* s, uint32_t B, uint64_t iteration,

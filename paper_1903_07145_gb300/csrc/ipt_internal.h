@@ -124,6 +124,10 @@ struct TraceParams {
   uint32_t sample_stride = 0;
   // megakernel: the pixel batch's drawn pixels (entries 0..n-1), or nullptr
   const uint32_t* pick = nullptr;
+  // megakernel, a residual pass that fits the radiance buffer: a pixel's
+  // samples are added one after the other, as the wavefront does, so that the
+  // image is its image bit for bit (false: by groups of lanes)
+  bool serial_sums = false;
 };
 
 struct Launcher {

@@ -67,7 +67,10 @@ __device__ __forceinline__ bool forward_vertex(const SceneDev& s, const SegDev& 
     const NeeResult ne = next_event(s, t, v, ua, ub, pp.profile, pp.mis, sa.y, sa.x, err);
     if (ne.valid) {
       const BrdfVal bv = brdf_eval(ma, mb, v.ns, v.wi, ne.wl);
-      p.L = p.L + p.beta * bv.f * xyz(__ldg(&t.emis[ne.seg])) * ne.k;
+      // rounded before it is added, as the wavefront keeps it in a queue: the
+      // integrators' radiances are equal
+      const float3 c = p.beta * bv.f * xyz(__ldg(&t.emis[ne.seg])) * ne.k;
+      p.L = f3(__fadd_rn(p.L.x, c.x), __fadd_rn(p.L.y, c.y), __fadd_rn(p.L.z, c.z));
     }
   }
   if (!(dot(v.wi, v.ns) > 0.0f)) return false;
@@ -209,8 +212,28 @@ __device__ void adjoint_path(const SceneDev& s, const SegDev& t, const ViewDev& 
 // lane tracing spp / group samples; the lanes' sums are combined with
 // butterfly shuffles, so the pixel estimate is deterministic.  kRad: the
 // samples' radiances were traced before (k_forward_samples) and are read from
-// `rad`; the sums are the same, in the same order.
+// `rad`; the sums are the same, in the same order, unless pp.serial asks for
+// the wavefront's.
 // ---------------------------------------------------------------------------
+
+// Adds a pixel's traced radiances one after the other: its group of G lanes
+// loads G of them at a time (one lane alone: 12 us for 64 samples of 64
+// pixels) and every lane adds all, so each ends with the pixel's sums.  All
+// 32 lanes call it together.
+template <typename Add>
+__device__ __forceinline__ void each_radiance(const float4* rad, bool active, uint32_t sub, uint32_t spp, uint32_t G,
+                                              Add add) {
+  for (uint32_t s0 = 0; s0 < spp; s0 += G) {
+    const float4 r = active && s0 + sub < spp ? rad[s0 + sub] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint32_t n = min(G, spp - s0);
+    for (uint32_t j = 0; j < n; ++j) {
+      const int src = (int)j;
+      add(f3(__shfl_sync(0xffffffffu, r.x, src, (int)G), __shfl_sync(0xffffffffu, r.y, src, (int)G),
+             __shfl_sync(0xffffffffu, r.z, src, (int)G)));
+    }
+  }
+}
+
 template <bool kRad>
 __global__ void __launch_bounds__(kBlockThreads) k_forward(SceneDev s, SegDev t, const ViewDev* views,
                                                            uint32_t n_views, uint32_t pix_begin, uint32_t n_pix,
@@ -232,6 +255,10 @@ __global__ void __launch_bounds__(kBlockThreads) k_forward(SceneDev s, SegDev t,
     const uint32_t local = task * ppw + lane / G;
     const bool active = local < n_pix;
     float3 a = f3(0.f, 0.f, 0.f), a2 = f3(0.f, 0.f, 0.f);
+    const auto add = [&](float3 L) {
+      a = a + L;
+      a2 = a2 + L * L;
+    };
     uint32_t pid = pix_begin + local;
     if (active) {
       uint32_t s0 = 0;
@@ -242,17 +269,15 @@ __global__ void __launch_bounds__(kBlockThreads) k_forward(SceneDev s, SegDev t,
       const ViewDev& vw = find_view(views, n_views, pid);
       const uint32_t lp = pid - vw.offset;
       const uint32_t px = lp % vw.w, py = lp / vw.w;
-      for (uint32_t smp = sub; smp < pp.spp; smp += G) {
-        float3 L;
+      for (uint32_t smp = sub; smp < pp.spp && !(kRad && pp.serial); smp += G) {
         if constexpr (kRad)
-          L = xyz(rad[local * pp.spp + smp]);
+          add(xyz(rad[local * pp.spp + smp]));
         else
-          L = forward_path(s, t, vw, px, py, pid, s0 + smp, pp, light, err);
-        a = a + L;
-        a2 = a2 + L * L;
+          add(forward_path(s, t, vw, px, py, pid, s0 + smp, pp, light, err));
       }
     }
-    for (uint32_t off = G >> 1; off >= 1; off >>= 1) {
+    if (kRad && pp.serial) each_radiance(rad + (size_t)local * pp.spp, active, sub, pp.spp, G, add);
+    for (uint32_t off = kRad && pp.serial ? 0u : G >> 1; off >= 1; off >>= 1) {
       a.x += __shfl_xor_sync(0xffffffffu, a.x, off);
       a.y += __shfl_xor_sync(0xffffffffu, a.y, off);
       a.z += __shfl_xor_sync(0xffffffffu, a.z, off);
@@ -448,7 +473,7 @@ __global__ void __launch_bounds__(kBlockThreads, 4)
       entry = p - e.pix_begin + e.pix_base;
       pid = e.pick ? e.pick[entry] : entry;
       if constexpr (kRad) {
-        for (uint32_t smp = sub; smp < pp.spp; smp += G) a = a + xyz(rad[p * pp.spp + smp]);
+        for (uint32_t smp = sub; smp < pp.spp && !pp.serial; smp += G) a = a + xyz(rad[p * pp.spp + smp]);
       } else {
         const uint32_t s0 = e.pick ? entry * pp.stride : 0u;
         const PathParams q = scene_params(pp, e, set_iter);
@@ -460,7 +485,9 @@ __global__ void __launch_bounds__(kBlockThreads, 4)
           a = a + forward_path(e.s, e.t, vw, px, py, pid, s0 + smp, q, light, err);
       }
     }
-    for (uint32_t off = G >> 1; off >= 1; off >>= 1) {
+    if (kRad && pp.serial)
+      each_radiance(rad + (size_t)p * pp.spp, active, sub, pp.spp, G, [&](float3 L) { a = a + L; });
+    for (uint32_t off = kRad && pp.serial ? 0u : G >> 1; off >= 1; off >>= 1) {
       a.x += __shfl_xor_sync(0xffffffffu, a.x, off);
       a.y += __shfl_xor_sync(0xffffffffu, a.y, off);
       a.z += __shfl_xor_sync(0xffffffffu, a.z, off);
@@ -870,6 +897,14 @@ static uint32_t few_lanes(const Launcher& L, uint64_t n) {
 static bool few_forward(const Launcher& L, uint64_t n) { return n <= L.rad_cap; }
 static bool few_adjoint(const Launcher& L, uint64_t n) { return n <= 32ull * kFewWarpsPerSm * (uint32_t)L.num_sms; }
 
+// In-order sums: a group loads what it can of a pixel's samples at once, its
+// size need not divide their number.
+static void serial_group(PathParams& pp) {
+  pp.serial = true;
+  pp.group = 1;
+  while (pp.group < 32 && pp.group < pp.spp) pp.group *= 2;
+}
+
 static int few_grid(uint32_t n, uint32_t lanes) {
   const uint32_t per_block = lanes * (kBlockThreads / 32u);
   return (int)((n + per_block - 1u) / per_block);
@@ -887,7 +922,8 @@ cudaError_t launch_forward(const Launcher& L, const SceneBuffers& s, const SegBu
                            uint32_t n_pix, const TraceParams& tp, float* img, float* msq,
                            const float* target, float* g_out, double* loss_partials,
                            float g_scale, int loss_kind, uint32_t* err, cudaStream_t st) {
-  const PathParams pp = make_path_params(tp, s);
+  PathParams pp = make_path_params(tp, s);
+  if (tp.serial_sums) serial_group(pp);
   const uint64_t tasks = (n_pix + (32 / pp.group) - 1) / (32 / pp.group);
   const int cap = L.num_sms * L.fwd_blocks_per_sm;
   // with a loss the grid is fixed, so the partial sums reduce in a fixed order
@@ -965,7 +1001,8 @@ cudaError_t launch_forward_batch(const Launcher& L, const WfScene* tab_dev, uint
                                  const TraceParams& tp, const uint32_t* iter_dev, int loss_kind, double* loss_rows,
                                  uint32_t* err, cudaStream_t st) {
   // one block per loss row: every row of the batch's loss reduction is written
-  const PathParams pp = batch_path_params(tp);
+  PathParams pp = batch_path_params(tp);
+  if (tp.serial_sums) serial_group(pp);
   const size_t sm = sizeof(double) * n_scenes;
   if (few_forward(L, (uint64_t)total * tp.spp)) {
     const uint32_t n = total * tp.spp, lanes = few_lanes(L, n);

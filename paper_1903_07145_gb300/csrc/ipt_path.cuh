@@ -27,6 +27,7 @@ struct PathParams {
   // pix_begin + i with counters s)
   const uint32_t* pick;
   uint32_t stride;
+  bool serial = false;  // k_forward<true>: samples added in order (TraceParams::serial_sums)
 };
 
 __host__ __device__ inline uint32_t lanes_per_pixel(uint32_t spp) {
