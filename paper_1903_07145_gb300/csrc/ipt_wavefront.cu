@@ -762,11 +762,16 @@ struct ArrayRays {
 // launch, 11 launches a pass): closest hit 0.33 -> 0.24 ms, shadow rays 0.32
 // -> 0.23 ms; two rays a warp at least: 0.25 and 0.24, four: 0.25 and 0.25,
 // eight: 0.27 and 0.27, 32: 0.30 and 0.29.
+// kFirst: a warp takes its first 32 rays by position and fetches from there on
+// (all warps of a wave fetching from one counter before their first ray cost
+// 1-2 us of a launch: 297k camera rays in the 61k room 64.0 -> 62.3 us; the
+// queues' kernels lose more to the registers of it, 35.7 -> 36.6 ms on the 61k
+// room, and do without).
 // kCount: counts node visits and triangle tests (a context with counters);
 // without it the two counters and their pointer stay out of the registers
 // (with the ray's permuted origin kept instead of selected per test: closest
 // hit 41.8 -> 39.8 ms, shadow rays 23.3 -> 22.1 ms on the 61k room).
-template <bool kAny, int kWidth, bool kFew, class Src>
+template <bool kAny, int kWidth, bool kFew, bool kFirst, class Src>
 __device__ __forceinline__ void trace_loop(Src& src, uint32_t n, uint32_t* fetch, int steps, uint32_t* err) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t lt_mask = (1u << lane) - 1u;
@@ -779,6 +784,7 @@ __device__ __forceinline__ void trace_loop(Src& src, uint32_t n, uint32_t* fetch
   uint32_t item = kNone;  // the lane's ray
   bool fin = false;       // wide BVHs: the lane's ray has ended, its result not yet stored
   bool drained = false;   // warp-uniform: no rays left to fetch
+  bool first = true;      // kFirst: the warp's first rays are still to come
   for (;;) {
     if (fin) {  // results are stored at the refill, by all ended lanes together
       src.finish(item, T);
@@ -795,10 +801,16 @@ __device__ __forceinline__ void trace_loop(Src& src, uint32_t n, uint32_t* fetch
         i = lane < lanes ? (blockIdx.x * (kWfThreads / 32u) + (threadIdx.x >> 5)) * lanes + lane : n;
         drained = true;
       } else {
-        const int leader = __ffs(m) - 1;
         uint32_t base = 0;
-        if ((int)lane == leader) base = atomicAdd(fetch, (uint32_t)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, leader);
+        if (kFirst && first) {
+          base = (blockIdx.x * (kWfThreads / 32u) + (threadIdx.x >> 5)) * 32u;
+          first = false;
+        } else {
+          const int leader = __ffs(m) - 1;
+          if ((int)lane == leader) base = atomicAdd(fetch, (uint32_t)__popc(m));
+          base = __shfl_sync(0xffffffffu, base, leader);
+          if (kFirst) base += gridDim.x * kWfThreads;
+        }
         drained = base + (uint32_t)__popc(m) >= n;
         i = base + (uint32_t)__popc(m & lt_mask);
       }
@@ -853,18 +865,19 @@ __global__ void __launch_bounds__(kWfThreads, 8) wf_trace(const WfScene* tab, Wf
   }
   const uint32_t n = kAny ? w.cnt[2] : w.cnt[cur];
   QueueRays<kMode, kWidth, kCount> src{tab, w, order ? order : queue(w, cur), one_scene, tab[0].s};
-  trace_loop<kAny, kWidth, kFew>(src, n, kAny ? &w.cnt[4] : &w.cnt[3], steps, err);
+  trace_loop<kAny, kWidth, kFew, false>(src, n, kAny ? &w.cnt[4] : &w.cnt[3], steps, err);
 }
 
 // Closest hits of rays given as arrays, by the same loops (one thread per ray
 // with whole leaves and its stack in local memory took 279 us for a million
-// random rays in the 61k room, 194 us here; 4099 rays 37.3 -> 31.5 us).
-// state: [0] rays fetched, [1] blocks done; both 0 before and after a launch.
+// random rays in the 61k room, 171 us here; 4099 rays 37.3 -> 29.2 us).
+// state: [0] rays fetched beyond the warps' first ones, [1] blocks done; both
+// 0 before and after a launch.
 template <int kWidth, bool kCount, bool kFew>
 __global__ void __launch_bounds__(kWfThreads, 8) k_trace_rays(SceneDev s, RayArrays a, uint32_t n, int steps,
                                                               uint32_t* state, uint32_t* err) {
   ArrayRays<kWidth, kCount> src{s, a};
-  trace_loop<false, kWidth, kFew>(src, n, state, steps, err);
+  trace_loop<false, kWidth, kFew, true>(src, n, state, steps, err);
   if constexpr (!kFew) {  // the last block clears the counters
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1966,6 +1979,22 @@ static void launch_rays_w(int grid, const SceneDev& s, const RayArrays& a, uint3
 cudaError_t launch_trace_rays(const Launcher& L, const SceneBuffers& s, const RayArrays& a, uint32_t n,
                               uint32_t* state, uint32_t* err, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
+  // the fetch counter runs past the rays by as many as a wave has lanes: a
+  // launch of at most 2^30 rays keeps it from wrapping
+  constexpr uint32_t kMostRays = 1u << 30;
+  if (n > kMostRays) {
+    const cudaError_t e = launch_trace_rays(L, s, a, kMostRays, state, err, st);
+    if (e != cudaSuccess) return e;
+    RayArrays rest = a;
+    rest.orig += 3ull * kMostRays;
+    rest.dir += 3ull * kMostRays;
+    rest.tri += kMostRays;
+    if (rest.skip) rest.skip += kMostRays;
+    if (rest.t) rest.t += kMostRays;
+    if (rest.u) rest.u += kMostRays;
+    if (rest.v) rest.v += kMostRays;
+    return launch_trace_rays(L, s, rest, n - kMostRays, state, err, st);
+  }
   const int most = wf_grid(L);
   RayArrays r = a;
   r.orig_to_internal = s.orig_to_internal;
