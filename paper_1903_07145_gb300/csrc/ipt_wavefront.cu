@@ -1999,14 +1999,24 @@ cudaError_t launch_trace_rays(const Launcher& L, const SceneBuffers& s, const Ra
   RayArrays r = a;
   r.orig_to_internal = s.orig_to_internal;
   const SceneDev sd = scene_dev(s);
-  if (s.counters) {
-    launch_rays_w<true, false>(most, sd, r, n, L.wf_steps, state, err, st);
-  } else if (n <= (uint32_t)most * kWfThreads) {
-    const int grid = (int)std::min<uint32_t>((n + kWfThreads / 32u - 1u) / (kWfThreads / 32u), (uint32_t)most);
-    launch_rays_w<false, true>(grid, sd, r, n, L.wf_steps, state, err, st);
-  } else {
-    launch_rays_w<false, false>(most, sd, r, n, L.wf_steps, state, err, st);
+  // up to a wave of rays: at least one a warp.  More of them are fetched, but
+  // not in a launch that the caller captures: its graph may run beside other
+  // launches, and they would share the fetch counter.
+  const bool wave = n <= (uint32_t)most * kWfThreads;
+  const int grid = wave ? (int)std::min<uint32_t>((n + kWfThreads / 32u - 1u) / (kWfThreads / 32u), (uint32_t)most)
+                        : (int)((n + kWfThreads - 1u) / kWfThreads);
+  bool fetch = !wave;
+  if (fetch) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    fetch = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    if (!fetch) cudaGetLastError();
   }
+  if (s.counters)
+    launch_rays_w<true, true>(grid, sd, r, n, L.wf_steps, state, err, st);
+  else if (fetch)
+    launch_rays_w<false, false>(most, sd, r, n, L.wf_steps, state, err, st);
+  else
+    launch_rays_w<false, true>(grid, sd, r, n, L.wf_steps, state, err, st);
   return cudaGetLastError();
 }
 

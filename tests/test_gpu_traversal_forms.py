@@ -97,3 +97,34 @@ def test_ray_counts_around_the_launch_forms(n):
             for a, b in zip(ref, got):
                 assert torch.equal(a[pick], b)
     tr.close()
+
+
+def test_a_captured_launch_keeps_no_counter():
+    """More rays than a wave has lanes, captured: graphs replayed side by side
+    and beside an eager call give each its own hits."""
+    sc = scenes.indoor_room(3, n_cuboids=6, cuboid_sub=4, room_sub=4, n_lights=2, n_views=1, width=8, height=8)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        tr = Tracer(sc, seed=1)
+        rays = [[torch.from_numpy(a).cuda() for a in scenes.random_rays(sc, 200003, k)] for k in (4, 5)]
+        ref = [[v.clone() for v in tr.trace_rays(*r)] for r in rays]
+        stream.synchronize()
+        graphs, outs = [], []
+        for r in rays:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream):
+                outs.append(tr.trace_rays(*r))
+            graphs.append(g)
+        torch.cuda.synchronize()
+    other = torch.cuda.Stream()
+    for _ in range(3):
+        with torch.cuda.stream(stream):
+            graphs[0].replay()
+            eager = tr.trace_rays(*rays[1])
+        with torch.cuda.stream(other):
+            graphs[1].replay()
+        torch.cuda.synchronize()
+        for got, want in ((outs[0], ref[0]), (outs[1], ref[1]), (eager, ref[1])):
+            for a, b in zip(got, want):
+                assert torch.equal(a, b)
+    tr.close()
