@@ -10,12 +10,13 @@
 // 64 -> 64 -> 16, ReLU on hidden layers, no biases; the first 3 outputs are
 // the predicted reflected radiance.
 //
-// Queries run on the fifth-generation tensor cores: a block of 128 threads
-// encodes 128 rows (one per thread) into a BF16 tile in shared memory, one
-// thread issues each layer as tcgen05.mma (M = 128 rows) into FP32
-// accumulators in tensor memory (TMEM), and every thread reads its row back
-// with tcgen05.ld, applies the ReLU and writes the next layer's tile.  The
-// input VJP and training run each warp's 16 rows forward and backward with
+// Queries run on the fifth-generation tensor cores: a block is four groups of
+// 128 threads that share one weight image.  A group encodes 128 rows (one per
+// thread) into its BF16 tile in shared memory, one of its threads issues each
+// layer as tcgen05.mma (M = 128 rows) into the group's FP32 accumulators in
+// tensor memory (TMEM), and every thread reads its row back with tcgen05.ld,
+// applies the ReLU and writes the next layer's tile; a group's gathers fill
+// the others' MMA round trips.  The input VJP and training run each warp's 16 rows forward and backward with
 // mma.sync m16n8k16: a layer's FP32 accumulator fragments are the next
 // layer's A fragments once packed to BF16, so the VJP needs only the hidden
 // layers' ReLU masks (one register per layer), and the backward pass loads
@@ -24,10 +25,10 @@
 // slower than these independent per-warp chains.)  Training keeps the
 // block's 64 rows of inputs, activations and pre-activation gradients in
 // shared memory in the core-matrix-blocked layout that the tensor cores
-// read: the weight gradients dW = A^T dZ over those rows (K = rows) are one
-// tcgen05.mma batch per tile, accumulated in TMEM across every tile the
-// block processes, then read back and added to the global gradient once per
-// launch.
+// read: the weight gradients dW = A^T dZ of layers 1..4 over those rows (K =
+// rows) are two tcgen05.mma batches per tile, accumulated in TMEM across every
+// tile the block processes, then read back and added to the global gradient
+// once per launch; dW5 is summed in registers.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
