@@ -392,7 +392,7 @@ ipt_status run_forward(ipt_ctx* ctx, int32_t scene_id, DeviceScene* s, uint32_t 
     }
     ipt::TraceParams tpk = tp;
     tpk.pick = pick;
-    tpk.serial_sums = ctx->cfg.integrator != 0;  // picked: the wavefront's image
+    tpk.serial_sums = use_wavefront(ctx, tp.spp);  // picked for its size: the wavefront's image
     Timed tm(ctx, IPT_KERNEL_FORWARD);
     IPT_CK(ipt::launch_forward(L, buffers(ctx, s), s->tab, s->views_dev, (uint32_t)s->views.size(), begin, n,
                                tpk, img, msq, target, g_out, partials, g_scale, loss_kind, ctx->err_dev,

@@ -90,3 +90,20 @@ def test_a_batch_recaptures_when_the_program_chooses():
             out.append(ss.batch_step(opts, AdamOptions()))
         rows[late] = np.stack(out)
     np.testing.assert_allclose(rows[True], rows[False], rtol=1e-4)
+
+
+def test_a_pixel_of_more_samples_than_slots_keeps_its_sums():
+    """A wavefront too small for one pixel's samples leaves the pass to the
+    megakernel, which adds them as a megakernel configured by the program."""
+    imgs = []
+    for integrator in ("wavefront", "megakernel"):
+        sc = _room()
+        tr = Tracer(sc, seed=4)
+        tr.configure(integrator=integrator, wavefront_slots=1024)
+        tr.set_params(sc.gt_params)
+        tr.set_targets(np.zeros((tr.n_pix, 3), np.float32))
+        small = tr.loss_grad(TraceOptions(spp_r=1030, spp_d=1, max_depth=2, pixel_batch=8), 1)[0]
+        imgs.append((tr.render(TraceOptions(spp_r=1030, max_depth=2), view=0), small))
+        tr.close()
+    assert torch.equal(imgs[0][0], imgs[1][0])
+    assert imgs[0][1] == imgs[1][1]
