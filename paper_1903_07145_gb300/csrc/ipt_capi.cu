@@ -330,9 +330,11 @@ ipt::WfScene wf_entry(const ipt_ctx* ctx, int32_t scene_id, const DeviceScene* s
   return e;
 }
 
+// The entry travels as a kernel argument: a graph that the caller captures
+// keeps its value, where a copy from the host would read `e` again at each
+// replay, after this frame is gone.
 ipt_status upload_entry(ipt_ctx* ctx, const ipt::WfScene& e) {
-  if (!ctx->wf_tab) IPT_CK(cudaMalloc(&ctx->wf_tab, sizeof(ipt::WfScene)));
-  IPT_CK(cudaMemcpyAsync(ctx->wf_tab, &e, sizeof(e), cudaMemcpyHostToDevice, ctx->stream));
+  IPT_CK(ipt::wf_set_entry(e, ctx->wf_tab, ctx->stream));
   return IPT_OK;
 }
 
@@ -655,6 +657,7 @@ ipt_status ipt_create(ipt_ctx** out, const ipt_options* opt) {
   // the error word, then the ray-casting kernel's two counters
   if (e == cudaSuccess) e = cudaMalloc(&ctx->err_dev, 3 * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(ctx->err_dev, 0, 3 * sizeof(uint32_t));
+  if (e == cudaSuccess) e = cudaMalloc(&ctx->wf_tab, sizeof(ipt::WfScene));
   if (e == cudaSuccess) e = cudaMallocHost(&ctx->loss_host, 16 + kStageBytes);
   if (e == cudaSuccess) {
     ctx->err_host = reinterpret_cast<uint32_t*>(ctx->loss_host + 1);

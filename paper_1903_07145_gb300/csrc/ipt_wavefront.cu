@@ -1817,6 +1817,13 @@ __global__ void __launch_bounds__(kWfThreads) wf_pick_k(const WfScene* tab, uint
   }
 }
 
+__global__ void wf_entry_k(const __grid_constant__ WfScene e, WfScene* out) {
+  static_assert(sizeof(WfScene) % sizeof(uint32_t) == 0, "copied by words");
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(&e);
+  for (uint32_t i = threadIdx.x; i < sizeof(WfScene) / sizeof(uint32_t); i += blockDim.x)
+    reinterpret_cast<uint32_t*>(out)[i] = src[i];
+}
+
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
@@ -2306,6 +2313,11 @@ static cudaError_t wf_adjoint_model(const Launcher& L, const WfScene* tab_dev, c
       wf_blk_reduce<<<(np + kReduceCols - 1) / kReduceCols, kReduceCols * kReduceGroups, 0, st>>>(wb.blk, rows, np,
                                                                                               grad_acc + P * c.seg_lo);
   }
+  return cudaGetLastError();
+}
+
+cudaError_t wf_set_entry(const WfScene& e, WfScene* tab_dev, cudaStream_t st) {
+  wf_entry_k<<<1, 128, 0, st>>>(e, tab_dev);
   return cudaGetLastError();
 }
 

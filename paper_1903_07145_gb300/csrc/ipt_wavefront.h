@@ -65,6 +65,9 @@ cudaError_t wf_forward(const Launcher& L, const WfScene* tab_dev, const std::vec
                        double* loss_rows, uint32_t* err, cudaStream_t st, const WfHook* hook,
                        const CachePass* cache = nullptr, bool disney = false);
 
+// Writes a one-entry scene table.
+cudaError_t wf_set_entry(const WfScene& e, WfScene* tab_dev, cudaStream_t st);
+
 // Draws the pixel batch of every table entry that has one, for the iteration
 // *iter_dev (or iter when iter_dev is null).
 cudaError_t wf_pick(const WfScene* tab_dev, const std::vector<WfScene>& tab, const uint32_t* iter_dev,

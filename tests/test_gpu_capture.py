@@ -1,0 +1,78 @@
+"""Calls under stream capture: a replayed graph repeats the captured call,
+whatever the context ran in between.  Images are equal bit for bit; gradients
+agree to the rounding of FP32 sums in another order (rel 1e-5)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1903_07145_gb300 import _lib as L
+from paper_1903_07145_gb300 import scenes
+from paper_1903_07145_gb300.tracer import TraceOptions, Tracer
+
+pytestmark = pytest.mark.gpu
+MODES = ["wavefront", "megakernel"]
+OPTS = TraceOptions(spp_r=9, spp_d=3, max_depth=3)
+PICKS = TraceOptions(spp_r=9, spp_d=3, max_depth=3, pixel_batch=33)
+
+
+def _room():
+    return scenes.indoor_room(9, n_cuboids=4, cuboid_sub=2, room_sub=2, n_lights=2, n_views=2, width=40, height=31)
+
+
+def _loss_grad(tr, opts, iteration, disney=False):
+    """The call without its loss, which would wait for the stream."""
+    out = torch.empty((tr.n_seg, 16 if disney else 10), device="cuda")
+    f = L.ipt_disney_loss_grad if disney else L.ipt_loss_grad
+    f(tr.ctx, tr.sid, opts.c(), iteration, False, out.data_ptr())
+    return out
+
+
+CALLS = {
+    "render": lambda tr, w: tr.render(OPTS, view=1, iteration=2),
+    "backward": lambda tr, w: tr.backward(w, OPTS, iteration=2),
+    "loss_grad": lambda tr, w: _loss_grad(tr, OPTS, 2),
+    "pixel_batch": lambda tr, w: _loss_grad(tr, PICKS, 2),
+    "disney_render": lambda tr, w: tr.disney_render(OPTS, view=1, iteration=2),
+    "disney_pixel_batch": lambda tr, w: _loss_grad(tr, PICKS, 2, disney=True),
+}
+
+
+def _tracer(mode, seed=4):
+    sc = _room()
+    tr = Tracer(sc, seed=seed)
+    if mode != "unset":
+        tr.configure(mode)
+    tr.set_params(sc.gt_params)
+    tr.disney_set_params(scenes.disney_materials(sc, 3))
+    rng = np.random.default_rng(2)
+    tr.set_targets(rng.random((tr.n_pix, 3)).astype(np.float32))
+    return tr, torch.from_numpy(rng.normal(size=(tr.n_pix, 3)).astype(np.float32)).cuda()
+
+
+def _same(name, got, want):
+    if "render" in name:
+        return torch.equal(got, want)
+    return (got.double() - want.double()).norm() <= 1e-5 * want.double().norm()
+
+
+@pytest.mark.parametrize("mode", MODES)
+def test_replays_repeat_the_call(mode):
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        tr, w = _tracer(mode)
+        want = {k: f(tr, w).clone() for k, f in CALLS.items()}
+        stream.synchronize()
+        graphs, got = {}, {}
+        for k, f in CALLS.items():
+            graphs[k] = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graphs[k], stream=stream):
+                got[k] = f(tr, w)
+        for k in CALLS:
+            # another view, other entries: whatever a replay shares with later calls is theirs by now
+            tr.render(OPTS, view=0, iteration=5)
+            _loss_grad(tr, PICKS, 7)
+            got[k].fill_(float("nan"))
+            graphs[k].replay()
+            assert _same(k, got[k], want[k]), k
+        tr.synchronize()
+        tr.close()
