@@ -15,6 +15,10 @@
  *     context's stream has finished; the library never frees them.
  *   - Device work is queued on the context's CUDA stream.  Calls that return
  *     host data (loss, parameters) synchronise that stream first.
+ *   - Under stream capture: a call that returns no host data may be captured
+ *     from the context's stream, after a call with the same options has
+ *     allocated what it needs.  Its graph uses the context's buffers: replay
+ *     it in order with the context's other work, while the context lives.
  *   - Argument errors are reported as IPT_ERR_INVALID_ARG before anything is
  *     launched.  Errors found on the device set a status word that the next
  *     synchronising call returns: a traversal stack overflow as IPT_ERR_CUDA,

@@ -164,12 +164,42 @@ ipt_status ensure_tables(ipt_ctx* ctx, DeviceScene* s, const float* params, cons
   return IPT_OK;
 }
 
-void wf_release(ipt_ctx* c) {
-  for (void* p : c->wf_owned) cudaFree(p);
+// Whether the caller captures the context's stream (or, for the legacy
+// stream, another one: nothing may be waited for either way).
+static bool capturing(const ipt_ctx* ctx) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
+// cudaMalloc, also while the caller captures a stream in any mode (an
+// allocation is no stream operation: nothing of it enters the graph).
+static cudaError_t malloc_in_capture(void** p, size_t bytes) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const cudaError_t e = cudaMalloc(p, bytes);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return e;
+}
+
+// Gives the wavefront buffers back after the work queued on them.  Those that
+// a graph of the caller's holds (and, under capture, all: the stream cannot be
+// waited for) stay allocated until the context ends.
+ipt_status wf_release(ipt_ctx* c, bool under_capture) {
+  if (c->wf_captured || under_capture) {
+    c->wf_kept.insert(c->wf_kept.end(), c->wf_owned.begin(), c->wf_owned.end());
+  } else if (!c->wf_owned.empty()) {
+    const cudaError_t e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "wavefront buffers");
+    for (void* p : c->wf_owned) cudaFree(p);
+  }
   c->wf_owned.clear();
   c->wf = ipt::WfBuffers();
   c->wf_adjoint = false;
   c->wf_disney = false;
+  c->wf_captured = false;
+  return IPT_OK;
 }
 
 // Wavefront buffers for `cap` slots (plus the adjoint's carry when asked),
@@ -180,20 +210,24 @@ ipt_status ensure_wf(ipt_ctx* ctx, bool adjoint, uint32_t n_params, bool disney,
   const bool fits = ctx->wf.cap == cap &&
                     (!adjoint || (ctx->wf_adjoint && ctx->wf.blk_params >= n_params && ctx->wf.depth_cap >= depth)) &&
                     (!disney || ctx->wf_disney);
-  if (fits) return IPT_OK;
-  IPT_CK(cudaStreamSynchronize(ctx->stream));
+  const bool cap_now = capturing(ctx);
+  if (fits) {
+    ctx->wf_captured = ctx->wf_captured || cap_now;
+    return IPT_OK;
+  }
   ++ctx->alloc_gen;
   const uint32_t keep_params = std::max(n_params, ctx->wf.blk_params);
   const uint32_t keep_depth = std::max(adjoint ? depth : 0u, ctx->wf_adjoint ? ctx->wf.depth_cap : 0u);
   const bool want_adj = adjoint || ctx->wf_adjoint;
   const bool want_disney = want_adj && (disney || ctx->wf_disney);
-  wf_release(ctx);
+  const ipt_status st = wf_release(ctx, cap_now);
+  if (st != IPT_OK) return st;
   ipt::WfBuffers& w = ctx->wf;
   cudaError_t e = cudaSuccess;
   auto A = [&](auto** p, size_t n) {
     if (e != cudaSuccess) return;
     void* q = nullptr;
-    e = cudaMalloc(&q, n * sizeof(**p));
+    e = malloc_in_capture(&q, n * sizeof(**p));
     if (e == cudaSuccess) {
       ctx->wf_owned.push_back(q);
       *p = static_cast<std::remove_reference_t<decltype(*p)>>(q);
@@ -235,9 +269,10 @@ ipt_status ensure_wf(ipt_ctx* ctx, bool adjoint, uint32_t n_params, bool disney,
     A(&w.blk, std::max((size_t)ipt::wf_max_blocks(ctx->L) * shared_params, (size_t)keep_params * 6 / 5 + 16));
   }
   if (e != cudaSuccess) {
-    wf_release(ctx);
+    wf_release(ctx, cap_now);
     return cuda_fail(ctx, e, "wavefront buffers");
   }
+  ctx->wf_captured = cap_now;
   w.cap = cap;
   w.blk_params = want_adj ? keep_params : 0;
   w.depth_cap = want_adj ? keep_depth : 0;
@@ -248,36 +283,21 @@ ipt_status ensure_wf(ipt_ctx* ctx, bool adjoint, uint32_t n_params, bool disney,
 
 // Grows the radiance buffer of the megakernel's residual pass to n samples.
 // It stays as it is when n is above its limit or memory is short: the pass
-// then takes the form that needs none.
+// then takes the form that needs none.  A smaller buffer is kept until the
+// context ends, as a batch's graph or a caller's may use it (all of them hold
+// less than twice the last, at most 32 MB).
 void ensure_rad(ipt_ctx* ctx, uint64_t n) {
   if (n <= ctx->L.rad_cap || n > ipt::kFewSamples) return;
   uint32_t want = 1u << 16;
   while (want < n) want *= 2;
-  if (ctx->L.rad) {
-    if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return;
-    cudaFree(ctx->L.rad);
-    ++ctx->alloc_gen;
+  void* p = nullptr;
+  if (malloc_in_capture(&p, sizeof(float4) * want) != cudaSuccess) {
+    cudaGetLastError();
+    return;
   }
-  ctx->L.rad = nullptr;
-  ctx->L.rad_cap = 0;
-  if (cudaMalloc(&ctx->L.rad, sizeof(float4) * want) == cudaSuccess)
-    ctx->L.rad_cap = want;
-  else
-    cudaGetLastError();
-}
-
-// The launcher of a residual pass of n samples.  A pass that the caller
-// captures gets no radiance buffer: its graph may outlive the buffer.
-static ipt::Launcher forward_launcher(ipt_ctx* ctx, uint64_t n) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  const bool eager = cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
-  if (eager)
-    ensure_rad(ctx, n);
-  else
-    cudaGetLastError();
-  ipt::Launcher L = ctx->L;
-  if (!eager) L.rad_cap = 0;
-  return L;
+  ctx->rad_owned.push_back(p);
+  ctx->L.rad = static_cast<float4*>(p);
+  ctx->L.rad_cap = want;
 }
 
 bool use_wavefront_cap(const ipt_ctx* ctx, uint32_t spp) {
@@ -360,13 +380,13 @@ ipt_status run_forward(ipt_ctx* ctx, int32_t scene_id, DeviceScene* s, uint32_t 
                        uint32_t* pick) {
   if (cache && !use_wavefront_cap(ctx, tp.spp))
     return fail(ctx, IPT_ERR_INVALID_ARG, "cached passes need spp <= wavefront_slots");
-  // a pass without the radiance buffer (under capture, or memory short) would
-  // run a pixel's samples in one warp: the wavefront is quicker then
-  ipt::Launcher L = ctx->L;
+  // a pass without the radiance buffer (memory short) would run a pixel's
+  // samples in one warp: the wavefront is quicker then
+  const uint64_t paths = (uint64_t)n * tp.spp;
   bool wavefront = cache || use_wavefront(ctx, tp.spp);
-  if (!wavefront || (!cache && picks_megakernel_forward(ctx, (uint64_t)n * tp.spp))) {
-    L = forward_launcher(ctx, (uint64_t)n * tp.spp);
-    wavefront = wavefront && L.rad_cap < (uint64_t)n * tp.spp;
+  if (!wavefront || (!cache && picks_megakernel_forward(ctx, paths))) {
+    ensure_rad(ctx, paths);
+    wavefront = wavefront && ctx->L.rad_cap < paths;
   }
   if (wavefront) {
     ipt_status st = ensure_wf(ctx, false, 10u * s->n_seg);
@@ -396,7 +416,7 @@ ipt_status run_forward(ipt_ctx* ctx, int32_t scene_id, DeviceScene* s, uint32_t 
     tpk.pick = pick;
     tpk.serial_sums = use_wavefront(ctx, tp.spp);  // picked for its size: the wavefront's image
     Timed tm(ctx, IPT_KERNEL_FORWARD);
-    IPT_CK(ipt::launch_forward(L, buffers(ctx, s), s->tab, s->views_dev, (uint32_t)s->views.size(), begin, n,
+    IPT_CK(ipt::launch_forward(ctx->L, buffers(ctx, s), s->tab, s->views_dev, (uint32_t)s->views.size(), begin, n,
                                tpk, img, msq, target, g_out, partials, g_scale, loss_kind, ctx->err_dev,
                                ctx->stream));
   }
@@ -689,13 +709,14 @@ ipt_status ipt_destroy(ipt_ctx* ctx) {
     }
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   for (DeviceScene* s : ctx->scenes) free_scene(s);
-  wf_release(ctx);
+  wf_release(ctx, false);
+  for (void* p : ctx->wf_kept) cudaFree(p);
+  for (void* p : ctx->rad_owned) cudaFree(p);
   if (ctx->wf_tab) cudaFree(ctx->wf_tab);
   resolve_timings(ctx);
   for (cudaEvent_t e : ctx->spare_events) cudaEventDestroy(e);
   if (ctx->counters_dev) cudaFree(ctx->counters_dev);
   if (ctx->err_dev) cudaFree(ctx->err_dev);
-  if (ctx->L.rad) cudaFree(ctx->L.rad);
   if (ctx->loss_host) cudaFreeHost(ctx->loss_host);
   if (ctx->own_stream) cudaStreamDestroy(ctx->stream);
   delete ctx;
@@ -1095,8 +1116,8 @@ ipt_status ipt_config_set(ipt_ctx* ctx, const ipt_config* cfg) {
   const uint32_t old_cap = ctx->cfg.wavefront_slots ? ctx->cfg.wavefront_slots : (1u << 20);
   const uint32_t new_cap = cfg->wavefront_slots ? cfg->wavefront_slots : (1u << 20);
   if (old_cap != new_cap || cfg->blocks_per_sm != ctx->cfg.blocks_per_sm) {
-    IPT_CK(cudaStreamSynchronize(ctx->stream));
-    wf_release(ctx);
+    const ipt_status st = wf_release(ctx, capturing(ctx));
+    if (st != IPT_OK) return st;
   }
   ctx->cfg = *cfg;
   ctx->cfg_set = true;

@@ -206,6 +206,9 @@ struct ipt_ctx {
   bool cfg_set = false;  // ipt_config_set was called: every pass runs the integrator it names
   ipt::WfBuffers wf;
   std::vector<void*> wf_owned;
+  bool wf_captured = false;       // a graph of the caller's holds the wavefront buffers
+  std::vector<void*> wf_kept;     // buffers that graphs hold, after their growth or release
+  std::vector<void*> rad_owned;   // radiance buffers; L.rad is the last
   bool wf_adjoint = false;
   // bumped whenever device buffers that a captured batch graph may use are
   // reallocated (wavefront state, pixel-batch buffers): a batch whose graph
@@ -234,7 +237,7 @@ ipt::TraceParams trace_params(const ipt_ctx* ctx, int32_t scene, const ipt_trace
                               uint32_t spp, uint64_t it);
 ipt_status ensure_pick(ipt_ctx* ctx, DeviceScene* s, uint32_t batch);
 ipt_status ensure_tables(ipt_ctx* ctx, DeviceScene* s, const float* params, const float* sparams);
-void wf_release(ipt_ctx* c);
+ipt_status wf_release(ipt_ctx* c, bool under_capture);
 // Wavefront state for the context's chunk size; an adjoint caller passes
 // the trace's max_depth (the per-vertex carry holds that many vertices) and
 // the S x 10 (or S x 16) parameters of its widest chunk.  Capacities only

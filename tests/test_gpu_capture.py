@@ -10,7 +10,7 @@ from paper_1903_07145_gb300 import scenes
 from paper_1903_07145_gb300.tracer import TraceOptions, Tracer
 
 pytestmark = pytest.mark.gpu
-MODES = ["wavefront", "megakernel"]
+MODES = ["unset", "wavefront", "megakernel"]  # unset: the integrator by the size of the pass
 OPTS = TraceOptions(spp_r=9, spp_d=3, max_depth=3)
 PICKS = TraceOptions(spp_r=9, spp_d=3, max_depth=3, pixel_batch=33)
 
@@ -76,3 +76,37 @@ def test_replays_repeat_the_call(mode):
             assert _same(k, got[k], want[k]), k
         tr.synchronize()
         tr.close()
+
+
+SMALL, LARGE = TraceOptions(spp_r=1, spp_d=1, max_depth=3), TraceOptions(spp_r=256, spp_d=128, max_depth=6)
+
+
+@pytest.mark.parametrize("warm", ["same", "smaller"])
+def test_a_capture_allocates_what_its_pass_needs(warm):
+    """A program that set no integrator captures passes on either side of the
+    size rule, warmed up by the same pass or by a smaller one on the other
+    integrator."""
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        ref, w = _tracer("unset")
+        for opts in (SMALL, OPTS, LARGE):
+            want = ref.render(opts), ref.backward(w, opts)
+            tr, _ = _tracer("unset")
+            tr.render(opts if warm == "same" else SMALL), tr.backward(w, opts if warm == "same" else SMALL)
+            stream.synchronize()
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream):
+                got = tr.render(opts), tr.backward(w, opts)
+            first = [v.clone() for v in (tr.render(SMALL), tr.backward(w, SMALL))]
+            # what a larger call allocates afterwards leaves the graph its buffers
+            tr.render(LARGE, iteration=4), tr.backward(w, LARGE, iteration=4)
+            for v in got:
+                v.fill_(float("nan"))
+            for _ in range(2):
+                g.replay()
+                assert _same("render", got[0], want[0]) and _same("backward", got[1], want[1])
+            again = tr.render(SMALL), tr.backward(w, SMALL)
+            assert _same("render", again[0], first[0]) and _same("backward", again[1], first[1])
+            tr.synchronize()
+            tr.close()
+        ref.close()
