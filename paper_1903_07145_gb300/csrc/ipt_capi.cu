@@ -154,23 +154,24 @@ ipt_status ensure_pick(ipt_ctx* ctx, DeviceScene* s, uint32_t batch) {
   return IPT_OK;
 }
 
+// Whether the caller captures the context's stream (or, for the legacy
+// stream, another one: nothing may be waited for either way).
+bool capturing(const ipt_ctx* ctx) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 ipt_status ensure_tables(ipt_ctx* ctx, DeviceScene* s, const float* params, const float* sparams) {
   const bool is_ctx = (params == s->params) && (sparams == nullptr || sparams == s->params);
-  if (is_ctx && s->tab_is_ctx) return IPT_OK;
+  s->tab_captured = s->tab_captured || capturing(ctx);
+  if (is_ctx && s->tab_is_ctx && !s->tab_captured) return IPT_OK;
   Timed tm(ctx, IPT_KERNEL_PREPARE);
   IPT_CK(ipt::launch_prepare(buffers(ctx, s), s->tab, params, sparams ? sparams : params, ctx->stream));
   s->tab_is_ctx = is_ctx;
   s->tab_batch = -1;
   return IPT_OK;
-}
-
-// Whether the caller captures the context's stream (or, for the legacy
-// stream, another one: nothing may be waited for either way).
-static bool capturing(const ipt_ctx* ctx) {
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
-  cudaGetLastError();
-  return true;
 }
 
 // cudaMalloc, also while the caller captures a stream in any mode (an
@@ -1010,6 +1011,7 @@ ipt_status ipt_adam_step(ipt_ctx* ctx, int32_t scene, const float* grad, const i
   IPT_CK(ipt::launch_adam(buffers(ctx, s), s->tab, s->params, s->adam_m, s->adam_v, s->free_mask, s->grad_acc, grad,
                           s->step_dev, adam_host(adam), loss, s->guard_dev, ctx->err_dev, ctx->stream));
   s->tab_is_ctx = true;  // the Adam kernel rebuilt the tables from the new parameters
+  s->tab_captured = s->tab_captured || capturing(ctx);
   s->tab_batch = -1;
   return IPT_OK;
 }

@@ -253,7 +253,8 @@ ipt_status ipt_batch_step(ipt_ctx* ctx, int32_t batch, const ipt_trace_opts* opt
   // the members' parameter tables (shared with the single-scene calls) hold
   // the batch's parameters unless a single-scene call rebuilt them since
   bool stale = false;
-  for (int32_t id : b->members) stale = stale || ctx->scenes[id]->tab_batch != batch;
+  for (int32_t id : b->members)
+    stale = stale || ctx->scenes[id]->tab_batch != batch || ctx->scenes[id]->tab_captured;
   if (stale) {
     IPT_CK(ipt::launch_prepare_batch(b->mem_dev, (uint32_t)b->members.size(), b->params, ctx->stream));
     for (int32_t id : b->members) ctx->scenes[id]->tab_batch = batch;

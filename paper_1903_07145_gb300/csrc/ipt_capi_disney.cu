@@ -76,7 +76,8 @@ ipt::WfScene disney_entry(const ipt_ctx* ctx, int32_t scene, const DeviceScene* 
 }
 
 ipt_status disney_tables(ipt_ctx* ctx, DeviceScene* s, DisneyState* d, const float* sparams) {
-  if (!sparams && d->tab_is_ctx) return IPT_OK;
+  d->tab_captured = d->tab_captured || capturing(ctx);
+  if (!sparams && d->tab_is_ctx && !d->tab_captured) return IPT_OK;
   Timed tm(ctx, IPT_KERNEL_PREPARE);
   IPT_CK(ipt::launch_disney_tables(buffers(ctx, s), d->tab, d->dt, d->params, sparams, ctx->stream));
   d->tab_is_ctx = sparams == nullptr;

@@ -79,6 +79,7 @@ struct DisneyState {
   ipt::SegBuffers tab{};     // emission, light selection (mat_a, mat_b unused)
   ipt::DisneyBuffers dt{};
   bool tab_is_ctx = false;
+  bool tab_captured = false;  // as DeviceScene's
   uint64_t iteration = 0;
   std::vector<void*> owned;
 };
@@ -112,6 +113,9 @@ struct DeviceScene {
   // parameter tables
   ipt::SegBuffers tab{};
   bool tab_is_ctx = false;  // tables were built from the context's own parameters
+  // a graph of the caller's builds the tables, whenever it is replayed: every
+  // call builds its own from then on, and so does every capture
+  bool tab_captured = false;
   int32_t tab_batch = -1;   // batch whose parameters built the tables (-1: a single-scene call did)
   // parameters and optimiser state
   float* params = nullptr;
@@ -236,6 +240,7 @@ ipt_status check_opts(ipt_ctx* ctx, const ipt_trace_opts* o, bool adjoint, bool 
 ipt::TraceParams trace_params(const ipt_ctx* ctx, int32_t scene, const ipt_trace_opts* o, uint32_t set,
                               uint32_t spp, uint64_t it);
 ipt_status ensure_pick(ipt_ctx* ctx, DeviceScene* s, uint32_t batch);
+bool capturing(const ipt_ctx* ctx);
 ipt_status ensure_tables(ipt_ctx* ctx, DeviceScene* s, const float* params, const float* sparams);
 ipt_status wf_release(ipt_ctx* c, bool under_capture);
 // Wavefront state for the context's chunk size; an adjoint caller passes

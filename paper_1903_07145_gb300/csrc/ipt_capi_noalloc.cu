@@ -54,7 +54,8 @@ extern "C" ipt_status ipt_backward_noalloc(ipt_ctx* ctx, int32_t scene, const ip
   IPT_CK(noalloc_scratch(ctx, &acc));
   const float* p = params ? params : s->params;
   const bool is_ctx = (p == s->params) && (sampling_params == nullptr || sampling_params == s->params);
-  if (!(is_ctx && s->tab_is_ctx)) {
+  s->tab_captured = s->tab_captured || capturing(ctx);
+  if (!(is_ctx && s->tab_is_ctx) || s->tab_captured) {
     Timed tm(ctx, IPT_KERNEL_PREPARE);
     IPT_CK(ipt::launch_prepare(buffers(ctx, s), s->tab, p, sampling_params ? sampling_params : p, ctx->stream));
     s->tab_is_ctx = is_ctx;

@@ -81,18 +81,19 @@ def test_replays_repeat_the_call(mode):
 SMALL, LARGE = TraceOptions(spp_r=1, spp_d=1, max_depth=3), TraceOptions(spp_r=256, spp_d=128, max_depth=6)
 
 
-@pytest.mark.parametrize("warm", ["same", "smaller"])
+@pytest.mark.parametrize("warm", ["same", "smaller", "none"])
 def test_a_capture_allocates_what_its_pass_needs(warm):
     """A program that set no integrator captures passes on either side of the
-    size rule, warmed up by the same pass or by a smaller one on the other
-    integrator."""
+    size rule, warmed up by the same pass, by a smaller one on the other
+    integrator, or not at all."""
     stream = torch.cuda.Stream()
     with torch.cuda.stream(stream):
         ref, w = _tracer("unset")
         for opts in (SMALL, OPTS, LARGE):
             want = ref.render(opts), ref.backward(w, opts)
             tr, _ = _tracer("unset")
-            tr.render(opts if warm == "same" else SMALL), tr.backward(w, opts if warm == "same" else SMALL)
+            if warm != "none":
+                tr.render(opts if warm == "same" else SMALL), tr.backward(w, opts if warm == "same" else SMALL)
             stream.synchronize()
             g = torch.cuda.CUDAGraph()
             with torch.cuda.graph(g, stream=stream):
@@ -110,3 +111,42 @@ def test_a_capture_allocates_what_its_pass_needs(warm):
             tr.synchronize()
             tr.close()
         ref.close()
+
+
+def test_tables_follow_the_parameters_through_replays():
+    """A call uses the parameters it is given, or the scene's at that time,
+    whatever the calls around it (eager or replayed) built tables from."""
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        tr, _ = _tracer("wavefront")
+        sc = tr.scene
+        rng = np.random.default_rng(8)
+        own, new, other = (np.asarray(sc.gt_params * s, np.float32) for s in (1.0, 0.7, 0.4))
+        given = torch.from_numpy(other).cuda()
+        mats = [scenes.disney_materials(sc, k) for k in (3, 5)]
+        spare = torch.from_numpy(scenes.disney_materials(sc, 9)).cuda()
+        r = lambda **k: tr.render(OPTS, **k).clone()  # noqa: E731
+        d = lambda **k: tr.disney_render(OPTS, **k).clone()  # noqa: E731
+        want = {}
+        for name, p, m in (("new", new, mats[1]), ("own", own, mats[0])):
+            tr.set_params(p), tr.disney_set_params(m)
+            want[name] = r(), r(params=given), d(), d(sampling_params=spare)
+        stream.synchronize()
+        g = [torch.cuda.CUDAGraph() for _ in range(4)]
+        outs = []
+        for graph, f in zip(g, (lambda: tr.render(OPTS), lambda: tr.render(OPTS, params=given),
+                                lambda: tr.disney_render(OPTS),
+                                lambda: tr.disney_render(OPTS, sampling_params=spare))):
+            with torch.cuda.graph(graph, stream=stream):
+                outs.append(f())
+        for name in ("own", "new"):
+            if name == "new":
+                tr.set_params(new), tr.disney_set_params(mats[1])
+            for order in rng.permuted(np.tile(np.arange(4), (6, 1)), axis=1):
+                for k in order:
+                    g[k].replay()
+                    assert torch.equal(outs[k], want[name][k])
+                    assert torch.equal(r(), want[name][0]) and torch.equal(d(), want[name][2])
+                    r(params=given), d(sampling_params=spare)
+        tr.synchronize()
+        tr.close()
