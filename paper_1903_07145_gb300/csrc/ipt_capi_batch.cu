@@ -257,7 +257,10 @@ ipt_status ipt_batch_step(ipt_ctx* ctx, int32_t batch, const ipt_trace_opts* opt
     stale = stale || ctx->scenes[id]->tab_batch != batch || ctx->scenes[id]->tab_captured;
   if (stale) {
     IPT_CK(ipt::launch_prepare_batch(b->mem_dev, (uint32_t)b->members.size(), b->params, ctx->stream));
-    for (int32_t id : b->members) ctx->scenes[id]->tab_batch = batch;
+    for (int32_t id : b->members) {
+      ctx->scenes[id]->tab_batch = batch;
+      ctx->scenes[id]->tab_is_ctx = false;
+    }
   }
   {
     Timed tm(ctx, IPT_KERNEL_BATCH_STEP);
