@@ -322,13 +322,17 @@ bool use_wavefront(const ipt_ctx* ctx, uint32_t spp) {
 //                61k    .46 | .16    .56 | .27    .71 | .36    .82 | .65   1.05 | 1.20
 //   ipt_backward  3k    .52 | .16    .60 | .23    .72 | .54    .80 | 1.01  1.13 | 1.85
 //                61k    .63 | .19    .74 | .28    .91 | .71   1.01 | 1.27  1.42 | 2.36
-// Hence 28 and 14 warps of paths an SM (136192 and 68096 paths on 152).  A
-// context with traversal counters keeps the wavefront, which counts.
+// Hence 28 and 14 warps of paths an SM (136192 and 68096 paths on 152).  The
+// samples a pixel do not matter to either pass: 66k derivative paths, 1, 7, 32,
+// 33 and 129 a pixel, ipt_loss_grad in the 3k room 1.28 | .84, 1.13 | .70, 1.07 |
+// .67, 1.07 | .66, 1.05 | .64, and with 5k segments 2.35 | 1.64, 2.21 | 1.48,
+// 2.15 | 1.45, 2.16 | 1.43, 2.13 | 1.41.  A context with traversal counters
+// keeps the wavefront, which counts.
 static bool picks_megakernel(const ipt_ctx* ctx, uint64_t n, uint32_t warps_per_sm) {
   return !ctx->cfg_set && !ctx->counters_dev && n <= 32ull * warps_per_sm * (uint32_t)ctx->L.num_sms;
 }
 bool picks_megakernel_forward(const ipt_ctx* ctx, uint64_t n) { return picks_megakernel(ctx, n, 28); }
-bool picks_megakernel_adjoint(const ipt_ctx* ctx, uint64_t n) { return picks_megakernel(ctx, n, 14); }
+bool picks_megakernel_adjoint(const ipt_ctx* ctx, uint64_t n) { return picks_megakernel(ctx, n, ipt::kFewAdjointWarps); }
 
 // Scene-table entry of one scene for a launch over its pixels
 // [pix_base, pix_base + n) (launch pixels 0..n-1).

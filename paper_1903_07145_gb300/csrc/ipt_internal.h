@@ -181,6 +181,11 @@ int loss_partials_capacity(const Launcher& L);
 // (their radiances, 16 bytes each, go through Launcher::rad, grown on demand;
 // a launch that it cannot hold keeps a pixel's samples in one warp).
 constexpr uint32_t kFewSamples = 1u << 20;
+// Warps of paths an SM up to which a derivative pass runs one path a thread on
+// the megakernel, and up to which a pass of a program that set no integrator
+// is given to it: one limit, as the form beyond it traces a pixel's paths on
+// as many lanes as divide them, one after the other for an odd number.
+constexpr uint32_t kFewAdjointWarps = 14;
 
 cudaError_t launch_prepare(const SceneBuffers& s, const SegBuffers& t, const float* params,
                            const float* sparams, cudaStream_t st);

@@ -893,9 +893,13 @@ static uint32_t few_lanes(const Launcher& L, uint64_t n) {
 
 // The residual pass runs one sample a thread up to the capacity of the
 // radiance buffer; the derivative pass, whose blocks each clear and flush
-// their accumulators, up to one wave of warps.
+// their accumulators, up to kFewAdjointWarps.  Above 8 warps an SM the blocks
+// come in more than one wave; with `group` lanes a pixel there instead, 527
+// pixels of 129 paths (a 3k-triangle room, depth 5, the whole call) took 31.5
+// ms for 0.64, 2060 of 33 8.3 for 0.66, and 2125 of 32 the same 0.66 (5k
+// segments: 45 for 1.4, 11.7 for 1.4, and 1.39 for 1.45).
 static bool few_forward(const Launcher& L, uint64_t n) { return n <= L.rad_cap; }
-static bool few_adjoint(const Launcher& L, uint64_t n) { return n <= 32ull * kFewWarpsPerSm * (uint32_t)L.num_sms; }
+static bool few_adjoint(const Launcher& L, uint64_t n) { return n <= 32ull * kFewAdjointWarps * (uint32_t)L.num_sms; }
 
 // In-order sums: a group loads what it can of a pixel's samples at once, its
 // size need not divide their number.
