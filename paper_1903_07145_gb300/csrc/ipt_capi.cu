@@ -616,18 +616,42 @@ ipt_status read_loss(ipt_ctx* ctx, DeviceScene* s, double* loss_out, uint64_t n_
   return IPT_OK;
 }
 
+// Waits for the stream's work and the error word that comes with it.
+static ipt_status wait_for_stream(ipt_ctx* ctx) {
+  IPT_CK(cudaMemcpyAsync(ctx->err_host, ctx->err_dev, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
+  IPT_CK(cudaStreamSynchronize(ctx->stream));
+  return IPT_OK;
+}
+
+// The error word that a wait brought back, as a status; clears it.
+static ipt_status device_status(ipt_ctx* ctx) {
+  const uint32_t err = *ctx->err_host;
+  if (err) {
+    cudaMemset(ctx->err_dev, 0, sizeof(uint32_t));
+    if (err & ipt::kErrStack)
+      return fail(ctx, IPT_ERR_CUDA, "device error word " + std::to_string(err) + " (traversal stack overflow)");
+    if (err & ipt::kErrTimeout)
+      return fail(ctx, IPT_ERR_TIMEOUT,
+                  "a bounded wait for the tensor cores gave up in the radiance cache's training pass; its "
+                  "gradients are incomplete");
+    return fail(ctx, IPT_ERR_NONFINITE,
+                "non-finite loss or gradient: the Adam step was skipped, parameters and Adam state are those of "
+                "the last good step");
+  }
+  return IPT_OK;
+}
+
 // Small results go through pinned memory (a copy to pageable memory waits by
 // itself: reading the 64 members'
 // parameters of a batch and checking the error word took 27 us each, 17 us here).
+// What an earlier call staged is not handed out when the wait fails.
 ipt_status read_back(ipt_ctx* ctx, void* dst, const void* src, size_t n) {
-  if (n > kStageBytes) {
-    IPT_CK(cudaMemcpyAsync(dst, src, n, cudaMemcpyDeviceToHost, ctx->stream));
-    return ipt_synchronize(ctx);
-  }
-  IPT_CK(cudaMemcpyAsync(ctx->stage_host, src, n, cudaMemcpyDeviceToHost, ctx->stream));
-  const ipt_status st = ipt_synchronize(ctx);
-  std::memcpy(dst, ctx->stage_host, n);
-  return st;
+  const bool staged = n <= kStageBytes;
+  IPT_CK(cudaMemcpyAsync(staged ? ctx->stage_host : dst, src, n, cudaMemcpyDeviceToHost, ctx->stream));
+  const ipt_status st = wait_for_stream(ctx);
+  if (st != IPT_OK) return st;
+  if (staged) std::memcpy(dst, ctx->stage_host, n);
+  return device_status(ctx);
 }
 
 ipt::AdamHost adam_host(const ipt_adam_opts* a) {
@@ -1069,23 +1093,8 @@ ipt_status ipt_philox(ipt_ctx* ctx, uint32_t n, const uint32_t* ctr, const uint3
 ipt_status ipt_synchronize(ipt_ctx* ctx) {
   if (!ctx) return IPT_ERR_INVALID_ARG;
   IPT_CK(cudaSetDevice(ctx->device));
-  // one wait for the stream's work and the error word
-  IPT_CK(cudaMemcpyAsync(ctx->err_host, ctx->err_dev, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream));
-  IPT_CK(cudaStreamSynchronize(ctx->stream));
-  const uint32_t err = *ctx->err_host;
-  if (err) {
-    cudaMemset(ctx->err_dev, 0, sizeof(uint32_t));
-    if (err & ipt::kErrStack)
-      return fail(ctx, IPT_ERR_CUDA, "device error word " + std::to_string(err) + " (traversal stack overflow)");
-    if (err & ipt::kErrTimeout)
-      return fail(ctx, IPT_ERR_TIMEOUT,
-                  "a bounded wait for the tensor cores gave up in the radiance cache's training pass; its "
-                  "gradients are incomplete");
-    return fail(ctx, IPT_ERR_NONFINITE,
-                "non-finite loss or gradient: the Adam step was skipped, parameters and Adam state are those of "
-                "the last good step");
-  }
-  return IPT_OK;
+  const ipt_status st = wait_for_stream(ctx);
+  return st == IPT_OK ? device_status(ctx) : st;
 }
 
 ipt_status ipt_scene_info(ipt_ctx* ctx, int32_t scene, uint32_t* n_tri, uint32_t* n_seg, uint32_t* n_nodes,

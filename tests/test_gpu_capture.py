@@ -150,3 +150,24 @@ def test_tables_follow_the_parameters_through_replays():
                     r(params=given), d(sampling_params=spare)
         tr.synchronize()
         tr.close()
+
+
+def test_a_read_that_cannot_wait_leaves_its_output():
+    """A call that returns host data fails under capture; it does not hand out
+    what an earlier call read."""
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        tr, _ = _tracer("wavefront")
+        before = tr.get_params()
+        assert np.isfinite(before).all()
+        out = np.full_like(before, np.nan)
+        g = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        g.capture_begin()
+        with pytest.raises(L.IptError):
+            L.ipt_params_get(tr.ctx, tr.sid, out.ctypes.data)
+        with pytest.raises(RuntimeError):
+            g.capture_end()
+        assert np.isnan(out).all()
+        np.testing.assert_array_equal(tr.get_params(), before)
+        tr.close()
