@@ -15,6 +15,7 @@ ipt_status fail(ipt_ctx* c, ipt_status s, const std::string& msg) {
 }
 
 ipt_status cuda_fail(ipt_ctx* c, cudaError_t e, const char* where) {
+  cudaGetLastError();  // reported here: the next launch's check must not find it again
   return fail(c, e == cudaErrorMemoryAllocation ? IPT_ERR_OUT_OF_MEMORY : IPT_ERR_CUDA,
               std::string(where) + ": " + cudaGetErrorString(e));
 }

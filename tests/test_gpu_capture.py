@@ -171,3 +171,20 @@ def test_a_read_that_cannot_wait_leaves_its_output():
         assert np.isnan(out).all()
         np.testing.assert_array_equal(tr.get_params(), before)
         tr.close()
+
+
+def test_an_error_is_reported_once():
+    """A call that failed under capture does not fail the next one."""
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        tr, w = _tracer("wavefront")
+        want = tr.render(OPTS).clone()
+        g = torch.cuda.CUDAGraph()
+        torch.cuda.synchronize()
+        g.capture_begin()
+        with pytest.raises(L.IptError):
+            tr.get_params()
+        with pytest.raises(RuntimeError):
+            g.capture_end()
+        assert torch.equal(tr.render(OPTS), want)
+        tr.close()
