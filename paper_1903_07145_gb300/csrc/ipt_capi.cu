@@ -302,14 +302,14 @@ void ensure_rad(ipt_ctx* ctx, uint64_t n) {
   ctx->L.rad_cap = want;
 }
 
-bool use_wavefront_cap(const ipt_ctx* ctx, uint32_t spp) {
-  const uint32_t cap = ctx->cfg.wavefront_slots ? ctx->cfg.wavefront_slots : (1u << 20);
-  return spp <= cap;
+static uint32_t wavefront_slots(const ipt_ctx* ctx) {
+  return ctx->cfg.wavefront_slots ? ctx->cfg.wavefront_slots : (1u << 20);
 }
 
+bool use_wavefront_cap(const ipt_ctx* ctx, uint32_t spp) { return spp <= wavefront_slots(ctx); }
+
 bool use_wavefront(const ipt_ctx* ctx, uint32_t spp) {
-  const uint32_t cap = ctx->cfg.wavefront_slots ? ctx->cfg.wavefront_slots : (1u << 20);
-  return ctx->cfg.integrator == 1 && spp <= cap;
+  return ctx->cfg.integrator == 1 && spp <= wavefront_slots(ctx);
 }
 
 // Whether a pass of n paths of a context whose program has set no integrator
@@ -386,13 +386,14 @@ ipt_status run_forward(ipt_ctx* ctx, int32_t scene_id, DeviceScene* s, uint32_t 
                        uint32_t* pick) {
   if (cache && !use_wavefront_cap(ctx, tp.spp))
     return fail(ctx, IPT_ERR_INVALID_ARG, "cached passes need spp <= wavefront_slots");
-  // a pass without the radiance buffer (memory short) would run a pixel's
-  // samples in one warp: the wavefront is quicker then
+  // a pass that finds no memory for its radiances (16 bytes a sample) runs the
+  // wavefront if its buffers (162 bytes a slot) are there, and else the form
+  // that needs none: a pixel's samples in one warp
   const uint64_t paths = (uint64_t)n * tp.spp;
   bool wavefront = cache || use_wavefront(ctx, tp.spp);
   if (!wavefront || (!cache && picks_megakernel_forward(ctx, paths))) {
     ensure_rad(ctx, paths);
-    wavefront = wavefront && ctx->L.rad_cap < paths;
+    wavefront = wavefront && ctx->L.rad_cap < paths && ctx->wf.cap == wavefront_slots(ctx);
   }
   if (wavefront) {
     ipt_status st = ensure_wf(ctx, false, 10u * s->n_seg);
