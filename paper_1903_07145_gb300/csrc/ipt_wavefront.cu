@@ -1795,13 +1795,16 @@ __global__ void wf_wide_reduce(const float* gacc, uint32_t np, double* grad_acc)
 // Pixel batches (Sec. 4.5): entry b of a scene with N pixels is
 // floor(x * N / 2^32), x the first word of Philox4x32-10 at the scene's key
 // and counter (b, 0, (4 << 24) | iteration, 0).  Launch pixels of scenes
-// without a batch are skipped.
+// without a batch are skipped.  kOne: a single scene's draw, its entry the
+// kernel parameter (no table to fill before it).
 constexpr uint32_t kSetPick = 4u;
-__global__ void __launch_bounds__(kWfThreads) wf_pick_k(const WfScene* tab, uint32_t n_scenes, uint32_t n_launch,
+template <bool kOne>
+__global__ void __launch_bounds__(kWfThreads) wf_pick_k(const WfScene* tab, const __grid_constant__ WfScene one,
+                                                        uint32_t n_scenes, uint32_t n_launch,
                                                         const uint32_t* iter_dev, uint32_t iter) {
   const uint32_t it = iter_dev ? *iter_dev : iter;
   for (uint32_t P = blockIdx.x * blockDim.x + threadIdx.x; P < n_launch; P += gridDim.x * blockDim.x) {
-    uint32_t lo = 0, hi = n_scenes - 1;
+    uint32_t lo = 0, hi = kOne ? 0u : n_scenes - 1;
     while (lo < hi) {
       const uint32_t mid = (lo + hi + 1) >> 1;
       if (tab[mid].pix_begin <= P)
@@ -1809,7 +1812,7 @@ __global__ void __launch_bounds__(kWfThreads) wf_pick_k(const WfScene* tab, uint
       else
         hi = mid - 1;
     }
-    const WfScene& e = tab[lo];
+    const WfScene& e = kOne ? one : tab[lo];
     if (!e.pick) continue;
     const uint32_t b = P - e.pix_begin;
     const uint4 x = philox4x32_10(make_uint4(b, 0u, (kSetPick << 24) | (it & 0xffffffu), 0u), e.key);
@@ -2327,7 +2330,8 @@ cudaError_t wf_pick(const WfScene* tab_dev, const std::vector<WfScene>& tab, con
   const WfScene& last = tab.back();
   const uint32_t n_launch = last.pix_begin + last.n_pix;
   const uint32_t blocks = std::min<uint32_t>((n_launch + kWfThreads - 1) / kWfThreads, 4096u);
-  wf_pick_k<<<std::max(blocks, 1u), kWfThreads, 0, st>>>(tab_dev, (uint32_t)tab.size(), n_launch, iter_dev, iter);
+  const auto k = tab_dev ? wf_pick_k<false> : wf_pick_k<true>;
+  k<<<std::max(blocks, 1u), kWfThreads, 0, st>>>(tab_dev, tab[0], (uint32_t)tab.size(), n_launch, iter_dev, iter);
   return cudaGetLastError();
 }
 

@@ -69,7 +69,8 @@ cudaError_t wf_forward(const Launcher& L, const WfScene* tab_dev, const std::vec
 cudaError_t wf_set_entry(const WfScene& e, WfScene* tab_dev, cudaStream_t st);
 
 // Draws the pixel batch of every table entry that has one, for the iteration
-// *iter_dev (or iter when iter_dev is null).
+// *iter_dev (or iter when iter_dev is null).  A table of one scene may stay on
+// the host (tab_dev null).
 cudaError_t wf_pick(const WfScene* tab_dev, const std::vector<WfScene>& tab, const uint32_t* iter_dev,
                     uint32_t iter, cudaStream_t st);
 
