@@ -374,7 +374,10 @@ __device__ __forceinline__ uint32_t node4_children(const SceneDev& s, int node, 
 // Rounding: with C = (lo - o) / d, the errors of A, B and the fma are below
 // 2^-22 (|A| + |C|), relative rounding of t included (|t| <= |A| + |C|).
 // Near planes use B - m, far planes B + m, m = 2^-21 (|A| + |C|): 2^-5 of a
-// grid step for an origin inside the grid, growing with its distance.
+// grid step for an origin inside the grid, growing with its distance.  m is
+// finite: an origin so far off that C is infinite (the distances overflow)
+// keeps its planes at that infinity and misses, where B - m and B + m would be
+// NaN on one side and accept every child, empty slots among them.
 // ---------------------------------------------------------------------------
 struct GridRay {
   float Ax, Ay, Az, Bnx, Bny, Bnz, Bfx, Bfy, Bfz;
@@ -386,7 +389,7 @@ __device__ __forceinline__ void grid_axis(float lo, float s, float o, float inv,
   A = s * inv;
   const float C = (lo - o) * inv;
   const float B = fmaf(lo - o, inv, -A);
-  const float m = 0x1p-21f * (fabsf(A) + fabsf(C));
+  const float m = fminf(0x1p-21f * (fabsf(A) + fabsf(C)), 0x1.fffffep127f);
   Bn = B - m;
   Bf = B + m;
   sel = inv < 0.0f ? 0x7324u : 0x7104u;  // bytes: 0, plane low, plane high, 0x3F
