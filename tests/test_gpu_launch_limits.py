@@ -38,17 +38,16 @@ def _sizes():
     return out
 
 
-@pytest.mark.parametrize("per_triangle", [False, True])
-def test_derivative_passes_around_the_limits(per_triangle):
+@pytest.mark.parametrize("sub", [0, 6, 9])
+def test_derivative_passes_around_the_limits(sub):
     """Gradients agree with the wavefront's to the rounding of FP32 sums in
-    another order (rel 1e-5), with accumulators in shared memory and (a
-    segment per triangle, above 2400) in global memory."""
-    if per_triangle:
-        sc = scenes.per_triangle(scenes.indoor_room(9, n_cuboids=6, cuboid_sub=6, room_sub=4, n_lights=2, n_views=2,
+    another order (rel 1e-5), with accumulators in shared memory (few segments,
+    and a segment per triangle) and in global memory (above 5120 segments)."""
+    sc = _room()
+    if sub:
+        sc = scenes.per_triangle(scenes.indoor_room(9, n_cuboids=6, cuboid_sub=sub, room_sub=4, n_lights=2, n_views=2,
                                                     width=40, height=31))
-        assert sc.n_segments > 2400
-    else:
-        sc = _room()
+        assert (sc.n_segments > 5120) == (sub == 9)
     tracers = {k: _tracer(k, sc) for k in ("wavefront", "megakernel", "unset")}
     for batch, spp_d in _sizes():
         opts = TraceOptions(spp_r=1, spp_d=spp_d, max_depth=3, pixel_batch=batch)
