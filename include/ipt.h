@@ -24,7 +24,7 @@
  *     synchronising call returns: a traversal stack overflow as IPT_ERR_CUDA,
  *     a non-finite loss or gradient met by an Adam step as IPT_ERR_NONFINITE,
  *     a bounded wait for the tensor cores that gave up (radiance-cache
- *     training) as IPT_ERR_TIMEOUT.
+ *     queries and training) as IPT_ERR_TIMEOUT.
  *   - Non-finite guard: every Adam step (ipt_adam_step, ipt_step,
  *     ipt_batch_step per member, ipt_disney_step) first checks, on the device,
  *     the gradient it is given and, for the context's own gradient, the loss

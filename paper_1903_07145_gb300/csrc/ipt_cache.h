@@ -62,7 +62,7 @@ struct CacheOut {
   float* gw;      // training: weight gradients (accumulated)
   float2* gt;     // training: hash-table gradients (accumulated)
   double* loss;   // training: sum over rows and channels of the relative L2 terms
-  uint32_t* err;  // training: error word (kErrTimeout), nullable
+  uint32_t* err;  // error word (kErrTimeout), nullable
 };
 
 // Query and record buffers of the wavefront integrator.

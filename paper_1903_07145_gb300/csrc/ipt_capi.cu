@@ -632,8 +632,8 @@ static ipt_status device_status(ipt_ctx* ctx) {
       return fail(ctx, IPT_ERR_CUDA, "device error word " + std::to_string(err) + " (traversal stack overflow)");
     if (err & ipt::kErrTimeout)
       return fail(ctx, IPT_ERR_TIMEOUT,
-                  "a bounded wait for the tensor cores gave up in the radiance cache's training pass; its "
-                  "gradients are incomplete");
+                  "a bounded wait for the tensor cores gave up in the radiance cache; the predictions or training "
+                  "gradients of that call are incomplete");
     return fail(ctx, IPT_ERR_NONFINITE,
                 "non-finite loss or gradient: the Adam step was skipped, parameters and Adam state are those of "
                 "the last good step");

@@ -221,6 +221,7 @@ ipt_status ipt_cache_eval(ipt_ctx* ctx, int32_t scene, uint32_t n, const float* 
   ipt::CacheOut o{};
   o.rgb = rgb_out;
   o.dp7 = vjp ? dparams_out : nullptr;
+  o.err = ctx->err_dev;
   if (!apart) {
     if ((st = cache_api_out(ctx, c, n)) != IPT_OK) return st;
     o.rgb = c->api_out;

@@ -2165,6 +2165,7 @@ cudaError_t wf_forward(const Launcher& L, const WfScene* tab_dev, const std::vec
       IPT_STAGE(16);
       CacheOut o{};
       o.rad = wb.rad;
+      o.err = err;
       cudaError_t e = cache_infer(cache->net, lp.cb.q, tab[0].t.mat_a, tab[0].t.mat_b, lp.cb.counts, wb.cap, o,
                                   false, L.num_sms, st);
       if (e != cudaSuccess) return e;
