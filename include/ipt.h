@@ -114,7 +114,8 @@ typedef struct {
  *   integrator: 0 = megakernel (one thread per path, every stage inline),
  *     1 = wavefront (chunks of path slots; persistent traversal kernels over
  *     compacted ray queues).  A context whose program never calls
- *     ipt_config_set reports 1 and runs the passes of ipt_render,
+ *     ipt_config_set (with any values: what ipt_config_get gave, written
+ *     back, sets the integrator too) reports 1 and runs the passes of ipt_render,
  *     ipt_backward, ipt_loss_grad(_shard), ipt_step and ipt_batch_step that
  *     have too few paths for the wavefront on the megakernel (the same paths;
  *     the timings of such a pass are IPT_KERNEL_FORWARD and
@@ -124,7 +125,11 @@ typedef struct {
  *     per slot, and once it has run an adjoint 52 + 40 D more (D: the
  *     largest max_depth its adjoints have used; the Disney model's adjoint
  *     adds 32 D + 64); the buffers are allocated on first use and grow, never
- *     shrink, while the context lives.
+ *     shrink, while the context lives.  A megakernel residual pass of up to
+ *     2^20 samples (the passes above included) keeps 16 bytes a sample,
+ *     rounded up to a power of two: at most 16 MB, and as much again of
+ *     smaller buffers that it has outgrown.  Buffers that a captured graph
+ *     holds are kept until the context ends when they grow.
  *   trace_steps: refill point of the persistent traversal kernels (0 = 16).
  *     4- and 8-wide BVHs: a warp fetches new rays once this many of its 32
  *     lanes are idle (values above 32 act as 32).  Binary BVH: node visits
@@ -184,8 +189,8 @@ typedef struct {
  *     b*spp .. b*spp+spp-1 of each set, and the loss and its gradient are
  *     normalised by the 3B entry-channels, so the batch loss is an unbiased
  *     estimate of the full-image loss.  Accepted by ipt_loss_grad, ipt_step
- *     and ipt_batch_step (every other call requires 0), on either integrator
- *     (batches of scenes: wavefront); not with the radiance cache.
+ *     and ipt_batch_step (every other call requires 0), on either integrator;
+ *     not with the radiance cache.
  *     B * max(spp_r, spp_d) must stay below 2^32. */
 typedef struct {
   uint32_t spp_r;

@@ -918,8 +918,11 @@ __global__ void __launch_bounds__(kThreads, 2)
 // groups run on their own (named barriers, an mbarrier and 128 TMEM columns
 // each) and share one image of the weights: one block per SM, whose groups'
 // gathers overlap the others' MMA round trips, and whose 130 KB leave the
-// rest of the SM's 256 KB to the L1 that the gathers go through.  The L1's
-// lookups bound the kernel (one for every line a gather touches).  4.9M rows
+// rest of the SM's 256 KB to the L1 that the gathers go through.  What bounds
+// it is the gathers' latency at 16 warps an SM: 500k random rows wait 3.7 of
+// the 9.6 cycles between a warp's instructions for them, the busiest unit is
+// the L1's path to the L2 (57% of its peak; L1 hits 19%, L2 91%), issue 42%.
+// 4.9M rows
 // of the 61k room's paths: 1.89 ms with two blocks of one group (148 KB, input
 // and activation tiles apart), 1.78 with a row's gathers of four levels issued
 // together, 1.44 with four groups (three: 1.55).
