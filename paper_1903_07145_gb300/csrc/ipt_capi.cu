@@ -371,7 +371,7 @@ ipt_status draw_picks(ipt_ctx* ctx, int32_t scene_id, const DeviceScene* s, uint
   ipt::WfScene e = wf_entry(ctx, scene_id, s, 0, B);
   e.pick = out;
   e.n_all = (uint32_t)s->n_pix;
-  IPT_CK(ipt::wf_pick(nullptr, std::vector<ipt::WfScene>{e}, nullptr, (uint32_t)iteration, ctx->stream));
+  IPT_CK(ipt::wf_pick_one(e, (uint32_t)iteration, ctx->stream));
   return IPT_OK;
 }
 

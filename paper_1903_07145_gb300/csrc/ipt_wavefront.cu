@@ -422,11 +422,11 @@ __device__ __forceinline__ uint2 st_pop(const Stack& S, Trav& T) {
   return T.sp < kShortStack ? S.sh[T.sp * kWfThreads] : S.deep[T.sp - kShortStack];
 }
 
-template <int kWidth>
+template <int kWidth, bool kFar = false>
 __device__ __forceinline__ void trav_init(const SceneDev& s, Trav& T, float3 o, float3 d, float tmax, int skip_a,
                                           int skip_b) {
   T.r = ray_pre(o, d);
-  if constexpr (kWidth == kGrid4) T.g = grid_ray(s.grid_lo, s.grid_s, T.r);
+  if constexpr (kWidth == kGrid4) T.g = grid_ray<kFar>(s.grid_lo, s.grid_s, T.r);
   T.oinv = f3(o.x * T.r.inv.x, o.y * T.r.inv.y, o.z * T.r.inv.z);
   T.tmax = tmax;
   T.skip_a = skip_a;
@@ -724,7 +724,7 @@ struct ArrayRays {
     const float* d = a.dir + 3 * (size_t)i;
     int sk = -1;
     if (a.skip && a.skip[i] >= 0 && (uint32_t)a.skip[i] < s.n_tri) sk = (int)a.orig_to_internal[a.skip[i]];
-    trav_init<kWidth>(s, T, f3(o[0], o[1], o[2]), f3(d[0], d[1], d[2]), __int_as_float(0x7f800000), sk, -1);
+    trav_init<kWidth, true>(s, T, f3(o[0], o[1], o[2]), f3(d[0], d[1], d[2]), __int_as_float(0x7f800000), sk, -1);
   }
 
   __device__ __forceinline__ void finish(uint32_t i, const Trav& T) const {
@@ -1794,17 +1794,19 @@ __global__ void wf_wide_reduce(const float* gacc, uint32_t np, double* grad_acc)
 
 // Pixel batches (Sec. 4.5): entry b of a scene with N pixels is
 // floor(x * N / 2^32), x the first word of Philox4x32-10 at the scene's key
-// and counter (b, 0, (4 << 24) | iteration, 0).  Launch pixels of scenes
-// without a batch are skipped.  kOne: a single scene's draw, its entry the
-// kernel parameter (no table to fill before it).
+// and counter (b, 0, (4 << 24) | iteration, 0).
 constexpr uint32_t kSetPick = 4u;
-template <bool kOne>
-__global__ void __launch_bounds__(kWfThreads) wf_pick_k(const WfScene* tab, const __grid_constant__ WfScene one,
-                                                        uint32_t n_scenes, uint32_t n_launch,
+__device__ __forceinline__ void draw_pick(const WfScene& e, uint32_t b, uint32_t it) {
+  const uint4 x = philox4x32_10(make_uint4(b, 0u, (kSetPick << 24) | (it & 0xffffffu), 0u), e.key);
+  e.pick[b] = (uint32_t)(((uint64_t)x.x * (uint64_t)e.n_all) >> 32);
+}
+
+// Launch pixels of scenes without a batch are skipped.
+__global__ void __launch_bounds__(kWfThreads) wf_pick_k(const WfScene* tab, uint32_t n_scenes, uint32_t n_launch,
                                                         const uint32_t* iter_dev, uint32_t iter) {
   const uint32_t it = iter_dev ? *iter_dev : iter;
   for (uint32_t P = blockIdx.x * blockDim.x + threadIdx.x; P < n_launch; P += gridDim.x * blockDim.x) {
-    uint32_t lo = 0, hi = kOne ? 0u : n_scenes - 1;
+    uint32_t lo = 0, hi = n_scenes - 1;
     while (lo < hi) {
       const uint32_t mid = (lo + hi + 1) >> 1;
       if (tab[mid].pix_begin <= P)
@@ -1812,12 +1814,17 @@ __global__ void __launch_bounds__(kWfThreads) wf_pick_k(const WfScene* tab, cons
       else
         hi = mid - 1;
     }
-    const WfScene& e = kOne ? one : tab[lo];
-    if (!e.pick) continue;
-    const uint32_t b = P - e.pix_begin;
-    const uint4 x = philox4x32_10(make_uint4(b, 0u, (kSetPick << 24) | (it & 0xffffffu), 0u), e.key);
-    e.pick[b] = (uint32_t)(((uint64_t)x.x * (uint64_t)e.n_all) >> 32);
+    const WfScene& e = tab[lo];
+    if (e.pick) draw_pick(e, P - e.pix_begin, it);
   }
+}
+
+// One scene's draw, its entry a kernel parameter: no table to fill before it (8
+// pixels on a Cornell box, the whole call: 105.6 us with the table filled by a
+// launch, 104.0 without).
+__global__ void __launch_bounds__(kWfThreads) wf_pick_one_k(const __grid_constant__ WfScene e, uint32_t iter) {
+  for (uint32_t b = blockIdx.x * blockDim.x + threadIdx.x; b < e.n_pix; b += gridDim.x * blockDim.x)
+    draw_pick(e, b, iter);
 }
 
 __global__ void wf_entry_k(const __grid_constant__ WfScene e, WfScene* out) {
@@ -2331,8 +2338,13 @@ cudaError_t wf_pick(const WfScene* tab_dev, const std::vector<WfScene>& tab, con
   const WfScene& last = tab.back();
   const uint32_t n_launch = last.pix_begin + last.n_pix;
   const uint32_t blocks = std::min<uint32_t>((n_launch + kWfThreads - 1) / kWfThreads, 4096u);
-  const auto k = tab_dev ? wf_pick_k<false> : wf_pick_k<true>;
-  k<<<std::max(blocks, 1u), kWfThreads, 0, st>>>(tab_dev, tab[0], (uint32_t)tab.size(), n_launch, iter_dev, iter);
+  wf_pick_k<<<std::max(blocks, 1u), kWfThreads, 0, st>>>(tab_dev, (uint32_t)tab.size(), n_launch, iter_dev, iter);
+  return cudaGetLastError();
+}
+
+cudaError_t wf_pick_one(const WfScene& e, uint32_t iter, cudaStream_t st) {
+  const uint32_t blocks = std::min<uint32_t>((e.n_pix + kWfThreads - 1) / kWfThreads, 4096u);
+  wf_pick_one_k<<<std::max(blocks, 1u), kWfThreads, 0, st>>>(e, iter);
   return cudaGetLastError();
 }
 

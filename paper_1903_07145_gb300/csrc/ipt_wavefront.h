@@ -69,10 +69,12 @@ cudaError_t wf_forward(const Launcher& L, const WfScene* tab_dev, const std::vec
 cudaError_t wf_set_entry(const WfScene& e, WfScene* tab_dev, cudaStream_t st);
 
 // Draws the pixel batch of every table entry that has one, for the iteration
-// *iter_dev (or iter when iter_dev is null).  A table of one scene may stay on
-// the host (tab_dev null).
+// *iter_dev (or iter when iter_dev is null).
 cudaError_t wf_pick(const WfScene* tab_dev, const std::vector<WfScene>& tab, const uint32_t* iter_dev,
                     uint32_t iter, cudaStream_t st);
+
+// The same for one scene (its entries 0..n_pix-1), without a table.
+cudaError_t wf_pick_one(const WfScene& e, uint32_t iter, cudaStream_t st);
 
 cudaError_t wf_adjoint(const Launcher& L, const WfScene* tab_dev, const std::vector<WfScene>& tab,
                        const TraceParams& tp, const uint32_t* iter_dev, const WfBuffers& wb, double* grad_acc,
