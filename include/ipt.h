@@ -19,6 +19,8 @@
  *     from the context's stream, after a call with the same options has
  *     allocated what it needs.  Its graph uses the context's buffers: replay
  *     it in order with the context's other work, while the context lives.
+ *     Buffers that larger calls outgrow stay for it; ipt_views_set and
+ *     ipt_cache_configure replace what it reads and end it.
  *   - Argument errors are reported as IPT_ERR_INVALID_ARG before anything is
  *     launched.  Errors found on the device set a status word that the next
  *     synchronising call returns: a traversal stack overflow as IPT_ERR_CUDA,

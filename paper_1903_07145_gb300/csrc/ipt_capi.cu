@@ -139,22 +139,6 @@ ipt::TraceParams trace_params(const ipt_ctx* ctx, int32_t scene, const ipt_trace
   return tp;
 }
 
-// Device buffers of a pixel batch of `batch` entries (grown, never shrunk).
-ipt_status ensure_pick(ipt_ctx* ctx, DeviceScene* s, uint32_t batch) {
-  if (s->pick_cap >= batch) return IPT_OK;
-  IPT_CK(cudaStreamSynchronize(ctx->stream));
-  ++ctx->alloc_gen;
-  cudaFree(s->pick);
-  cudaFree(s->g_pick);
-  s->pick = nullptr;
-  s->g_pick = nullptr;
-  s->pick_cap = 0;
-  IPT_CK(cudaMalloc(&s->pick, batch * sizeof(uint32_t)));
-  IPT_CK(cudaMalloc(&s->g_pick, 3 * (size_t)batch * sizeof(float)));
-  s->pick_cap = batch;
-  return IPT_OK;
-}
-
 // Whether the caller captures the context's stream (or, for the legacy
 // stream, another one: nothing may be waited for either way).
 bool capturing(const ipt_ctx* ctx) {
@@ -162,6 +146,40 @@ bool capturing(const ipt_ctx* ctx) {
   if (cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess) return cap != cudaStreamCaptureStatusNone;
   cudaGetLastError();
   return true;
+}
+
+// cudaMalloc, also while the caller captures a stream in any mode (an
+// allocation is no stream operation: nothing of it enters the graph).
+static cudaError_t malloc_in_capture(void** p, size_t bytes) {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  const cudaError_t e = cudaMalloc(p, bytes);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return e;
+}
+
+// Whether a graph of the caller's holds the scene's buffers.
+static bool in_a_graph(const DeviceScene* s) { return s->tab_captured || (s->disney && s->disney->tab_captured); }
+
+// Device buffers of a pixel batch of `batch` entries (grown, never shrunk).
+ipt_status ensure_pick(ipt_ctx* ctx, DeviceScene* s, uint32_t batch) {
+  if (s->pick_cap >= batch) return IPT_OK;
+  ++ctx->alloc_gen;
+  if (in_a_graph(s)) {  // kept with the scene
+    s->owned.push_back(s->pick);
+    s->owned.push_back(s->g_pick);
+  } else {
+    IPT_CK(cudaStreamSynchronize(ctx->stream));
+    cudaFree(s->pick);
+    cudaFree(s->g_pick);
+  }
+  s->pick = nullptr;
+  s->g_pick = nullptr;
+  s->pick_cap = 0;
+  IPT_CK(malloc_in_capture(reinterpret_cast<void**>(&s->pick), batch * sizeof(uint32_t)));
+  IPT_CK(malloc_in_capture(reinterpret_cast<void**>(&s->g_pick), 3 * (size_t)batch * sizeof(float)));
+  s->pick_cap = batch;
+  return IPT_OK;
 }
 
 ipt_status ensure_tables(ipt_ctx* ctx, DeviceScene* s, const float* params, const float* sparams) {
@@ -173,16 +191,6 @@ ipt_status ensure_tables(ipt_ctx* ctx, DeviceScene* s, const float* params, cons
   s->tab_is_ctx = is_ctx;
   s->tab_batch = -1;
   return IPT_OK;
-}
-
-// cudaMalloc, also while the caller captures a stream in any mode (an
-// allocation is no stream operation: nothing of it enters the graph).
-static cudaError_t malloc_in_capture(void** p, size_t bytes) {
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  const cudaError_t e = cudaMalloc(p, bytes);
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  return e;
 }
 
 // Gives the wavefront buffers back after the work queued on them.  Those that
@@ -487,21 +495,24 @@ ipt::CacheNet cache_net(const DeviceScene* s, bool unit_inputs) {
 
 // Query buffers for the context's wavefront capacity (reallocated when the
 // capacity grew).
-ipt_status cache_query_buffers(ipt_ctx* ctx, CacheState* c) {
+ipt_status cache_query_buffers(ipt_ctx* ctx, const DeviceScene* s) {
+  CacheState* c = s->cache;
   const uint32_t cap = ctx->cfg.wavefront_slots ? ctx->cfg.wavefront_slots : (1u << 20);
   if (c->buf.q_cap >= cap) return IPT_OK;
-  IPT_CK(cudaStreamSynchronize(ctx->stream));
-  void* ptrs[6] = {c->buf.q.x, c->buf.q.d, c->buf.q.n, c->buf.q.u, c->buf.qc, c->buf.qdp};
-  for (void* q : ptrs) {
-    if (!q) continue;
-    cudaFree(q);
-    c->owned.erase(std::remove(c->owned.begin(), c->owned.end(), q), c->owned.end());
+  if (!in_a_graph(s)) {  // else they stay with the cache
+    IPT_CK(cudaStreamSynchronize(ctx->stream));
+    void* ptrs[6] = {c->buf.q.x, c->buf.q.d, c->buf.q.n, c->buf.q.u, c->buf.qc, c->buf.qdp};
+    for (void* q : ptrs) {
+      if (!q) continue;
+      cudaFree(q);
+      c->owned.erase(std::remove(c->owned.begin(), c->owned.end(), q), c->owned.end());
+    }
   }
   c->buf.q_cap = 0;
   cudaError_t e = cudaSuccess;
   auto A = [&](auto** p, size_t n) {
     void* q = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc(&q, n * sizeof(**p));
+    if (e == cudaSuccess) e = malloc_in_capture(&q, n * sizeof(**p));
     if (e == cudaSuccess) {
       c->owned.push_back(q);
       *p = static_cast<std::remove_reference_t<decltype(*p)>>(q);
@@ -520,7 +531,7 @@ ipt_status cache_query_buffers(ipt_ctx* ctx, CacheState* c) {
 
 // The cache's part of a pass over scene s (query or record mode).
 ipt_status cache_pass(ipt_ctx* ctx, DeviceScene* s, bool record, ipt::CachePass* out) {
-  ipt_status st = cache_query_buffers(ctx, s->cache);
+  ipt_status st = cache_query_buffers(ctx, s);
   if (st != IPT_OK) return st;
   out->net = cache_net(s, false);
   out->buf = s->cache->buf;

@@ -159,7 +159,7 @@ ipt_status ipt_cache_configure(ipt_ctx* ctx, int32_t scene, const ipt_cache_opts
   if (!s->cache && (st = cache_create(ctx, s, opts)) != IPT_OK) return st;
   CacheState* c = s->cache;
   if ((st = cache_record_buffers(ctx, c, opts->record_capacity)) != IPT_OK) return st;
-  if ((st = cache_query_buffers(ctx, c)) != IPT_OK) return st;
+  if ((st = cache_query_buffers(ctx, s)) != IPT_OK) return st;
   c->opts = *opts;
   c->active = opts->enabled != 0;
   c->fell_back = false;

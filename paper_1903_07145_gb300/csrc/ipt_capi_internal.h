@@ -269,7 +269,7 @@ ipt_status run_adjoint(ipt_ctx* ctx, int32_t scene_id, DeviceScene* s, uint32_t 
                        const ipt::CachePass* cache = nullptr, uint32_t* pick = nullptr);
 bool cache_on(const DeviceScene* s);
 ipt::CacheNet cache_net(const DeviceScene* s, bool unit_inputs);
-ipt_status cache_query_buffers(ipt_ctx* ctx, CacheState* c);
+ipt_status cache_query_buffers(ipt_ctx* ctx, const DeviceScene* s);
 ipt_status cache_pass(ipt_ctx* ctx, DeviceScene* s, bool record, ipt::CachePass* out);
 ipt_status cache_train_pass(ipt_ctx* ctx, int32_t scene, DeviceScene* s, const ipt_trace_opts* opts,
                             uint64_t iteration);

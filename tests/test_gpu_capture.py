@@ -10,7 +10,7 @@ import torch
 
 from paper_1903_07145_gb300 import _lib as L
 from paper_1903_07145_gb300 import scenes
-from paper_1903_07145_gb300.tracer import TraceOptions, Tracer
+from paper_1903_07145_gb300.tracer import CacheOptions, TraceOptions, Tracer
 
 pytestmark = pytest.mark.gpu
 MODES = ["unset", "wavefront", "megakernel"]  # unset: the integrator by the size of the pass
@@ -152,6 +152,50 @@ def test_tables_follow_the_parameters_through_replays():
                     assert torch.equal(r(), want[name][0]) and torch.equal(d(), want[name][2])
                     r(params=given), d(sampling_params=spare)
         tr.synchronize()
+        tr.close()
+
+
+@pytest.mark.parametrize("mode", MODES)
+def test_a_graph_keeps_buffers_that_are_outgrown(mode):
+    """Pixel batches (both models) and, on the wavefront, cached passes: the
+    entries' and queries' buffers of a graph outlive their growth."""
+    big = TraceOptions(spp_r=2, spp_d=2, max_depth=3, pixel_batch=5000)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        tr, w = _tracer(mode)
+        calls = ["pixel_batch", "disney_pixel_batch"]
+        want = {k: CALLS[k](tr, w).clone() for k in calls}
+        if mode == "wavefront":
+            tr.configure(mode, wavefront_slots=4096)
+            tr.configure_cache(CacheOptions())
+            calls.append("render")
+            want["render"] = CALLS["render"](tr, w).clone()
+            tr.configure_cache(CacheOptions(enabled=False))
+            plain = CALLS["render"](tr, w)
+            assert not torch.equal(plain, want["render"])
+        stream.synchronize()
+        graphs, got = {}, {}
+        for k in calls:
+            if k == "render":
+                tr.configure_cache(CacheOptions())
+                CALLS[k](tr, w)
+                stream.synchronize()
+            graphs[k] = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graphs[k], stream=stream):
+                got[k] = CALLS[k](tr, w)
+        if mode == "wavefront":  # larger buffers for the queries and the path state
+            tr.configure(mode, wavefront_slots=8192)
+            CALLS["render"](tr, w)
+            tr.configure_cache(CacheOptions(enabled=False))
+        _loss_grad(tr, big, 5), _loss_grad(tr, big, 5, disney=True)
+        stream.synchronize()
+        spare = [torch.full((1 << 16,), float("nan"), device="cuda") for _ in range(64)]  # in freed memory, if any
+        for k in calls:
+            got[k].fill_(float("nan"))
+            graphs[k].replay()
+            assert _same(k, got[k], want[k]), k
+        tr.synchronize()
+        del spare
         tr.close()
 
 
